@@ -95,6 +95,7 @@ struct AssignParams {
     uint8_t *moving;
     DevCounters *ctr;
     double eps, eta;
+    float eps_f, eta_q;        // eps and eta / quantum for the quick bound test
     // instances: objects [inst_obj[m], inst_obj[m+1]) and clusters
     // [inst_k[m], inst_k[m+1]) form instance m; moving ids of instance m are
     // mov_list[mov_beg[m] .. mov_beg[m+1]). The scan arrays hold local ids.
@@ -205,6 +206,38 @@ __device__ __forceinline__ double error_bound(double x, int64_t n, int nd, doubl
     const double c = eps + (1.0 + eps) * g;
     const double a = 2.0 * (double)n * FIX_QUANTUM + (1.0 + g) * eta * S;
     return (c * x + a) / (1.0 - c) * (1.0 + 1e-12);
+}
+
+// Whether a gap of `gap` quanta between the best score and the second is
+// certainly larger than 2 E(best): the bound in FP32 with 1e-4 (and one
+// quantum) to spare over every rounding of this evaluation. Most objects pass
+// it, and the FP64 bound (two divisions on a pipe that retires about one
+// operation per clock and SM, with the CTA waiting) is formed for the rest
+// only; the decision is the FP64 bound's in every case. eta_q = eta * S in quanta.
+__device__ __forceinline__ bool clear_of_bound(uint32_t best, uint32_t gap, int64_t n, int nd, float eps,
+                                               float eta_q) {
+    const float m = nd > 1 ? (float)nd : 1.0f;
+    if (!(m < 1.0e6f)) return false;
+    const float mu = m * 5.9604644775390625e-08f;
+    const float g = mu / (1.0f - mu);
+    const float c = eps + (1.0f + eps) * g;
+    const float E = (c * __uint2float_ru(best) + 2.0f * (float)n + (1.0f + g) * eta_q) / (1.0f - c);
+    return __uint2float_rd(gap) > 2.0f * (E * 1.0001f + 1.0f);
+}
+
+// Largest and second largest (equal to the largest when two lanes hold it) of
+// the warp's values; b >= s in every lane.
+__device__ __forceinline__ void warp_top2(uint32_t &b, uint32_t &s) {
+    const uint32_t best = __reduce_max_sync(0xffffffffu, b);
+    const unsigned at = __ballot_sync(0xffffffffu, b == best);
+    const uint32_t rest = __reduce_max_sync(0xffffffffu, b == best ? s : b);
+    b = best;
+    s = __popc(at) > 1 ? best : rest;
+}
+
+__device__ __forceinline__ void top2_add(uint32_t &b, uint32_t &s, uint32_t v) {
+    s = max(s, min(b, v));
+    b = max(b, v);
 }
 
 template <int T>
@@ -433,24 +466,32 @@ __device__ __forceinline__ void rho_zero(uint32_t *p) {
     else *p = 0u;
 }
 
-// Dense head rows: 8 consecutive entries of a row (one 16-byte load for
-// BF16/FP16, two for FP32), loaded raw and decoded to FP32 afterwards, so
-// that the loads of several rows can be in flight together. FP16 rows hold
-// u * 2^14 (the scale is folded into the object value by the caller).
+// Dense head rows: 8 entries of a row per thread, loaded raw and decoded to
+// FP32 afterwards, so that the loads of several rows can be in flight
+// together. BF16/FP16: one 16-byte load of 8 consecutive entries. FP32: two
+// 16-byte loads of 4 consecutive entries each, `half` positions apart, so
+// that the lanes of a warp read contiguous memory in each load (8 consecutive
+// FP32 entries per lane would leave a 16-byte gap between neighbouring lanes:
+// every load touched twice the sectors it used, and the L1 data pipe ran at
+// 93 % on the 300K x 100K, k = 1000 corpus). FP16 rows hold u * 2^14 (the
+// scale is folded into the object value by the caller).
 template <int PREC>
 struct Raw8 {
     uint4 w[PREC == SIVF_FP32 ? 2 : 1];
 };
 
+// e0: address of the first entry of row 0 that the thread owns; row8 = row
+// offset in 8-entry units; second = the FP32 form's second half lies in the row
 template <int PREC>
-__device__ __forceinline__ Raw8<PREC> load_raw8(const void *dense, int64_t e) {
+__device__ __forceinline__ Raw8<PREC> load_raw8(const char *e0, int row8, int half, bool second) {
     Raw8<PREC> r;
     if constexpr (PREC == SIVF_FP32) {
-        const uint4 *p = reinterpret_cast<const uint4 *>(static_cast<const float *>(dense) + e);
-        r.w[0] = __ldg(p);
-        r.w[1] = __ldg(p + 1);
+        const char *p = e0 + (uint64_t)(uint32_t)row8 * 32u;
+        r.w[0] = __ldg(reinterpret_cast<const uint4 *>(p));
+        r.w[1] = make_uint4(0u, 0u, 0u, 0u);
+        if (second) r.w[1] = __ldg(reinterpret_cast<const uint4 *>(p + 4 * half));
     } else {
-        r.w[0] = __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(dense) + e));
+        r.w[0] = __ldg(reinterpret_cast<const uint4 *>(e0 + (uint64_t)(uint32_t)row8 * 16u));
     }
     return r;
 }
@@ -481,41 +522,82 @@ __device__ __forceinline__ void fma_raw8(const Raw8<PREC> &r, float vs, float ac
     }
 }
 
-// Dense phase of one staged chunk: thread tid owns the 8 scan positions
-// base + 8 tid of each pass (8 T positions per pass) and accumulates, in FP32
+// Four consecutive scores with one 16-byte access (p a multiple of 4).
+template <bool GRHO>
+__device__ __forceinline__ uint4 rho_ld4(const uint32_t *p) {
+    if constexpr (GRHO) return __ldcg(reinterpret_cast<const uint4 *>(p));
+    else return *reinterpret_cast<const uint4 *>(p);
+}
+template <bool GRHO>
+__device__ __forceinline__ void rho_st4(uint32_t *p, uint4 v) {
+    if constexpr (GRHO) __stcg(reinterpret_cast<uint4 *>(p), v);
+    else *reinterpret_cast<uint4 *>(p) = v;
+}
+template <bool GRHO>
+__device__ __forceinline__ void rho_put4(uint32_t *p, const float *acc, bool init) {
+    uint4 q = make_uint4(__float2uint_ru(acc[0]), __float2uint_ru(acc[1]), __float2uint_ru(acc[2]),
+                         __float2uint_ru(acc[3]));
+    if (!init) {
+        const uint4 o = rho_ld4<GRHO>(p);
+        q = make_uint4(q.x + o.x, q.y + o.y, q.z + o.z, q.w + o.w);
+    }
+    rho_st4<GRHO>(p, q);
+}
+
+// Dense phase of one staged chunk: each pass covers 8 T score positions, 8 per
+// thread (BF16/FP16: base + 8 tid and the seven after; FP32: base + 4 tid and
+// base + 4 T + 4 tid with the three after each). A thread accumulates, in FP32
 // registers, v * u over the chunk's dense terms in staging order; each
-// position's partial sum is then added to the score as one fixed-point value.
-// The loads of DENSE_U consecutive terms are issued together (about 128 bytes
-// in flight per thread), their multiply-adds follow in term order. Positions
-// [0, npos) are covered: the moving clusters for a front scan, all of the
-// instance's clusters otherwise. A position's sum depends only on the chunk's
-// terms, never on which thread or pass covers it, so front and full scans give
-// the same scores.
+// position's partial sum is then put into the score as one fixed-point value:
+// stored in the object's first chunk (init, so that the scores need no zeroing
+// pass; a chunk without dense terms then stores zeros), added in later ones.
+// No other thread touches the positions during this phase (the caller puts a
+// barrier before the posting atomics), so these are 16-byte accesses instead
+// of atomics, which hit every bank eight times per warp. The loads of U
+// consecutive terms are issued together (about 128 bytes in flight per
+// thread), their multiply-adds follow in term order. Positions [0, npos) are
+// covered: the moving clusters for a front scan, all of the instance's
+// clusters otherwise. Up to 7 positions beyond npos (inside the vector) may
+// receive values; nothing reads them. A position's sum depends only on the
+// chunk's terms, never on which thread or pass covers it, so front and full
+// scans give the same scores.
 template <int T, int PREC, bool GRHO>
 __device__ __forceinline__ void dense_chunk(const AssignParams &P, uint32_t *rho, const int2 *s_dense, int nd,
-                                            int npos) {
+                                            int npos, bool init) {
     constexpr int U = PREC == SIVF_FP32 ? 4 : 8;
+    constexpr int W = PREC == SIVF_FP32 ? 4 : 8;          // consecutive positions of a thread
+    constexpr int HALF = PREC == SIVF_FP32 ? 4 * T : 4;   // from its first four positions to its last four
+    constexpr int ESIZE = PREC == SIVF_FP32 ? 4 : 2;
+    const int4 *pair = reinterpret_cast<const int4 *>(s_dense);
     for (int base = 0; base < npos; base += 8 * T) {
-        const int p = base + 8 * (int)threadIdx.x;
+        const int p = base + W * (int)threadIdx.x;
         if (p >= npos) continue;  // rows are padded to multiples of 8: a load at p < npos stays in the row
+        const bool second = p + HALF < npos;
+        const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * ESIZE;
         float acc[8];
 #pragma unroll
         for (int m = 0; m < 8; ++m) acc[m] = 0.f;
         int d = 0;
         for (; d + U <= nd; d += U) {
             Raw8<PREC> r[U];
+            float vs[U];
 #pragma unroll
-            for (int q = 0; q < U; ++q) r[q] = load_raw8<PREC>(P.dense, (int64_t)s_dense[d + q].x * 8 + p);
+            for (int q = 0; q < U; q += 2) {
+                const int4 e = pair[(d + q) >> 1];
+                r[q] = load_raw8<PREC>(e0, e.x, HALF, second);
+                r[q + 1] = load_raw8<PREC>(e0, e.z, HALF, second);
+                vs[q] = __int_as_float(e.y);
+                vs[q + 1] = __int_as_float(e.w);
+            }
 #pragma unroll
-            for (int q = 0; q < U; ++q) fma_raw8<PREC>(r[q], __int_as_float(s_dense[d + q].y), acc);
+            for (int q = 0; q < U; ++q) fma_raw8<PREC>(r[q], vs[q], acc);
         }
         for (; d < nd; ++d) {
-            const Raw8<PREC> r = load_raw8<PREC>(P.dense, (int64_t)s_dense[d].x * 8 + p);
-            fma_raw8<PREC>(r, __int_as_float(s_dense[d].y), acc);
+            const int2 e = s_dense[d];
+            fma_raw8<PREC>(load_raw8<PREC>(e0, e.x, HALF, second), __int_as_float(e.y), acc);
         }
-#pragma unroll
-        for (int m = 0; m < 8; ++m)
-            if (p + m < npos && acc[m] > 0.f) atomicAdd(rho + p + m, __float2uint_ru(acc[m]));
+        rho_put4<GRHO>(rho + p, acc, init);
+        if (second) rho_put4<GRHO>(rho + p + HALF, acc + 4, init);
     }
 }
 
@@ -550,15 +632,13 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
     __shared__ int4 warp_i4[32];
     __shared__ int4 s_total4;
     __shared__ long long s_obj;
-    __shared__ Top2 warp_t[NW];
+    __shared__ uint32_t warp_b[NW], warp_s[NW];
     __shared__ double warp_d[NW];
     __shared__ int warp_j[NW];
-    __shared__ int s_winner;
     __shared__ int s_flag;
     __shared__ uint32_t s_thr;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int j = tid; j < kpad; j += T) rho_zero<GRHO>(rho + j);
     if constexpr (CB) {
         const int nbits = ((P.k + 31) >> 5) << 5;
         for (int j = tid; j < nbits; j += T) {  // a warp covers 32 consecutive clusters
@@ -654,8 +734,8 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         constexpr int RMIN = 16;
         for (int pass = 0;; ++pass) {
         const bool front = (filt || relax) && pass == 0;  // scan the fronts only
-        const int npos = front ? n_mov_inst : km;         // score positions this pass covers
-        for (int64_t cb = rb; cb < re; cb += T) {
+        const int npos = front && !CB ? n_mov_inst : km;  // score positions this pass covers
+        for (int64_t cb = rb; cb == rb || cb < re; cb += T) {  // an empty row still sets its scores
             const int cn = (int)min((int64_t)T, re - cb);
             int4 cnt = make_int4(0, 0, 0, 0);
             int2 dent = make_int2(-1, 0);
@@ -696,10 +776,11 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
             const int4 tot = s_total4;
 
             // dense rows
-            if (tot.z > 0) {
+            if (tot.z > 0 || cb == rb) {
                 nd_obj += tot.z;
-                dense_chunk<T, PREC, GRHO>(P, rho, s_dense, tot.z, npos);
+                dense_chunk<T, PREC, GRHO>(P, rho, s_dense, tot.z, npos, cb == rb);
                 if (tid == 0) s_cnt[5] += (unsigned long long)tot.z * (unsigned long long)npos;
+                if (tot.x > 0 || tot.y > 0) __syncthreads();  // plain accesses above, atomics below
             }
 
             // items
@@ -834,9 +915,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         }
         __syncthreads();
         if (s_flag) break;
-        for (int m = tid; m < n_mov_inst; m += T) rho_zero<GRHO>(rho + mov_at(m));
-        __syncthreads();
-        relax = false;
+        relax = false;  // the full scan sets every score again (the next barrier follows the staging)
         wasted = true;
         nd_obj = 0;  // the full scan counts its dense terms again
         }
@@ -844,61 +923,105 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         const int n_mov = sub ? n_mov_inst : 0;
 
         // ---- argmax over the candidates (Algorithm 4, lines 14-16) ----
-        // largest score, lowest cluster id on ties (ids are looked up only
-        // when a score ties or beats the running best)
-        PosTop2 pt;
-        pt.bv = 0u;
-        pt.bp = -1;
-        pt.sv = -1;
-        if (!sub) {
-            for (int p = tid; p < km; p += T) pos_push(pt, rho_ld<GRHO>(rho + p), p, id_at);
+        // The two largest scores, without ids: an object whose gap is clear of
+        // the error bound has one winner, found by looking for its score again.
+        uint32_t bv = 0u, sv = 0u;  // scores are >= 0: a start of 0 never wins over a candidate
+        const int ncand = sub ? n_mov : km;
+        if constexpr (CB) {
+            for (int m = tid; m < ncand; m += T) top2_add(bv, sv, rho_ld<GRHO>(rho + (sub ? mov_at(m) : m)));
         } else {
-            for (int m = tid; m < n_mov; m += T) {
-                const int p = mov_at(m);
-                pos_push(pt, rho_ld<GRHO>(rho + p), p, id_at);
+            for (int p = 4 * tid; p < ncand; p += 4 * T) {
+                const uint4 q = rho_ld4<GRHO>(rho + p);
+                top2_add(bv, sv, q.x);
+                if (p + 1 < ncand) top2_add(bv, sv, q.y);
+                if (p + 2 < ncand) top2_add(bv, sv, q.z);
+                if (p + 3 < ncand) top2_add(bv, sv, q.w);
             }
         }
-        Top2 t = pos_top2(pt, id_at);
-        if (sub && tid == 0) top2_push(t, own_q, a_loc);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t = top2_merge(t, top2_shfl(t, o));
-        if (lane == 0) warp_t[warp] = t;
+        const uint32_t mine = bv;  // this thread's largest
+        warp_top2(bv, sv);
+        if (lane == 0) {
+            warp_b[warp] = bv;
+            warp_s[warp] = sv;
+        }
         __syncthreads();
-        if (tid == 0) {
-            Top2 b = warp_t[0];
-            for (int w = 1; w < NW; ++w) b = top2_merge(b, warp_t[w]);
-            int flag = 0;
-            uint32_t thr = 0;
-            if (b.bv > 0u && b.sv >= 0) {
-                const double best = (double)b.bv * FIX_QUANTUM;
-                // a filtered object's carried own score may come from a scan with
-                // other dense terms: count every term as dense for it
-                const double E = error_bound(best, re - rb, filt ? (int)(re - rb) : nd_obj, (double)P.sumv[i],
-                                             P.eps, P.eta);
-                const double gap = (double)((long long)b.bv - b.sv) * FIX_QUANTUM;
-                if (gap <= 2.0 * E) {
-                    flag = 1;
-                    const double span = ceil(2.0 * E / FIX_QUANTUM);
-                    thr = span >= (double)b.bv ? 0u : b.bv - (uint32_t)span;
+        // every warp reduces the warps' results: all threads hold the block's
+        bv = lane < NW ? warp_b[lane] : 0u;
+        sv = lane < NW ? warp_s[lane] : 0u;
+        warp_top2(bv, sv);
+        const uint32_t top = bv;      // largest scanned score
+        if (filt) top2_add(bv, sv, own_q);
+        const int64_t n_terms = re - rb;
+        // a filtered object's carried own score may come from a scan with
+        // other dense terms: count every term as dense for it
+        const int nd_bound = filt ? (int)n_terms : nd_obj;
+        bool flag = bv > 0u && ncand + (filt ? 1 : 0) > 1 &&
+                    !clear_of_bound(bv, bv - sv, n_terms, nd_bound, P.eps_f,
+                                    P.eta_q != 0.f ? P.eta_q * P.sumv[i] : 0.f);
+        if (flag) {  // block-uniform: the exact form of the bound
+            if (tid == 0) {
+                const double E = error_bound((double)bv * FIX_QUANTUM, n_terms, nd_bound, (double)P.sumv[i], P.eps,
+                                             P.eta);
+                const bool f = (double)(bv - sv) * FIX_QUANTUM <= 2.0 * E;
+                const double span = ceil(2.0 * E / FIX_QUANTUM);
+                s_flag = f;
+                s_thr = span >= (double)bv ? 0u : bv - (uint32_t)span;
+            }
+            __syncthreads();
+            flag = s_flag;
+        }
+        // the thread that knows the label writes it and marks the moving
+        // clusters (Algorithm 4, lines 17-19); al = local id
+        auto finish = [&](int al, uint32_t q) {
+            const int a = k_off + al;
+            P.labels[i] = a;
+            P.own[i] = q;
+            if (a != a_prev) {
+                s_cnt[2] += 1;
+                P.moving[a] = 1;
+                if (a_prev >= 0) P.moving[a_prev] = 1;
+                if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
+            }
+            s_cnt[0] += sub ? 1ull : 0ull;
+            s_cnt[1] += (unsigned long long)ncand + (wasted ? (unsigned long long)n_mov_inst : 0ull);
+        };
+        if (!flag) {
+            if (bv == 0u || (filt && own_q == bv)) {
+                if (tid == 0) {
+                    // all scores zero: the lowest id among the candidates
+                    // (position 0 holds the lowest moving id, and id 0 unfiltered);
+                    // else the own cluster, which no scanned score reaches
+                    int al = filt ? a_loc : INT32_MAX;
+                    if (bv == 0u && ncand > 0) al = min(al, sub ? movs[0] - k_off : 0);
+                    finish(al, bv);
+                }
+            } else if (mine == top) {  // one thread: a second one would make the gap zero
+                if constexpr (CB) {
+                    for (int m = tid; m < ncand; m += T)
+                        if (rho_ld<GRHO>(rho + (sub ? mov_at(m) : m)) == top) finish(sub ? mov_at(m) : m, top);
+                } else {
+                    for (int p = 4 * tid; p < ncand; p += 4 * T) {
+                        const uint4 q = rho_ld4<GRHO>(rho + p);
+                        const int e = q.x == top ? 0 : (q.y == top ? 1 : (q.z == top ? 2 : (q.w == top ? 3 : 4)));
+                        if (e < 4 && p + e < ncand) {
+                            finish(id_at(p + e), top);
+                            break;
+                        }
+                    }
                 }
             }
-            s_winner = b.bi;
-            s_flag = flag;
-            s_thr = thr;
         }
-        __syncthreads();
 
         // ---- exact re-score of the candidates inside the bound ----
-        if (s_flag) {
+        if (flag) {
             const uint32_t thr = s_thr;
             double wbest = -1.0;
             int wj = INT32_MAX;
-            int ncand = 0;
-            const int total = sub ? n_mov : km;
-            for (int base = warp * 32; base < total; base += T) {
+            int nresc = 0;
+            for (int base = warp * 32; base < ncand; base += T) {
                 const int m = base + lane;
                 int j = -1;
-                if (m < total) {
+                if (m < ncand) {
                     const int p = sub ? mov_at(m) : m;
                     if (rho_ld<GRHO>(rho + p) >= thr) j = id_at(p);
                 }
@@ -908,7 +1031,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
                     bal &= bal - 1;
                     const int jc = __shfl_sync(0xffffffffu, j, src);
                     const double x = exact_score(P, rb, re, k_off + jc, lane);
-                    ++ncand;
+                    ++nresc;
                     if (x > wbest || (x == wbest && jc < wj)) {
                         wbest = x;
                         wj = jc;
@@ -917,7 +1040,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
             }
             if (filt && warp == 0 && own_q >= thr) {
                 const double x = exact_score(P, rb, re, a_prev, lane);
-                ++ncand;
+                ++nresc;
                 if (x > wbest || (x == wbest && a_loc < wj)) {
                     wbest = x;
                     wj = a_loc;
@@ -926,7 +1049,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
             if (lane == 0) {
                 warp_d[warp] = wbest;
                 warp_j[warp] = wj;
-                if (ncand) atomicAdd(&s_cnt[4], (unsigned long long)ncand);
+                if (nresc) atomicAdd(&s_cnt[4], (unsigned long long)nresc);
             }
             __syncthreads();
             if (tid == 0) {
@@ -938,33 +1061,9 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
                         bj = warp_j[w];
                     }
                 }
-                if (bj != INT32_MAX) s_winner = bj;
                 s_cnt[3] += 1;
+                finish(bj, (filt && bj == a_loc) ? own_q : rho_ld<GRHO>(rho + (CB ? bj : P.clu_pos[k_off + bj])));
             }
-            __syncthreads();
-        }
-
-        // ---- write the assignment, mark moving clusters (lines 17-19) ----
-        if (tid == 0) {
-            const int al = s_winner;  // local id
-            const int a = k_off + al;
-            P.labels[i] = a;
-            P.own[i] = (filt && al == a_loc) ? own_q : rho_ld<GRHO>(rho + (CB ? al : P.clu_pos[a]));
-            if (a != a_prev) {
-                s_cnt[2] += 1;
-                P.moving[a] = 1;
-                if (a_prev >= 0) P.moving[a_prev] = 1;
-                if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
-            }
-            s_cnt[0] += sub ? 1ull : 0ull;
-            s_cnt[1] += (sub ? (unsigned long long)n_mov : (unsigned long long)km) +
-                        (wasted ? (unsigned long long)n_mov_inst : 0ull);
-        }
-        __syncthreads();
-        if (!sub) {
-            for (int p = tid; p < km; p += T) rho_zero<GRHO>(rho + p);
-        } else {
-            for (int m = tid; m < n_mov; m += T) rho_zero<GRHO>(rho + mov_at(m));
         }
         __syncthreads();
     }
@@ -1009,6 +1108,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
 // 648 ms per assignment) and lost above (1,802: 800 vs 726 ms).
 constexpr int LIGHT_WARPS = 8;
 constexpr int LIGHT_MAX = 1472;  // the largest moving count of a light object
+static_assert(LIGHT_MAX % 8 == 0, "vector accesses of a slice");
 static_assert(LIGHT_WARPS * (LIGHT_MAX * 4 + 32 * 8) <= 48 * 1024, "static shared memory of the light kernel");
 
 __device__ __forceinline__ int instance_of(const AssignParams &P, int64_t i) {
@@ -1091,14 +1191,17 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
             if (lane == 0) P.labels[i] = a_prev;
             continue;
         }
-        for (int p = lane; p < n_mov; p += 32) rho[p] = 0u;
+        for (int p = lane; p < n_mov; p += 32) rho[p] = 0u;  // positions beyond n_mov are never read as scores
         __syncwarp();
         int nd_obj = 0;
         for (int64_t cb = rb; cb < re; cb += P.chunk) {
             const int64_t ce = min(re, cb + (int64_t)P.chunk);
             // dense rows: the front (positions below n_mov) of each dense term of the chunk
             for (int base = 0; base < n_mov; base += 256) {
-                const int p = base + 8 * lane;
+                const int p = PREC == SIVF_FP32 ? base + 4 * lane : base + 8 * lane;
+                constexpr int HALF = PREC == SIVF_FP32 ? 128 : 4;
+                const bool second = p + HALF < n_mov;
+                const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * (PREC == SIVF_FP32 ? 4 : 2);
                 float acc[8];
 #pragma unroll
                 for (int m = 0; m < 8; ++m) acc[m] = 0.f;
@@ -1126,16 +1229,13 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
                     if (p < n_mov)
                         for (int d = 0; d < cnt; ++d) {  // staging (term) order
                             const int2 x = dn[d];
-                            fma_raw8<PREC>(load_raw8<PREC>(P.dense, (int64_t)x.x * 8 + p), __int_as_float(x.y), acc);
+                            fma_raw8<PREC>(load_raw8<PREC>(e0, x.x, HALF, second), __int_as_float(x.y), acc);
                         }
                     nd_chunk += cnt;
                     __syncwarp();
                 }
-                if (p < n_mov) {
-#pragma unroll
-                    for (int m = 0; m < 8; ++m)
-                        if (p + m < n_mov && acc[m] > 0.f) rho[p + m] += __float2uint_ru(acc[m]);
-                }
+                if (p < n_mov) rho_put4<false>(rho + p, acc, false);  // LIGHT_MAX is a multiple of 8: stays in the slice
+                if (second) rho_put4<false>(rho + p + HALF, acc + 4, false);
                 if (base == 0) {
                     nd_obj += nd_chunk;
                     if (lane == 0) c_dent += (unsigned long long)nd_chunk * (unsigned long long)n_mov;
@@ -1412,6 +1512,8 @@ cudaError_t launch_assign(sivf_ctx *c) {
         P.eps = 0.0;
         P.eta = 0.0;
     }
+    P.eps_f = (float)P.eps;                    // powers of two: exact
+    P.eta_q = (float)(P.eta / FIX_QUANTUM);
     P.heavy_ids = c->heavy_ids;
     P.light_ids = c->light_ids;
     P.chunk = c->assign_threads;

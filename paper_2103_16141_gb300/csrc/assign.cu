@@ -1412,7 +1412,16 @@ cudaError_t launch_t(sivf_ctx *c, const AssignParams &P, int ctas_per_sm) {
     // the attribute and occupancy queries are host calls that a stream capture
     // refuses: they run on the first (host-launched) step and are cached
     if (c->assign_grid <= 0) {
-        SIVF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // the limit belongs to the kernel, not to this context: it is raised to
+        // the most that any context may ask for, as one sized for this
+        // context's k would make another context's launches fail
+        cudaFuncAttributes fa;
+        int optin = 0;
+        SIVF_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
+        SIVF_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+        if (smem + fa.sharedSizeBytes > (size_t)optin) return cudaErrorInvalidConfiguration;
+        SIVF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           optin - (int)fa.sharedSizeBytes));
         int occ = 0;
         SIVF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, T, smem));
         if (occ < 1) return cudaErrorInvalidConfiguration;

@@ -53,3 +53,25 @@ def test_cluster_counts_around_the_tiles(k, threads, precision, buf):
 def test_other_modes_with_empty_rows(icp, precision):
     c = _corpus_with_empty_rows(1_300, 2_500, 31)
     lockstep(c, 130, _seeds(c, 130, 5), 8, precision=precision, icp=icp, dense_min_fraction=0.05)
+
+
+def test_contexts_of_different_k_take_turns():
+    """Two live contexts whose score vectors differ in size, stepped in turn."""
+    from tests.gpu_harness import gpu_instance
+    c = _corpus_with_empty_rows(1_300, 2_500, 77)
+    runs = {}
+    for turns in (False, True):
+        a, b = (gpu_instance(c, k, _seeds(c, k, 5), threads=64) for k in (900, 33))
+        try:
+            for _ in range(3):
+                a.assign(), a.update()
+                if turns:
+                    b.assign(), b.update()
+            if not turns:
+                for _ in range(3):
+                    b.assign(), b.update()
+            runs[turns] = (a.labels(), b.labels())
+        finally:
+            a.close()
+            b.close()
+    assert all(np.array_equal(x, y) for x, y in zip(runs[False], runs[True]))

@@ -49,11 +49,11 @@ cudaError_t dmalloc(sivf_ctx *c, T **p, size_t n) {
 void free_all(sivf_ctx *c) {
     void *ptrs[] = {c->labels, c->labels_prev, c->own, c->sumv, c->lam, c->lam_prev, c->moving, c->mov_list,
                     c->n_mov_dev, c->snorm, c->snorm_new, c->coff[0], c->coff[1], c->cterm[0], c->cterm[1],
-                    c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->if_cid, c->if_val, c->sc_off, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
+                    c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->if_cid, c->if_val, c->tdesc, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
                     c->ctr, c->obj_dev, c->ws.base, c->inst_obj, c->inst_k, c->mov_beg, c->clu_koff,
                     c->inst_changed, c->own_row_ptr, c->own_idx, c->own_val, c->clu_doff,
                     c->loop_dev, c->done_dev, c->objf_dev, c->grho, c->acc, c->acc_off, c->acc_lab,
-                    c->clu_pos, c->pos_clu, c->dense_row, c->dense_val, c->inst_d, c->dense_thr,
+                    c->clu_pos, c->pos_clu, c->dense_val, c->inst_d, c->dense_thr,
                     c->heavy_ids, c->light_ids};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -231,7 +231,7 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     c->cap_s = capc + 3 * (int64_t)D + IF_PAD;
     const size_t caps = (size_t)c->cap_s;
     const bool ids16 = c->kmax <= 65536;
-    INIT_CUDA(dmalloc(c, &c->sc_off, (size_t)D + 1), "alloc");
+    INIT_CUDA(dmalloc(c, &c->tdesc, D), "alloc");
     if (c->cfg.prec == SIVF_FP32) {
         if (ids16) INIT_CUDA(dmalloc(c, &c->sc_id16, caps), "alloc");
         else INIT_CUDA(dmalloc(c, &c->sc_id32, caps), "alloc");
@@ -245,7 +245,6 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     // scan order and dense head rows
     INIT_CUDA(dmalloc(c, &c->clu_pos, k), "alloc");
     INIT_CUDA(dmalloc(c, &c->pos_clu, k), "alloc");
-    INIT_CUDA(dmalloc(c, &c->dense_row, D), "alloc");
     INIT_CUDA(dmalloc(c, &c->inst_d, (size_t)ni + 1), "alloc");
     INIT_CUDA(dmalloc(c, &c->dense_thr, 1), "alloc");
     {
@@ -328,7 +327,7 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
         size_t phase1 = 4 * (size_t)N * 4 + 2 * n8 + 14 * k8 + (c->dense ? 0 : 64 * ((size_t)nnz + 1)) + 32 * 4096;
         // u5: sort arrays (16 B x entries), per-term counts, lengths, dense widths
         // and offsets (40 B x terms), the dense-length histogram
-        size_t phase2 = 16 * ((size_t)capc + 1) + 48 * ((size_t)D + 1) + 16 * 4096;
+        size_t phase2 = 16 * ((size_t)capc + 1) + 40 * ((size_t)D + 1) + 16 * 4096;
         size_t ws = phase1 > phase2 ? phase1 : phase2;
         size_t maxn = (size_t)(capc > N ? capc : N);
         ws += (maxn / 4096 + 2) * 1024 * 4 + (maxn / 2048 + 2) * 16 + 64 * 256 + (1 << 20);

@@ -65,10 +65,10 @@ struct AssignParams {
     const int32_t *idx;
     const float *val;
     const float *sumv;
-    const int64_t *if_off;
-    const int32_t *if_mf0;
-    // scan copy of the inverted file (tiled layout, local ids)
-    const int64_t *sc_off;
+    // per term: {start in the scan copy, front length, list length, first
+    // entry / 8 of its dense row or -1}
+    const int4 *tdesc;
+    // scan copy of the inverted file (ids are scan positions)
     const uint16_t *sc_id16;
     const int32_t *sc_id32;
     const float *sc_val;
@@ -77,7 +77,6 @@ struct AssignParams {
     // scan order and dense head rows
     const int32_t *clu_pos;    // cluster (global id) -> scan position in its instance
     const int32_t *pos_clu;    // instance cluster offset + scan position -> local id
-    const int32_t *dense_row;  // [D]: first entry / 8 of the term's dense row, -1 = sparse
     const void *dense;         // dense rows: u16 (BF16, FP16 x 2^14) or f32
     const int32_t *heavy_ids;  // objects of the CTA-per-object kernel (ctr->n_heavy of them)
     const int32_t *light_ids;  // objects of the warp-per-object kernel (ctr->n_light of them)
@@ -267,67 +266,42 @@ __device__ __forceinline__ int block_inclusive_scan_int(int x, int *warp_s, int 
     return warp_s[warp] + inc;
 }
 
-// Inclusive scan of an int4 over the block (all components at once).
+// Inclusive scan of an int2 over the block (both components at once) and its
+// total. One barrier: every warp scans the warps' sums for itself. warp_s must
+// not be written again before the block's next barrier.
 template <int T>
-__device__ __forceinline__ int4 block_inclusive_scan_int4(int4 v, int4 *warp_s, int4 *total) {
+__device__ __forceinline__ int2 block_inclusive_scan_int2(int2 v, int2 *warp_s, int2 &total) {
+    constexpr int NW = T / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int4 inc = v;
+    int2 inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int a = __shfl_up_sync(0xffffffffu, inc.x, o);
         const int b = __shfl_up_sync(0xffffffffu, inc.y, o);
-        const int c = __shfl_up_sync(0xffffffffu, inc.z, o);
         if (lane >= o) {
             inc.x += a;
             inc.y += b;
-            inc.z += c;
         }
     }
     if (lane == 31) warp_s[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        constexpr int NW = T / 32;
-        const int4 w = lane < NW ? warp_s[lane] : make_int4(0, 0, 0, 0);
-        int4 winc = w;
+    int2 w = lane < NW ? warp_s[lane] : make_int2(0, 0);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int a = __shfl_up_sync(0xffffffffu, winc.x, o);
-            const int b = __shfl_up_sync(0xffffffffu, winc.y, o);
-            const int c = __shfl_up_sync(0xffffffffu, winc.z, o);
-            if (lane >= o) {
-                winc.x += a;
-                winc.y += b;
-                winc.z += c;
-            }
+    for (int o = 1; o < NW; o <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, w.x, o);
+        const int b = __shfl_up_sync(0xffffffffu, w.y, o);
+        if (lane >= o) {
+            w.x += a;
+            w.y += b;
         }
-        if (lane < NW) warp_s[lane] = make_int4(winc.x - w.x, winc.y - w.y, winc.z - w.z, 0);
-        if (lane == NW - 1) *total = winc;
     }
-    __syncthreads();
-    const int4 base = warp_s[warp];
-    return make_int4(base.x + inc.x, base.y + inc.y, base.z + inc.z, 0);
-}
-
-// First index h in [0, T) with a[h] > x, for an ascending array whose last
-// entry exceeds x.
-template <int T>
-__device__ __forceinline__ int first_greater(const int *a, int x) {
-    int lo = 0, hi = T - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] > x) hi = mid; else lo = mid + 1;
+    total = make_int2(__shfl_sync(0xffffffffu, w.x, NW - 1), __shfl_sync(0xffffffffu, w.y, NW - 1));
+    if (warp > 0) {
+        inc.x += __shfl_sync(0xffffffffu, w.x, warp - 1);
+        inc.y += __shfl_sync(0xffffffffu, w.y, warp - 1);
     }
-    return lo;
+    return inc;
 }
-
-// Position of entry o of a list in the tiled scan layout (fb = end of the
-// list's full 128-entry blocks): transposed inside full blocks, canonical in
-// the tail.
-__device__ __forceinline__ int tiled_offset(int o, int fb) {
-    return o < fb ? ((o & ~(SC_BLK - 1)) | ((o & 31) << 2) | ((o >> 5) & 3)) : o;
-}
-
-constexpr int CH = 2 * SC_BLK;  // postings per fast item: two blocks of the tiled layout
 
 // L2 eviction priority (createpolicy + ld.global.nc.L2::cache_hint): when the
 // sparse posting lists do not fit in L2 they are streamed (evict_first), so
@@ -366,61 +340,59 @@ __device__ __forceinline__ float decode_u(unsigned b) {
     else return __half2float(__ushort_as_half((unsigned short)b)) * FP16_INV_SCALE;
 }
 
-// Four postings of one lane: entries 32m + lane (m = 0..3) of a block.
-struct Post4 {
-    int id[4];
-    float u[4];
+// Four consecutive postings of a list, as loaded: one 16-byte load (packed
+// words), or one load per array. pos is a multiple of 4 entries, so the loads
+// are aligned; a list's room is a multiple of 4 entries, so they stay in it.
+template <int PREC, bool CID16>
+struct Quad {
+    uint4 a;     // packed words, or ids
+    uint4 v[1];  // FP32 or 16-bit values of the separate arrays
 };
 
-// One vector load per array of a full block in the tiled layout (block
-// position 4 * lane + m holds entry 32m + lane). pos = list start + block
-// offset + 4 * lane: a multiple of 4 entries, so the loads are aligned.
 template <int PREC, bool CID16>
-__device__ __forceinline__ Post4 load_tiled(const AssignParams &P, int pos) {
-    Post4 r;
+__device__ __forceinline__ Quad<PREC, CID16> load_quad(const AssignParams &P, int pos) {
+    Quad<PREC, CID16> r;
     if constexpr (CID16 && PREC != SIVF_FP32) {
-        const uint4 w = ld_sparse_v4(P.sc_pack + pos, P.stream_sparse);
-        const unsigned ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            r.id[m] = (int)(ws[m] >> 16);
-            r.u[m] = decode_u<PREC>(ws[m] & 0xFFFFu);
-        }
-        return r;
+        r.a = ld_sparse_v4(P.sc_pack + pos, P.stream_sparse);
     } else {
         if constexpr (CID16) {
             const uint2 w = ld_sparse_v2(P.sc_id16 + pos, P.stream_sparse);
-            r.id[0] = (int)(w.x & 0xFFFFu);
-            r.id[1] = (int)(w.x >> 16);
-            r.id[2] = (int)(w.y & 0xFFFFu);
-            r.id[3] = (int)(w.y >> 16);
+            r.a.x = w.x;
+            r.a.y = w.y;
         } else {
-            const uint4 w = ld_sparse_v4(P.sc_id32 + pos, P.stream_sparse);
-            r.id[0] = (int)w.x;
-            r.id[1] = (int)w.y;
-            r.id[2] = (int)w.z;
-            r.id[3] = (int)w.w;
+            r.a = ld_sparse_v4(P.sc_id32 + pos, P.stream_sparse);
         }
         if constexpr (PREC == SIVF_FP32) {
-            const uint4 vw = ld_sparse_v4(P.sc_val + pos, P.stream_sparse);
-            const float4 v = make_float4(__uint_as_float(vw.x), __uint_as_float(vw.y), __uint_as_float(vw.z),
-                                         __uint_as_float(vw.w));
-            r.u[0] = v.x;
-            r.u[1] = v.y;
-            r.u[2] = v.z;
-            r.u[3] = v.w;
+            r.v[0] = ld_sparse_v4(P.sc_val + pos, P.stream_sparse);
         } else {
-            const uint2 v = ld_sparse_v2(P.sc_lp + pos, P.stream_sparse);
-            r.u[0] = decode_u<PREC>(v.x & 0xFFFFu);
-            r.u[1] = decode_u<PREC>(v.x >> 16);
-            r.u[2] = decode_u<PREC>(v.y & 0xFFFFu);
-            r.u[3] = decode_u<PREC>(v.y >> 16);
+            const uint2 w = ld_sparse_v2(P.sc_lp + pos, P.stream_sparse);
+            r.v[0].x = w.x;
+            r.v[0].y = w.y;
         }
-        return r;
+    }
+    return r;
+}
+
+__device__ __forceinline__ unsigned word_of(const uint4 &w, int m) {
+    return m == 0 ? w.x : (m == 1 ? w.y : (m == 2 ? w.z : w.w));
+}
+
+// position and value of posting m (0..3, a compile-time constant) of a quad
+template <int PREC, bool CID16>
+__device__ __forceinline__ void quad_entry(const Quad<PREC, CID16> &r, int m, int &id, float &u) {
+    if constexpr (CID16 && PREC != SIVF_FP32) {
+        const unsigned w = word_of(r.a, m);
+        id = (int)(w >> 16);
+        u = decode_u<PREC>(w & 0xFFFFu);
+    } else {
+        if constexpr (CID16) id = (int)((word_of(r.a, m >> 1) >> (16 * (m & 1))) & 0xFFFFu);
+        else id = (int)word_of(r.a, m);
+        if constexpr (PREC == SIVF_FP32) u = __uint_as_float(word_of(r.v[0], m));
+        else u = decode_u<PREC>((word_of(r.v[0], m >> 1) >> (16 * (m & 1))) & 0xFFFFu);
     }
 }
 
-// One posting at a canonical (tail) position.
+// One posting.
 template <int PREC, bool CID16>
 __device__ __forceinline__ void load_one(const AssignParams &P, int pos, int &id, float &u) {
     if constexpr (CID16 && PREC != SIVF_FP32) {
@@ -620,17 +592,13 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
     constexpr int NW = T / 32;
     const int kpad = (P.kmax + 3) & ~3;
     uint32_t *rho = GRHO ? P.grho + (size_t)blockIdx.x * kpad : smem;
-    // staged segment of thread h: {scan start, full-block end, end of the full
-    // fully scanned blocks, scaled value bits}, scanned length, item and
-    // row-posting prefixes; dense terms of the chunk: {row / 8, scaled value}
+    // staged segments (the sparse terms with postings to scan, in staging
+    // order): {scan start, postings, scaled value, end in quads of the chunk};
+    // dense terms of the chunk: {row / 8, scaled value}
     int4 *s_seg = reinterpret_cast<int4 *>(GRHO ? smem : smem + kpad);
     int2 *s_dense = reinterpret_cast<int2 *>(s_seg + T);
-    int *s_len = reinterpret_cast<int *>(s_dense + T);
-    int *s_item = s_len + T;
-    int *s_rend = s_item + T;
-    uint32_t *s_lam = reinterpret_cast<uint32_t *>(s_rend + T);  // CB: lambda^[r-1] bits of all clusters
-    __shared__ int4 warp_i4[32];
-    __shared__ int4 s_total4;
+    uint32_t *s_lam = reinterpret_cast<uint32_t *>(s_dense + T);  // CB: lambda^[r-1] bits of all clusters
+    __shared__ int2 warp_i2[NW];
     __shared__ long long s_obj;
     __shared__ uint32_t warp_b[NW], warp_s[NW];
     __shared__ double warp_d[NW];
@@ -651,7 +619,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
     // candidates, dense-row entries read
     __shared__ unsigned long long s_cnt[6];
     if (tid < 6) s_cnt[tid] = 0ull;
-    unsigned long long c_post_obj = 0, c_dpost = 0;
+    unsigned long long c_post_obj = 0, c_dpost = 0;  // per thread
     __syncthreads();
 
     const long long n_obj = (long long)P.ctr->n_heavy;
@@ -659,12 +627,17 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         if (tid == 0) s_obj = (long long)atomicAdd(&P.ctr->work, 1ull);
         __syncthreads();
         if (s_obj >= n_obj) break;
-        const int64_t i = P.heavy_ids[s_obj];
-        int64_t rb = P.row_ptr[i], re = P.row_ptr[i + 1];
-        if (P.checked && (rb < 0 || re < rb || re > P.nnz)) {
-            // the borrowed CSR changed since it was validated: record it, read nothing
-            if (tid == 0) atomicOr(&P.ctr->error, 1ull);
-            rb = re = 0;
+        const int i = P.heavy_ids[s_obj];
+        int rb, re;  // nnz < 2^31
+        {
+            int64_t b = P.row_ptr[i], e = P.row_ptr[i + 1];
+            if (P.checked && (b < 0 || e < b || e > P.nnz)) {
+                // the borrowed CSR changed since it was validated: record it, read nothing
+                if (tid == 0) atomicOr(&P.ctr->error, 1ull);
+                b = e = 0;
+            }
+            rb = (int)b;
+            re = (int)e;
         }
         // instance of object i: largest m with inst_obj[m] <= i
         int inst = 0;
@@ -680,14 +653,12 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         const int km = P.inst_k[inst + 1] - k_off;
         const int32_t a_prev = P.labels_prev[i];  // global id, -1 before the first assignment
         const int a_loc = a_prev >= 0 ? a_prev - k_off : -1;
-        const int a_pos = a_prev < 0 ? -1 : (CB ? a_loc : P.clu_pos[a_prev]);  // index of its score
         const uint32_t own_q = P.own[i];
         const bool filt = P.icp && a_prev >= 0 && own_q != OWN_INVALID && P.lam_prev[a_prev] != 0;
         const int mb = P.mov_beg[inst];
         const int n_mov_inst = P.mov_beg[inst + 1] - mb;
-        const int32_t *movs = P.mov_list + mb;
         // score index of the m-th moving cluster, and cluster id of a score index
-        auto mov_at = [&](int m) { return CB ? movs[m] - k_off : m; };
+        auto mov_at = [&](int m) { return CB ? P.mov_list[mb + m] - k_off : m; };
         auto id_at = [&](int p) { return CB ? p : P.pos_clu[k_off + p]; };
         // relaxed filter (icp = 3): the own cluster moved, and at most half of
         // the instance's clusters are moving; decided after the front scan
@@ -717,182 +688,107 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         // The object's terms are staged T at a time. A term with a dense row
         // is accumulated from it (dense_chunk). Every other term's segment
         // (the part of its posting list that is scanned: the front, or the
-        // whole list) splits into its full 128-entry blocks of the tiled
-        // layout whose postings are all scanned, and a remainder of fewer
-        // than 128 postings (the part of a block that a front ends inside, or
-        // the list's ragged tail). Work is done in two forms:
-        //  - items: two full blocks (the last one of a segment may hold one),
-        //    or a remainder of at least RMIN postings. In a full block lane l
-        //    reads postings l, 32+l, 64+l, 96+l with one vector load per
-        //    array; step m of the warp then touches postings 32m .. 32m+31,
-        //    whose positions are distinct banks on dense lists. Warp w takes a
-        //    contiguous range of the items;
-        //  - rows: the shorter remainders of all staged segments are laid end
-        //    to end and cut into rows of 32 postings, one posting per lane, so
-        //    short fronts keep every lane busy. Warp w takes a contiguous range
-        //    of rows; each lane walks forward through the segments.
-        constexpr int RMIN = 16;
+        // whole list) is cut into quads of four postings, each read with one
+        // vector load per array. The quads of all staged segments are laid end
+        // to end and dealt to the warps in rows of 32, one quad per lane, four
+        // rows in flight, so that long lists, short lists and fronts share the
+        // work evenly; a lane walks forward through the segments. (Work items
+        // of whole 128-posting blocks with separate remainders left a warp one
+        // dependent load batch per list: the sparse phase of the k = 20,000
+        // corpus was paid per list, not per posting.)
         for (int pass = 0;; ++pass) {
         const bool front = (filt || relax) && pass == 0;  // scan the fronts only
         const int npos = front && !CB ? n_mov_inst : km;  // score positions this pass covers
-        for (int64_t cb = rb; cb == rb || cb < re; cb += T) {  // an empty row still sets its scores
-            const int cn = (int)min((int64_t)T, re - cb);
-            int4 cnt = make_int4(0, 0, 0, 0);
+        for (int cb = rb; cb == rb || cb < re; cb += T) {  // an empty row still sets its scores; cb < nnz + T
+            const int cn = min(T, re - cb);
+            int2 cnt = make_int2(0, 0);  // quads; segments << 16 | dense terms
             int2 dent = make_int2(-1, 0);
+            int4 seg = make_int4(0, 0, 0, 0);
             if (tid < cn) {
                 int t = P.idx[cb + tid];
                 if (P.checked && (t < 0 || t >= P.D)) {  // a term outside [0, D): record it, skip it
                     atomicOr(&P.ctr->error, 2ull);
                     t = -1;
                 }
-                const int64_t o0 = t >= 0 ? P.if_off[t] : 0;
-                const int lfull = t >= 0 ? (int)(P.if_off[t + 1] - o0) : 0;
-                const int len = t < 0 ? 0 : ((front && !CB) ? P.if_mf0[t] : lfull);
+                const int4 td = t >= 0 ? __ldg(P.tdesc + t) : make_int4(0, 0, 0, -1);
+                const int len = (front && !CB) ? td.y : td.z;
                 float vs = P.val[cb + tid] * FIX_SCALE;  // exact: power-of-two scaling
-                const int dr = (CB || t < 0) ? -1 : P.dense_row[t];
                 c_post_obj += (unsigned long long)len;
-                if (dr >= 0) {  // dense row: no segment to scan
+                if (td.w >= 0) {  // dense row: no segment to scan
                     if constexpr (PREC == SIVF_FP16) vs *= FP16_INV_SCALE;  // rows hold u * 2^14 (exact)
-                    dent = make_int2(dr, __float_as_int(vs));
-                    cnt.z = 1;
+                    dent = make_int2(td.w, __float_as_int(vs));
+                    cnt.y = 1;
                     c_dpost += (unsigned long long)len;
-                    s_seg[tid] = make_int4(0, 0, 0, 0);
-                    s_len[tid] = 0;
-                } else {
-                    const int fb = lfull & ~(SC_BLK - 1);
-                    const int r0 = min(len, fb) & ~(SC_BLK - 1);  // postings in full, fully scanned blocks
-                    s_seg[tid] = make_int4(t >= 0 ? (int)P.sc_off[t] : 0, fb, r0, __float_as_int(vs));
-                    s_len[tid] = len;
-                    const int rem = len - r0;
-                    cnt.x = rem >= RMIN ? (r0 + CH - 1) / CH + 1 : (r0 + CH - 1) / CH;
-                    cnt.y = rem >= RMIN ? 0 : rem;
+                } else if (len > 0) {
+                    seg = make_int4(td.x, len, __float_as_int(vs), 0);
+                    cnt = make_int2((len + 3) >> 2, 1 << 16);
                 }
             }
-            const int4 incl = block_inclusive_scan_int4<T>(cnt, warp_i4, &s_total4);
-            s_item[tid] = incl.x;
-            s_rend[tid] = incl.y;
-            if (dent.x >= 0) s_dense[incl.z - 1] = dent;  // dense terms in staging order
+            int2 tot;
+            const int2 incl = block_inclusive_scan_int2<T>(cnt, warp_i2, tot);
+            if (cnt.x > 0) {
+                seg.w = incl.x;
+                s_seg[(incl.y >> 16) - 1] = seg;
+            }
+            if (dent.x >= 0) s_dense[(incl.y & 0xFFFF) - 1] = dent;  // dense terms in staging order
             __syncthreads();
-            const int4 tot = s_total4;
+            const int n_quads = tot.x, n_seg = tot.y >> 16, n_dense = tot.y & 0xFFFF;
 
             // dense rows
-            if (tot.z > 0 || cb == rb) {
-                nd_obj += tot.z;
-                dense_chunk<T, PREC, GRHO>(P, rho, s_dense, tot.z, npos, cb == rb);
-                if (tid == 0) s_cnt[5] += (unsigned long long)tot.z * (unsigned long long)npos;
-                if (tot.x > 0 || tot.y > 0) __syncthreads();  // plain accesses above, atomics below
+            if (n_dense > 0 || cb == rb) {
+                nd_obj += n_dense;
+                dense_chunk<T, PREC, GRHO>(P, rho, s_dense, n_dense, npos, cb == rb);
+                if (tid == 0) s_cnt[5] += (unsigned long long)n_dense * (unsigned long long)npos;
+                if (n_quads > 0) __syncthreads();  // plain accesses above, atomics below
             }
 
-            // items
+            // sparse postings
             {
-                const int per_warp = (tot.x + NW - 1) / NW;
-                const int it0 = warp * per_warp;
-                const int it1 = min(tot.x, it0 + per_warp);
-                if (it0 < it1) {
-                    int h = first_greater<T>(s_item, it0);
-                    int h_first = h ? s_item[h - 1] : 0, h_end = s_item[h];
-                    int4 sg = s_seg[h];
-                    for (int it = it0; it < it1;) {
-                        int step = 1;
-                        if (it >= h_end) {
-                            do {
-                                ++h;
-                            } while (s_item[h] <= it);
-                            h_first = s_item[h - 1];
-                            h_end = s_item[h];
-                            sg = s_seg[h];
-                        }
-                        const int sb = sg.x, fb = sg.y, r0 = sg.z;
-                        const float vs = __int_as_float(sg.w);
-                        const int off = (it - h_first) * CH;
-                        if (off + CH + SC_BLK < r0 && it + 1 < it1 && it + 1 < h_end) {
-                            // this item and the next are two full blocks each in
-                            // the same segment: four loads in flight
-                            const int pos = sb + off + 4 * lane;
-                            const Post4 a = load_tiled<PREC, CID16>(P, pos);
-                            const Post4 b = load_tiled<PREC, CID16>(P, pos + SC_BLK);
-                            const Post4 c = load_tiled<PREC, CID16>(P, pos + 2 * SC_BLK);
-                            const Post4 e = load_tiled<PREC, CID16>(P, pos + 3 * SC_BLK);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(a.id[m], vs * a.u[m]);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(b.id[m], vs * b.u[m]);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(c.id[m], vs * c.u[m]);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(e.id[m], vs * e.u[m]);
-                            step = 2;
-                        } else if (off + SC_BLK < r0) {  // two full blocks
-                            const int pos = sb + off + 4 * lane;
-                            const Post4 a = load_tiled<PREC, CID16>(P, pos);
-                            const Post4 b = load_tiled<PREC, CID16>(P, pos + SC_BLK);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(a.id[m], vs * a.u[m]);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(b.id[m], vs * b.u[m]);
-                        } else if (off < r0) {  // the segment's odd last full block
-                            const Post4 a = load_tiled<PREC, CID16>(P, sb + off + 4 * lane);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) add(a.id[m], vs * a.u[m]);
-                        } else {  // a remainder of RMIN .. 127 postings, starting at r0
-                            const int rem = s_len[h] - r0;
-                            if (r0 < fb) {
-                                // inside a full block of the list (the load stays in it)
-                                const Post4 a = load_tiled<PREC, CID16>(P, sb + r0 + 4 * lane);
-#pragma unroll
-                                for (int m = 0; m < 4; ++m)
-                                    if (32 * m + lane < rem) add(a.id[m], vs * a.u[m]);
-                            } else {  // the ragged tail, canonical order
-                                int id[4];
-                                float u[4];
-#pragma unroll
-                                for (int m = 0; m < 4; ++m)
-                                    if (32 * m + lane < rem) load_one<PREC, CID16>(P, sb + r0 + 32 * m + lane, id[m], u[m]);
-#pragma unroll
-                                for (int m = 0; m < 4; ++m)
-                                    if (32 * m + lane < rem) add(id[m], vs * u[m]);
-                            }
-                        }
-                        it += step;
-                    }
-                }
-            }
-
-            // rows: remainders shorter than RMIN, one posting per lane
-            if (tot.y > 0) {
-                constexpr int RU = 2;  // rows per step
-                const int rows = (tot.y + 31) >> 5;
+                constexpr int RU = CID16 && PREC != SIVF_FP32 ? 4 : 2;  // rows in flight
+                const int rows = (n_quads + 31) >> 5;
                 const int per_warp = (rows + NW - 1) / NW;
                 const int w0 = warp * per_warp;
                 const int w1 = min(rows, w0 + per_warp);
                 if (w0 < w1) {
-                    int h = first_greater<T>(s_rend, min(w0 * 32 + lane, tot.y - 1));
-                    int hb = h ? s_rend[h - 1] : 0, he = s_rend[h];
+                    // the segment of this lane's first quad: smallest h whose end lies beyond it
+                    int h = 0;
+                    {
+                        const int q = min(w0 * 32 + lane, n_quads - 1);
+                        int hi = n_seg - 1;
+                        while (h < hi) {
+                            const int mid = (h + hi) >> 1;
+                            if (s_seg[mid].w > q) hi = mid; else h = mid + 1;
+                        }
+                    }
                     int4 sg = s_seg[h];
                     for (int row = w0; row < w1; row += RU) {
-                        int id[RU];
-                        float u[RU], vv[RU];
-                        bool ok[RU];
+                        Quad<PREC, CID16> qd[RU];
+                        float vv[RU];
+                        int left[RU];  // postings of the quad that belong to the segment (more than 4: all)
 #pragma unroll
                         for (int m = 0; m < RU; ++m) {
                             const int q = (row + m) * 32 + lane;
-                            ok[m] = row + m < w1 && q < tot.y;
-                            if (ok[m]) {
-                                if (q >= he) {
-                                    do {
-                                        ++h;
-                                        hb = he;
-                                        he = s_rend[h];
-                                    } while (q >= he);
-                                    sg = s_seg[h];
-                                }
-                                load_one<PREC, CID16>(P, sg.x + tiled_offset(sg.z + (q - hb), sg.y), id[m], u[m]);
-                                vv[m] = __int_as_float(sg.w);
+                            left[m] = 0;
+                            if (row + m < w1 && q < n_quads) {
+                                while (q >= sg.w) sg = s_seg[++h];
+                                const int o = 4 * (q - sg.w + ((sg.y + 3) >> 2));
+                                left[m] = sg.y - o;
+                                vv[m] = __int_as_float(sg.z);
+                                qd[m] = load_quad<PREC, CID16>(P, sg.x + o);
                             }
                         }
 #pragma unroll
-                        for (int m = 0; m < RU; ++m)
-                            if (ok[m]) add(id[m], vv[m] * u[m]);
+                        for (int m = 0; m < RU; ++m) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                if (e < left[m]) {
+                                    int id;
+                                    float u;
+                                    quad_entry<PREC, CID16>(qd[m], e, id, u);
+                                    add(id, vv[m] * u);
+                                }
+                            }
+                        }
                     }
                 }
             }
@@ -905,13 +801,13 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         // rho~_new - E(rho~_new) >= rho~_old + E(rho~_old), which implies it
         // for the exact scores; otherwise scan everything again.
         if (tid == 0) {
-            const double xn = (double)rho_ld<GRHO>(rho + a_pos) * FIX_QUANTUM;
+            const double xn = (double)rho_ld<GRHO>(rho + (CB ? a_loc : P.clu_pos[a_prev])) * FIX_QUANTUM;
             const double xo = (double)own_q * FIX_QUANTUM;
             const double S = (double)P.sumv[i];
             // the old score came from an earlier scan, whose dense terms may
             // have differed: bound it with every term counted as dense
             s_flag = xn - error_bound(xn, re - rb, nd_obj, S, P.eps, P.eta) >=
-                     xo + error_bound(xo, re - rb, (int)(re - rb), S, P.eps, P.eta);
+                     xo + error_bound(xo, re - rb, re - rb, S, P.eps, P.eta);
         }
         __syncthreads();
         if (s_flag) break;
@@ -951,10 +847,10 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         warp_top2(bv, sv);
         const uint32_t top = bv;      // largest scanned score
         if (filt) top2_add(bv, sv, own_q);
-        const int64_t n_terms = re - rb;
+        const int n_terms = re - rb;
         // a filtered object's carried own score may come from a scan with
         // other dense terms: count every term as dense for it
-        const int nd_bound = filt ? (int)n_terms : nd_obj;
+        const int nd_bound = filt ? n_terms : nd_obj;
         bool flag = bv > 0u && ncand + (filt ? 1 : 0) > 1 &&
                     !clear_of_bound(bv, bv - sv, n_terms, nd_bound, P.eps_f,
                                     P.eta_q != 0.f ? P.eta_q * P.sumv[i] : 0.f);
@@ -992,7 +888,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
                     // (position 0 holds the lowest moving id, and id 0 unfiltered);
                     // else the own cluster, which no scanned score reaches
                     int al = filt ? a_loc : INT32_MAX;
-                    if (bv == 0u && ncand > 0) al = min(al, sub ? movs[0] - k_off : 0);
+                    if (bv == 0u && ncand > 0) al = min(al, sub ? P.mov_list[mb] - k_off : 0);
                     finish(al, bv);
                 }
             } else if (mine == top) {  // one thread: a second one would make the gap zero
@@ -1215,7 +1111,7 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
                             atomicOr(&P.ctr->error, 2ull);
                             t = -1;
                         }
-                        const int dr = t >= 0 ? P.dense_row[t] : -1;
+                        const int dr = t >= 0 ? P.tdesc[t].w : -1;
                         if (dr >= 0) {
                             float vs = P.val[h] * FIX_SCALE;
                             if constexpr (PREC == SIVF_FP16) vs *= FP16_INV_SCALE;
@@ -1245,20 +1141,20 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
             // sparse fronts of the chunk's other terms, one segment at a time, lane-strided
             for (int64_t s0 = cb; s0 < ce; s0 += 32) {
                 const int64_t h = s0 + lane;
-                int len = 0, sb = 0, fb = 0;
+                int len = 0, sb = 0;
                 float vs = 0.f;
                 if (h < ce) {
                     int t = P.idx[h];
                     if (P.checked && (t < 0 || t >= P.D)) t = -1;
                     if (t >= 0) {
-                        len = P.if_mf0[t];
+                        const int4 td = __ldg(P.tdesc + t);
+                        len = td.y;
                         c_post += (unsigned long long)len;
-                        if (P.dense_row[t] >= 0) {
+                        if (td.w >= 0) {
                             c_dpost += (unsigned long long)len;
                             len = 0;
                         } else {
-                            sb = (int)P.sc_off[t];
-                            fb = (int)(P.if_off[t + 1] - P.if_off[t]) & ~(SC_BLK - 1);
+                            sb = td.x;
                             vs = P.val[h] * FIX_SCALE;
                         }
                     }
@@ -1268,12 +1164,11 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
                     const int src = __ffs(m) - 1;
                     m &= m - 1;
                     const int L = __shfl_sync(FULL, len, src), b = __shfl_sync(FULL, sb, src);
-                    const int f = __shfl_sync(FULL, fb, src);
                     const float v = __shfl_sync(FULL, vs, src);
                     for (int o = lane; o < L; o += 32) {
                         int id;
                         float u;
-                        load_one<PREC, CID16>(P, b + tiled_offset(o, f), id, u);
+                        load_one<PREC, CID16>(P, b + o, id, u);
                         atomicAdd(rho + id, __float2uint_ru(v * u));
                     }
                 }
@@ -1482,9 +1377,7 @@ cudaError_t launch_assign(sivf_ctx *c) {
     P.idx = c->idx;
     P.val = c->val;
     P.sumv = c->sumv;
-    P.if_off = c->if_off;
-    P.if_mf0 = c->if_mf0;
-    P.sc_off = c->sc_off;
+    P.tdesc = c->tdesc;
     P.sc_id16 = c->sc_id16;
     P.sc_id32 = c->sc_id32;
     P.sc_val = c->sc_val;
@@ -1492,7 +1385,6 @@ cudaError_t launch_assign(sivf_ctx *c) {
     P.sc_lp = c->sc_lp;
     P.clu_pos = c->clu_pos;
     P.pos_clu = c->pos_clu;
-    P.dense_row = c->dense_row;
     P.dense = c->dense_val;
     P.grho = c->grho;
     P.coff = c->coff[c->cur];

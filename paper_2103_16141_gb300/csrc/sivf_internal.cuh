@@ -15,18 +15,16 @@
 //                                        if_val f32[cap]: canonical order (front ids
 //                                        ascending, then back ids ascending), built
 //                                        on demand for the getters
-//   scan copy of the file sc_off int64[D+1]: each list starts at a multiple of 4
-//                                        entries; a list's full 128-entry blocks are
-//                                        stored transposed (entry 32m + l of a block at
-//                                        block position 4l + m), so that lane l reads
-//                                        entries l, 32+l, 64+l, 96+l with one vector
-//                                        load; the ragged tail keeps list order. Inside
-//                                        a segment the postings are in the order the
-//                                        build's atomic cursor handed out.
-//                                        Arrays (scan positions): sc_id16 u16 or
-//                                        sc_id32 int32, plus sc_val f32 (FP32), or
-//                                        sc_pack u32 = id << 16 | bf16/fp16 value
-//                                        (16-bit ids and values), or sc_lp u16
+//   term table            tdesc int4[D]: start of term t's list in the scan copy,
+//                                        front length, list length, and first entry / 8
+//                                        of its dense row or -1 (the term is scanned
+//                                        from the sparse copy)
+//   scan copy of the file sc_*           lists without a dense row, front then back; each
+//                                        starts at a multiple of 4 entries and has room
+//                                        for a multiple of 4, so that four postings are
+//                                        one vector load. Inside a segment the postings
+//                                        are in the order the build's atomic cursor
+//                                        handed out.
 //                                        Ids in the scan copy are scan positions (below).
 //   scan order            clu_pos int32[k]: position of cluster j in its instance's
 //                                        scan order (moving clusters of lambda^[r] first,
@@ -34,8 +32,7 @@
 //                                        id); pos_clu int32[k]: the inverse (instance
 //                                        offset + position -> local id). Score vectors are
 //                                        indexed by position. IVF-CBICP keeps id order.
-//   dense head rows       dense_row int32[D]: first entry / 8 of term t's dense row, or
-//                                        -1 (the term is scanned from the sparse copy);
+//   dense head rows
 //                                        dense_val (u16 or f32) [cap_dense]: one row per dense
 //                                        term, the term's value for every cluster of its
 //                                        instance at the cluster's scan position (0 where
@@ -64,12 +61,10 @@ namespace sivf {
 constexpr uint32_t OWN_INVALID = 0xFFFFFFFFu;
 // tail padding (entries) of the inverted-file posting arrays
 constexpr int64_t IF_PAD = 256;
-// block of the tiled scan layout: 32 lanes x 4 entries
-constexpr int SC_BLK = 128;
 // shared memory the assignment kernel stages per thread besides the score
-// vector: list start, full-block end, end of the full scanned blocks, scaled
-// value, scanned length, item prefix, row-posting prefix, dense row and value
-constexpr int ASSIGN_STAGE_BYTES = 36;
+// vector: a segment (scan start, postings, scaled value, end in quads) and a
+// dense term (row, scaled value)
+constexpr int ASSIGN_STAGE_BYTES = 24;
 // Scores are accumulated as unsigned fixed point with quantum 2^-31:
 // q = ceil(fl(v * u) * 2^31). Cosine scores are <= 1 (+ rounding), so the
 // sum of an object's terms stays below 2^32.
@@ -162,9 +157,9 @@ struct sivf_ctx {
     float *if_val = nullptr;
     int64_t if_nnz = 0;
     bool canon_stale = true;  // if_cid / if_val predate the last inverted-file build
-    // scan copy (tiled layout, local ids); which arrays exist depends on the
+    // term table and scan copy (local ids); which arrays exist depends on the
     // id width (16 bits when every instance has k <= 65536) and the precision
-    int64_t *sc_off = nullptr;
+    int4 *tdesc = nullptr;
     uint16_t *sc_id16 = nullptr;
     int32_t *sc_id32 = nullptr;
     float *sc_val = nullptr;      // FP32 postings
@@ -173,7 +168,6 @@ struct sivf_ctx {
     int64_t cap_s = 0;            // entries of each scan array
     // scan order and dense head rows (see the layout above)
     int32_t *clu_pos = nullptr, *pos_clu = nullptr;
-    int32_t *dense_row = nullptr;
     void *dense_val = nullptr;    // dense rows: u16 (BF16/FP16) or f32 entries
     int64_t cap_dense = 0;        // entries of dense (0: no dense rows)
     float dense_frac = 0.f;       // list length / k from which a term gets a dense row

@@ -717,15 +717,6 @@ __global__ void k_if_lens(int32_t D, const uint32_t *cnt2, int64_t *len, int64_t
     }
 }
 
-// Position of entry p of a list of length L in the tiled scan layout: inside
-// the list's full 128-entry blocks, entry 32m + l of a block sits at block
-// position 4l + m; the ragged tail keeps canonical order.
-__device__ __forceinline__ int64_t tiled_pos(int64_t p, int64_t L) {
-    const int64_t fb = L & ~(int64_t)(SC_BLK - 1);
-    if (p >= fb) return p;
-    return (p & ~(int64_t)(SC_BLK - 1)) | ((p & 31) << 2) | ((p >> 5) & 3);
-}
-
 // Canonical arrays (if_cid: global cluster ids, if_val) in sorted order.
 __global__ void k_if_fill(const int64_t *n_dev, int64_t cap, const uint32_t *order, const int32_t *cclu,
                           const float *cval, int32_t *if_cid, float *if_val) {
@@ -832,12 +823,14 @@ __global__ void k_dense_width(int32_t D, int32_t n_inst, const int32_t *inst_d, 
     }
 }
 
-__global__ void k_dense_rows(int32_t D, const int64_t *w8, const int64_t *base8, int32_t *dense_row,
-                             DevCounters *ctr) {
+// What the assignment reads about a term, in one 16-byte load: where its list
+// starts in the scan copy, its front and list lengths, and its dense row.
+__global__ void k_term_desc(int32_t D, const int64_t *w8, const int64_t *base8, const int64_t *sc_off,
+                            const int32_t *mf0, const int64_t *len, int4 *tdesc, DevCounters *ctr) {
     long long n = 0;
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D; g += (int64_t)gridDim.x * blockDim.x) {
         const bool d = w8[g] > 0;
-        dense_row[g] = d ? (int32_t)base8[g] : -1;
+        tdesc[g] = make_int4((int)sc_off[g], mf0[g], (int)len[g], d ? (int)base8[g] : -1);
         n += d;
     }
     if (n) atomicAdd(reinterpret_cast<unsigned long long *>(&ctr->dense_terms), (unsigned long long)n);
@@ -871,30 +864,27 @@ __global__ void k_if_count(const int64_t *n_dev, int64_t cap, const int32_t *cte
 // centroid entries (one pass, no sort): an entry of a term with a dense row
 // goes to the row at its cluster's scan position; any other entry takes the
 // next free slot of its term's front (moving cluster) or back (invariant
-// cluster) in the scan copy, stored at the slot's tiled position with the
-// cluster's scan position as its id. The order of the postings inside a
+// cluster) in the scan copy, with the cluster's scan position as its id. The order of the postings inside a
 // segment follows the atomic cursor; no score depends on it (each posting is
 // one integer add).
 __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
                             const float *cval, const uint8_t *lam, int structured, const int32_t *clu_pos,
-                            const int32_t *dense_row, const int64_t *if_off, const int32_t *if_mf0,
-                            const int64_t *sc_off, uint32_t *cursor, int prec, void *dense, uint16_t *sc_id16,
+                            const int4 *tdesc, uint32_t *cursor, int prec, void *dense, uint16_t *sc_id16,
                             int32_t *sc_id32, float *sc_val, uint32_t *sc_pack, uint16_t *sc_lp) {
     const int64_t n = min(*n_dev, cap);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t t = cterm[e], j = cclu[e];
         const float u = cval[e];
         const uint32_t p = (uint32_t)clu_pos[j];
-        const int32_t r = dense_row[t];
-        if (r >= 0) {
-            const int64_t d = (int64_t)r * 8 + p;
+        const int4 td = tdesc[t];
+        if (td.w >= 0) {
+            const int64_t d = (int64_t)td.w * 8 + p;
             if (prec == SIVF_FP32) static_cast<float *>(dense)[d] = u;
             else static_cast<uint16_t *>(dense)[d] = encode_lp(u, prec);
             continue;
         }
         const uint32_t part = (structured && lam[j]) ? 1u : 0u;
-        const int64_t slot = (int64_t)atomicAdd(cursor + (((uint32_t)t << 1) | part), 1u) + (part ? if_mf0[t] : 0);
-        const int64_t pos = sc_off[t] + tiled_pos(slot, if_off[t + 1] - if_off[t]);
+        const int64_t pos = (int64_t)td.x + atomicAdd(cursor + (((uint32_t)t << 1) | part), 1u) + (part ? td.y : 0);
         if (sc_id16) sc_id16[pos] = (uint16_t)p;
         if (sc_id32) sc_id32[pos] = (int32_t)p;
         if (prec == SIVF_FP32) {
@@ -1045,11 +1035,10 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     SIVF_CUDA_TRY(cudaGetLastError());
     SIVF_CUDA_TRY(scan_exclusive_i64(len, c->if_off, D, total, ws, s));
     SIVF_CUDA_TRY(cudaMemcpyAsync(c->if_off + D, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(scan_exclusive_i64(slen, c->sc_off, D, total + 1, ws, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->sc_off + D, total + 1, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    SIVF_CUDA_TRY(scan_exclusive_i64(slen, slen, D, total + 1, ws, s));
     SIVF_CUDA_TRY(scan_exclusive_i64(w8, base8, D, total + 2, ws, s));
     SIVF_CUDA_TRY(cudaMemsetAsync(&c->ctr->dense_terms, 0, sizeof(long long), s));
-    k_dense_rows<<<blocks_gs(D), TPB, 0, s>>>(D, w8, base8, c->dense_row, c->ctr);
+    k_term_desc<<<blocks_gs(D), TPB, 0, s>>>(D, w8, base8, slen, c->if_mf0, len, c->tdesc, c->ctr);
     note_launch();
     if (dense) {
         const int esize = c->cfg.prec == SIVF_FP32 ? 4 : 2;
@@ -1060,8 +1049,7 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     // the counts are consumed: the same array now hands out the slots
     SIVF_CUDA_TRY(cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * 2 * D, s));
     k_scan_fill<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, c->cterm[cur], c->cclu, c->cval[cur], c->lam, cb ? 0 : 1,
-                                                c->clu_pos, c->dense_row, c->if_off, c->if_mf0, c->sc_off, cnt2,
-                                                (int)c->cfg.prec, c->dense_val, c->sc_id16, c->sc_id32, c->sc_val,
+                                                c->clu_pos, c->tdesc, cnt2, (int)c->cfg.prec, c->dense_val, c->sc_id16, c->sc_id32, c->sc_val,
                                                 c->sc_pack, c->sc_lp);
     note_launch();
     SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->dense_used, total + 2, sizeof(long long), cudaMemcpyDeviceToDevice, s));

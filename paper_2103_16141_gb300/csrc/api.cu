@@ -85,12 +85,29 @@ cudaError_t read_file_counters(sivf_ctx *c) {
 void pick_assign_config(sivf_ctx *c) {
     int T = c->cfg.threads;
     if (T != 32 && T != 64 && T != 128 && T != 256 && T != 512) T = 0;
-    if (T == 0) T = c->kmax <= 2048 ? 64 : (c->kmax <= 4096 ? 128 : 512);  // measured on the k = 1000 and k = 10,000 corpora
-    c->assign_threads = T;
-    c->assign_ctas_per_sm = c->cfg.ctas_per_sm > 0 ? c->cfg.ctas_per_sm : 0;
-    int dev = 0, smem = 0;
+    int dev = 0, smem = 0, sm_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (T == 0) {
+        // The smallest CTA of which 1024 threads (the register budget's 32
+        // warps) still reside on an SM: CTAs wait at their own barriers only,
+        // so more and smaller ones overlap the phases of more objects, until
+        // the score vectors take the room. Assignment times, ms per iteration
+        // from the second on, at 64 / 128 / 256 / 512 threads: k = 1000 FP32
+        // 11.0 / 11.3 / 16.4 / -; k = 3001 FP16 2.45 / 2.13 / 2.59 / -;
+        // k = 10,000 BF16 - / - / 23.3 / 28.7; k = 20,000 BF16 - / - / 82 / 55.
+        T = 512;
+        for (int t = 64; t < 512; t *= 2) {
+            const size_t cta = (size_t)((c->kmax + 3) & ~3) * 4 + (size_t)t * ASSIGN_STAGE_BYTES + 2560;  // + static, reserved
+            if ((size_t)sm_smem / cta * (size_t)t >= 1024) {
+                T = t;
+                break;
+            }
+        }
+    }
+    c->assign_threads = T;
+    c->assign_ctas_per_sm = c->cfg.ctas_per_sm > 0 ? c->cfg.ctas_per_sm : 0;
     const bool fits = ((size_t)((c->kmax + 3) & ~3) * 4 + (size_t)T * ASSIGN_STAGE_BYTES) <= (size_t)smem;
     c->assign_global = c->cfg.score_buffer == 2 || (c->cfg.score_buffer == 0 && !fits) ? 1 : 0;
     if (c->cfg.icp == 2) {  // IVF-CBICP: 128 threads, shared score vector, no tuning

@@ -99,7 +99,7 @@ void pick_assign_config(sivf_ctx *c) {
         // k = 10,000 BF16 - / - / 23.3 / 28.7; k = 20,000 BF16 - / - / 82 / 55.
         T = 512;
         for (int t = 64; t < 512; t *= 2) {
-            const size_t cta = (size_t)((c->kmax + 3) & ~3) * 4 + (size_t)t * ASSIGN_STAGE_BYTES + 2560;  // + static, reserved
+            const size_t cta = (size_t)((c->kmax + 7) & ~7) * 4 + (size_t)t * ASSIGN_STAGE_BYTES + 2560;  // + static, reserved
             if ((size_t)sm_smem / cta * (size_t)t >= 1024) {
                 T = t;
                 break;
@@ -108,7 +108,7 @@ void pick_assign_config(sivf_ctx *c) {
     }
     c->assign_threads = T;
     c->assign_ctas_per_sm = c->cfg.ctas_per_sm > 0 ? c->cfg.ctas_per_sm : 0;
-    const bool fits = ((size_t)((c->kmax + 3) & ~3) * 4 + (size_t)T * ASSIGN_STAGE_BYTES) <= (size_t)smem;
+    const bool fits = ((size_t)((c->kmax + 7) & ~7) * 4 + (size_t)T * ASSIGN_STAGE_BYTES) <= (size_t)smem;
     c->assign_global = c->cfg.score_buffer == 2 || (c->cfg.score_buffer == 0 && !fits) ? 1 : 0;
     if (c->cfg.icp == 2) {  // IVF-CBICP: 128 threads, shared score vector, no tuning
         c->assign_threads = 128;
@@ -186,7 +186,7 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     if (c->cfg.icp == 2) {  // the IVF-CBICP kernel keeps the score vector and lambda bits in shared memory
         int smem = 0;
         INIT_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device), "attr");
-        const size_t need = (size_t)((c->kmax + 3) & ~3) * 4 + 128 * (size_t)ASSIGN_STAGE_BYTES +
+        const size_t need = (size_t)((c->kmax + 7) & ~7) * 4 + 128 * (size_t)ASSIGN_STAGE_BYTES +
                             (size_t)((k + 31) >> 5) * 4;
         if (need > (size_t)smem) {
             free_all(c);
@@ -241,11 +241,11 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     INIT_CUDA(dmalloc(c, &c->cclu, capc), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_off, (size_t)D + 1), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_mf0, D), "alloc");
-    // posting arrays carry a small tail pad; the scan copy also pads every
-    // list to a multiple of 4 entries
+    // posting arrays carry a small tail pad; the scan copy also fills the front
+    // and the back of every list up to a multiple of 4 entries
     INIT_CUDA(dmalloc(c, &c->if_cid, capc + IF_PAD), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_val, capc + IF_PAD), "alloc");
-    c->cap_s = capc + 3 * (int64_t)D + IF_PAD;
+    c->cap_s = capc + 3 * std::min<int64_t>(2 * (int64_t)D, capc) + IF_PAD;
     const size_t caps = (size_t)c->cap_s;
     const bool ids16 = c->kmax <= 65536;
     INIT_CUDA(dmalloc(c, &c->tdesc, D), "alloc");
@@ -295,8 +295,8 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     if (c->assign_global || c->cfg.autotune) {
         // global score vectors: one kmax slab per resident CTA (at most 16 per SM)
         c->grho_ctas = (int64_t)c->num_sms * 16;
-        INIT_CUDA(dmalloc(c, &c->grho, (size_t)c->grho_ctas * ((c->kmax + 3) & ~3)), "alloc");
-        INIT_CUDA(cudaMemsetAsync(c->grho, 0, sizeof(uint32_t) * (size_t)c->grho_ctas * ((c->kmax + 3) & ~3),
+        INIT_CUDA(dmalloc(c, &c->grho, (size_t)c->grho_ctas * ((c->kmax + 7) & ~7)), "alloc");
+        INIT_CUDA(cudaMemsetAsync(c->grho, 0, sizeof(uint32_t) * (size_t)c->grho_ctas * ((c->kmax + 7) & ~7),
                                   c->stream), "memset");
     }
     INIT_CUDA(dmalloc(c, &c->loop_dev, 4), "alloc");
@@ -344,7 +344,8 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
         size_t phase1 = 4 * (size_t)N * 4 + 2 * n8 + 14 * k8 + (c->dense ? 0 : 64 * ((size_t)nnz + 1)) + 32 * 4096;
         // u5: sort arrays (16 B x entries), per-term counts, lengths, dense widths
         // and offsets (40 B x terms), the dense-length histogram
-        size_t phase2 = 16 * ((size_t)capc + 1) + 40 * ((size_t)D + 1) + 16 * 4096;
+        // (per-term counts with the first, all of the second's arrays without it)
+        size_t phase2 = std::max(16 * ((size_t)capc + 1) + 8 * ((size_t)D + 1), 40 * ((size_t)D + 1)) + 16 * 4096;
         size_t ws = phase1 > phase2 ? phase1 : phase2;
         size_t maxn = (size_t)(capc > N ? capc : N);
         ws += (maxn / 4096 + 2) * 1024 * 4 + (maxn / 2048 + 2) * 16 + 64 * 256 + (1 << 20);

@@ -15,17 +15,17 @@
 //                                        if_val f32[cap]: canonical order (front ids
 //                                        ascending, then back ids ascending), built
 //                                        on demand for the getters
-//   term table            tdesc int4[D]: start of term t's list in the scan copy,
+//   term table            tdesc int4[D]: first quad of term t's list in the scan copy,
 //                                        front length, list length, and first entry / 8
 //                                        of its dense row or -1 (the term is scanned
 //                                        from the sparse copy)
-//   scan copy of the file sc_*           lists without a dense row, front then back; each
-//                                        starts at a multiple of 4 entries and has room
-//                                        for a multiple of 4, so that four postings are
-//                                        one vector load. Inside a segment the postings
-//                                        are in the order the build's atomic cursor
-//                                        handed out.
-//                                        Ids in the scan copy are scan positions (below).
+//   scan copy of the file sc_*           lists without a dense row, front then back, each
+//                                        filled up to a multiple of 4 entries with zero
+//                                        postings, so that four postings are one vector
+//                                        load. Inside a part the postings are in the
+//                                        order the build's atomic cursor handed out.
+//                                        Ids in the scan copy are score slots (score_slot of the
+//                                        scan position, below).
 //   scan order            clu_pos int32[k]: position of cluster j in its instance's
 //                                        scan order (moving clusters of lambda^[r] first,
 //                                        ascending id, then the invariant ones, ascending
@@ -62,7 +62,7 @@ constexpr uint32_t OWN_INVALID = 0xFFFFFFFFu;
 // tail padding (entries) of the inverted-file posting arrays
 constexpr int64_t IF_PAD = 256;
 // shared memory the assignment kernel stages per thread besides the score
-// vector: a segment (scan start, postings, scaled value, end in quads) and a
+// vector: a segment (first quad, quads, scaled value, end in quads) and a
 // dense term (row, scaled value)
 constexpr int ASSIGN_STAGE_BYTES = 24;
 // Scores are accumulated as unsigned fixed point with quantum 2^-31:
@@ -74,6 +74,13 @@ constexpr double FIX_QUANTUM = 4.656612873077392578125e-10;  // 2^-31
 // normal half-precision number.
 constexpr float FP16_SCALE = 16384.0f;
 constexpr float FP16_INV_SCALE = 1.0f / 16384.0f;
+
+// Where the score of scan position p is kept in a score vector: an involution
+// inside each aligned group of eight positions. A warp's lanes add to positions
+// that are 8 (or 4) apart when they finish a dense tile; these slots of theirs
+// are distinct shared-memory banks. The scan copy stores slots as ids
+// (IVF-CBICP keeps cluster ids).
+__host__ __device__ __forceinline__ int score_slot(int p) { return p ^ ((p >> 5) & 7); }
 
 struct DevCounters {
     unsigned long long changed;

@@ -712,7 +712,8 @@ __global__ void k_if_lens(int32_t D, const uint32_t *cnt2, int64_t *len, int64_t
     if (t < D) {
         const int64_t l = (int64_t)cnt2[2 * t] + (int64_t)cnt2[2 * t + 1];
         len[t] = l;
-        slen[t] = (l + 3) & ~(int64_t)3;  // scan copy: lists start at multiples of 4 entries
+        // scan copy: fronts and backs take whole quads of 4 entries
+        slen[t] = (((int64_t)cnt2[2 * t] + 3) & ~(int64_t)3) + (((int64_t)cnt2[2 * t + 1] + 3) & ~(int64_t)3);
         mf0[t] = (int32_t)cnt2[2 * t];
     }
 }
@@ -824,14 +825,32 @@ __global__ void k_dense_width(int32_t D, int32_t n_inst, const int32_t *inst_d, 
 }
 
 // What the assignment reads about a term, in one 16-byte load: where its list
-// starts in the scan copy, its front and list lengths, and its dense row.
+// starts in the scan copy, its front and list lengths, and its dense row. The
+// last quads of a sparse list's front and back are filled up with zero
+// postings here (they add 0 to a score).
 __global__ void k_term_desc(int32_t D, const int64_t *w8, const int64_t *base8, const int64_t *sc_off,
-                            const int32_t *mf0, const int64_t *len, int4 *tdesc, DevCounters *ctr) {
+                            const int32_t *mf0, const int64_t *len, int4 *tdesc, uint16_t *sc_id16, int32_t *sc_id32,
+                            float *sc_val, uint32_t *sc_pack, uint16_t *sc_lp, DevCounters *ctr) {
     long long n = 0;
+    auto fill = [&](int64_t from, int64_t to) {
+        for (int64_t p = from; p < to; ++p) {
+            if (sc_id16) sc_id16[p] = 0;
+            if (sc_id32) sc_id32[p] = 0;
+            if (sc_val) sc_val[p] = 0.0f;
+            if (sc_pack) sc_pack[p] = 0;
+            if (sc_lp) sc_lp[p] = 0;
+        }
+    };
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D; g += (int64_t)gridDim.x * blockDim.x) {
         const bool d = w8[g] > 0;
-        tdesc[g] = make_int4((int)sc_off[g], mf0[g], (int)len[g], d ? (int)base8[g] : -1);
+        const int64_t at = sc_off[g], f = mf0[g], l = len[g];
+        tdesc[g] = make_int4((int)(at >> 2), (int)f, (int)l, d ? (int)base8[g] : -1);
         n += d;
+        if (!d) {
+            const int64_t f4 = (f + 3) & ~(int64_t)3, b4 = (l - f + 3) & ~(int64_t)3;
+            fill(at + f, at + f4);
+            fill(at + f4 + (l - f), at + f4 + b4);
+        }
     }
     if (n) atomicAdd(reinterpret_cast<unsigned long long *>(&ctr->dense_terms), (unsigned long long)n);
 }
@@ -884,15 +903,17 @@ __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *ct
             continue;
         }
         const uint32_t part = (structured && lam[j]) ? 1u : 0u;
-        const int64_t pos = (int64_t)td.x + atomicAdd(cursor + (((uint32_t)t << 1) | part), 1u) + (part ? td.y : 0);
-        if (sc_id16) sc_id16[pos] = (uint16_t)p;
-        if (sc_id32) sc_id32[pos] = (int32_t)p;
+        const int64_t pos = (int64_t)(unsigned)td.x * 4 + atomicAdd(cursor + (((uint32_t)t << 1) | part), 1u) +
+                            (part ? (td.y + 3) & ~3 : 0);
+        const uint32_t id = structured ? (uint32_t)score_slot((int)p) : p;  // IVF-CBICP keeps cluster ids
+        if (sc_id16) sc_id16[pos] = (uint16_t)id;
+        if (sc_id32) sc_id32[pos] = (int32_t)id;
         if (prec == SIVF_FP32) {
             sc_val[pos] = u;
             continue;
         }
         const uint16_t lp = encode_lp(u, prec);
-        if (sc_pack) sc_pack[pos] = (p << 16) | (uint32_t)lp;
+        if (sc_pack) sc_pack[pos] = (id << 16) | (uint32_t)lp;
         else sc_lp[pos] = lp;
     }
 }
@@ -1038,7 +1059,8 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     SIVF_CUDA_TRY(scan_exclusive_i64(slen, slen, D, total + 1, ws, s));
     SIVF_CUDA_TRY(scan_exclusive_i64(w8, base8, D, total + 2, ws, s));
     SIVF_CUDA_TRY(cudaMemsetAsync(&c->ctr->dense_terms, 0, sizeof(long long), s));
-    k_term_desc<<<blocks_gs(D), TPB, 0, s>>>(D, w8, base8, slen, c->if_mf0, len, c->tdesc, c->ctr);
+    k_term_desc<<<blocks_gs(D), TPB, 0, s>>>(D, w8, base8, slen, c->if_mf0, len, c->tdesc, c->sc_id16, c->sc_id32,
+                                              c->sc_val, c->sc_pack, c->sc_lp, c->ctr);
     note_launch();
     if (dense) {
         const int esize = c->cfg.prec == SIVF_FP32 ? 4 : 2;

@@ -75,3 +75,15 @@ def test_contexts_of_different_k_take_turns():
             a.close()
             b.close()
     assert all(np.array_equal(x, y) for x, y in zip(runs[False], runs[True]))
+
+
+@pytest.mark.parametrize("threads", [32, 64, 128, 256, 512])
+@pytest.mark.parametrize("precision", ["fp32", "bf16", "fp16"])
+@pytest.mark.parametrize("buf", ["shared", "global"])
+def test_every_kernel_form(threads, precision, buf):
+    """All block sizes, precisions and score buffers, with and without dense
+    rows, over numbers of clusters that leave warps without tiles or rows."""
+    for k, frac in ((3, 1.0), (40, 0.05), (300, 1.0), (300, 0.05)):
+        c = _corpus_with_empty_rows(700, 1_500, 40 + k)
+        lockstep(c, k, _seeds(c, k, 9), 3, precision=precision, threads=threads, score_buffer=buf,
+                 dense_min_fraction=frac)

@@ -52,7 +52,7 @@ void free_all(sivf_ctx *c) {
                     c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->if_cid, c->if_val, c->tdesc, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
                     c->ctr, c->obj_dev, c->ws.base, c->inst_obj, c->inst_k, c->mov_beg, c->clu_koff,
                     c->inst_changed, c->own_row_ptr, c->own_idx, c->own_val, c->clu_doff,
-                    c->loop_dev, c->done_dev, c->objf_dev, c->grho, c->acc, c->acc_off, c->acc_lab,
+                    c->loop_dev, c->done_dev, c->objf_dev, c->grho, c->acc, c->acc_off, c->acc_lab, c->acc_bits, c->acc_bit_off,
                     c->clu_pos, c->pos_clu, c->dense_val, c->inst_d, c->dense_thr,
                     c->heavy_ids, c->light_ids};
     for (void *p : ptrs)
@@ -352,6 +352,29 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
         c->ws_bytes = ws;
         INIT_CUDA(dmalloc(c, reinterpret_cast<char **>(&c->ws.base), ws), "alloc workspace");
         c->ws.cap = ws;
+    }
+    if (c->dense && nnz * 16 / 3 <= c->acc_total) {
+        // The accumulator's occupancy map: where rows are mostly empty (the
+        // line of through_map in update.cu for the average cluster; with
+        // fuller rows its upkeep costs 10 % of the scatter for nothing). It is
+        // allocated last and only where the memory cap has room for it: a
+        // context that fitted without it still does.
+        std::vector<int64_t> boff((size_t)k + 1, 0);
+        for (int32_t m = 0; m < ni; ++m)
+            for (int32_t j = inst_k[(size_t)m]; j < inst_k[(size_t)m + 1]; ++j)
+                boff[(size_t)j + 1] = boff[(size_t)j] + (inst_d[(size_t)m + 1] - inst_d[(size_t)m] + 1 + 31) / 32;
+        c->acc_words = boff[(size_t)k];
+        if (dmalloc(c, &c->acc_bits, (size_t)c->acc_words) != cudaSuccess ||
+            dmalloc(c, &c->acc_bit_off, (size_t)k + 1) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(c->acc_bits);
+            c->acc_bits = nullptr;
+            c->acc_bit_off = nullptr;
+        } else {
+            INIT_CUDA(cudaMemcpyAsync(c->acc_bit_off, boff.data(), sizeof(int64_t) * ((size_t)k + 1),
+                                      cudaMemcpyHostToDevice, c->stream), "copy");
+            INIT_CUDA(cudaStreamSynchronize(c->stream), "sync");
+        }
     }
     for (auto &ev : c->ev) INIT_CUDA(cudaEventCreate(&ev), "event");
     {

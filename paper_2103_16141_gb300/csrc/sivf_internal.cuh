@@ -43,7 +43,8 @@
 //   update accumulator    acc int64 (dense form): one row of the instance's D terms per
 //                                        cluster (acc_off), the fixed-point sums
 //                                        q(x) = ceil(x 2^shift) of the current members,
-//                                        kept across iterations
+//                                        kept across iterations; acc_bits: a bit per entry
+//                                        that may be non-zero (1/64 of acc)
 //   object lists          heavy_ids, light_ids int32[N]: the objects of the CTA and the
 //                                        warp-per-object assignment kernels
 #pragma once
@@ -191,6 +192,14 @@ struct sivf_ctx {
     int64_t *acc_off = nullptr;
     int32_t *acc_lab = nullptr;
     int64_t acc_total = 0;  // entries of acc
+    // occupancy map of acc: a bit per entry, set where an entry may be
+    // non-zero; cluster j's words are [acc_bit_off[j], acc_bit_off[j + 1]).
+    // Null where rows are full enough to be read whole, or the memory cap
+    // leaves no room for it.
+    uint32_t *acc_bits = nullptr;
+    int64_t *acc_bit_off = nullptr;
+    int64_t acc_words = 0;
+    bool acc_ready = false;  // acc and acc_bits have been zeroed once
     int acc_shift = 0;
 
     // counters and step scratch

@@ -473,10 +473,12 @@ __global__ void k_label_counts(int64_t N, const int32_t *labels, int64_t *cnt) {
 }
 
 // One warp per object whose label changed since it was last added: its q
-// values move from the old cluster's row to the new one's.
+// values move from the old cluster's row to the new one's, and every entry
+// added to has its bit set in the occupancy map (bits, 32 entries per word;
+// null: no map).
 __global__ void k_acc_scatter(int64_t N, const int32_t *labels, int32_t *acc_lab, const int64_t *row_ptr,
                               const int32_t *idx, const float *val, const int32_t *clu_doff, const int64_t *acc_off,
-                              float fscale, int64_t *acc, int64_t *moved) {
+                              float fscale, int64_t *acc, uint32_t *bits, const int64_t *bit_off, int64_t *moved) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     long long mv = 0;
@@ -484,19 +486,54 @@ __global__ void k_acc_scatter(int64_t N, const int32_t *labels, int32_t *acc_lab
         const int32_t jn = labels[i], jo = acc_lab[i];
         if (jn == jo) continue;
         const int64_t rb = row_ptr[i], re = row_ptr[i + 1];
-        unsigned long long *rn = reinterpret_cast<unsigned long long *>(acc + acc_off[jn] - clu_doff[jn]);
+        const int32_t dn = clu_doff[jn];
+        unsigned long long *rn = reinterpret_cast<unsigned long long *>(acc + acc_off[jn] - dn);
+        uint32_t *bn = bits ? bits + bit_off[jn] : nullptr;
         unsigned long long *ro =
             jo >= 0 ? reinterpret_cast<unsigned long long *>(acc + acc_off[jo] - clu_doff[jo]) : nullptr;
         for (int64_t h = rb + lane; h < re; h += 32) {
             const unsigned long long q = (unsigned long long)__float2ll_ru(val[h] * fscale);
-            atomicAdd(rn + idx[h], q);
-            if (ro) atomicAdd(ro + idx[h], 0ull - q);  // two's complement: subtracts q
+            const int32_t t = idx[h];
+            atomicAdd(rn + t, q);
+            if (ro) atomicAdd(ro + t, 0ull - q);  // two's complement: subtracts q
+            const uint32_t bit = 1u << ((t - dn) & 31);
+            if (bn && !(bn[(t - dn) >> 5] & bit)) atomicOr(bn + ((t - dn) >> 5), bit);
         }
         mv += (re - rb) * (jo >= 0 ? 2 : 1);
         __syncwarp();
         if (lane == 0) acc_lab[i] = jn;
     }
     if (lane == 0 && mv) atomicAdd(reinterpret_cast<unsigned long long *>(moved), (unsigned long long)mv);
+}
+
+// Empties the accumulator through its occupancy map, one CTA per cluster:
+// only the entries that a member has touched (0.6 % of them at k = 20,000
+// over 140,000 terms) are written.
+__global__ void k_acc_clear(int32_t k, const int64_t *acc_off, const int64_t *bit_off, int64_t *acc, uint32_t *bits) {
+    for (int j = blockIdx.x; j < k; j += gridDim.x) {
+        const int64_t wb = bit_off[j], nw = bit_off[j + 1] - wb;
+        int64_t *row = acc + acc_off[j];
+        for (int64_t w = threadIdx.x; w < nw; w += blockDim.x) {
+            uint32_t b = bits[wb + w];
+            if (!b) continue;
+            bits[wb + w] = 0;
+            for (; b; b &= b - 1) row[32 * w + __ffs(b) - 1] = 0;
+        }
+    }
+}
+
+// Whether row j's accumulator entries are read through the occupancy map: the
+// row passes below read 16 bytes per lane in sequence otherwise, which is
+// cheaper once a word of the map (32 entries, eight sectors) has a few bits.
+// Measured per update, whole rows / through the map: k = 20,000 over 140,000
+// terms (0.6 % of the entries non-zero) 6.8 / 2.4 ms, k = 10,000 (1 %) 3.8 /
+// 1.8, k = 3001 over 61,000 (2 %) 0.52 / 0.41, k = 1000 over 100,000 (17 %)
+// 1.72 / 2.0 (before the passes kept 8 CTAs on an SM). The line is at 1/16, by
+// the length of the previous row, or by a third of the members' entries
+// (avg_len each) where the row has grown.
+__device__ __forceinline__ bool through_map(const uint32_t *bits, int64_t old_len, int64_t members, int64_t avg_len,
+                                            int64_t L) {
+    return bits && max(old_len, members * avg_len / 3) * 16 <= L;
 }
 
 __device__ __forceinline__ long long block_sum_ll(long long x, long long *sh) {
@@ -533,12 +570,14 @@ __device__ __forceinline__ void block_sum_u128(unsigned long long &hi, unsigned 
 
 // Pass 1, one CTA per cluster: size of the new row, ||s_j|| (the squared
 // integer sums added exactly in 128 bits, one rounding to FP64) and
-// <s_j, mu_j^[r-1]> in FP64 over the previous row.
+// <s_j, mu_j^[r-1]> in FP64 over the previous row. Where the row is read through
+// its map, the bits of entries that became zero are cleared.
 // Other clusters keep their row (sizes and objective pieces as in k_write_rows).
-__global__ void __launch_bounds__(WR_THREADS) k_acc_rows1(
+__global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     int32_t k, const int64_t *flag, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
-    const int64_t *acc, double inv_scale, const int64_t *coff_old, const int32_t *cterm_old, const float *cval_old,
-    const double *snorm_old, int64_t *sz, double *snorm_new, double *jA, double *jU) {
+    const int64_t *acc, uint32_t *bits, const int64_t *bit_off, int64_t avg_len, double inv_scale,
+    const int64_t *coff_old, const int32_t *cterm_old, const float *cval_old, const double *snorm_old, int64_t *sz, double *snorm_new,
+    double *jA, double *jU) {
     __shared__ double sh[WR_THREADS];
     __shared__ long long shl[WR_THREADS];
     __shared__ unsigned long long sh128[2][WR_THREADS];
@@ -563,10 +602,6 @@ __global__ void __launch_bounds__(WR_THREADS) k_acc_rows1(
     // and ||S|| = ||s_j|| 2^shift <= |C_j| 2^shift < 2^63, so the sum of
     // squares stays below 2^126.
     unsigned long long ss_hi = 0ull, ss_lo = 0ull;
-    // rows start at even entries and have even lengths: 16-byte loads, two
-    // of them in flight per thread
-    const longlong2 *row = reinterpret_cast<const longlong2 *>(acc + base);
-    const int64_t L2 = L >> 1;
     auto take = [&](long long v) {
         if (v) {
             ++nz;
@@ -576,13 +611,40 @@ __global__ void __launch_bounds__(WR_THREADS) k_acc_rows1(
             ss_hi += __umul64hi(u, u) + (ss_lo < lo ? 1ull : 0ull);
         }
     };
-    for (int64_t p = threadIdx.x; p < L2; p += 2 * WR_THREADS) {
-        const longlong2 a = row[p];
-        const longlong2 b = p + WR_THREADS < L2 ? row[p + WR_THREADS] : make_longlong2(0, 0);
-        take(a.x);
-        take(a.y);
-        take(b.x);
-        take(b.y);
+    if (through_map(bits, ce - cb, cnt[j], avg_len, L)) {
+        uint32_t *map = bits + bit_off[j];
+        const int64_t nw = (L + 31) >> 5;
+        for (int64_t w = threadIdx.x; w < nw; w += WR_THREADS) {
+            const uint32_t all = map[w];
+            uint32_t keep = all;
+            const int64_t *e = acc + base + 32 * w;
+            for (uint32_t b = all; b;) {  // two entries in flight
+                const uint32_t b0 = b & (0u - b);
+                b ^= b0;
+                const uint32_t b1 = b & (0u - b);
+                b ^= b1;
+                const long long v0 = e[__ffs(b0) - 1];
+                const long long v1 = b1 ? e[__ffs(b1) - 1] : 0;
+                take(v0);
+                take(v1);
+                if (!v0) keep ^= b0;
+                if (!v1) keep &= ~b1;
+            }
+            if (keep != all) map[w] = keep;
+        }
+    } else {
+        // rows start at even entries and have even lengths: 16-byte loads, two
+        // of them in flight per thread
+        const longlong2 *row = reinterpret_cast<const longlong2 *>(acc + base);
+        const int64_t L2 = L >> 1;
+        for (int64_t p = threadIdx.x; p < L2; p += 2 * WR_THREADS) {
+            const longlong2 a = row[p];
+            const longlong2 b = p + WR_THREADS < L2 ? row[p + WR_THREADS] : make_longlong2(0, 0);
+            take(a.x);
+            take(a.y);
+            take(b.x);
+            take(b.y);
+        }
     }
     nz = block_sum_ll(nz, shl);
     block_sum_u128(ss_hi, ss_lo, sh128);
@@ -602,24 +664,24 @@ __global__ void __launch_bounds__(WR_THREADS) k_acc_rows1(
 }
 
 // Pass 2, one CTA per cluster: the new row in ascending term order (block
-// compaction of the non-zero entries) and u = s * (2^-shift / ||s||) as FP32.
-// Other clusters copy their row.
-__global__ void __launch_bounds__(WR_THREADS) k_acc_rows2(
-    int32_t k, const int64_t *flag, const int64_t *acc_off, const int32_t *clu_doff, const int64_t *acc,
-    double inv_scale, const int64_t *coff_old, const int32_t *cterm_old, const float *cval_old,
-    const double *snorm_new, const int64_t *coff_new, int32_t *cterm_new, float *cval_new, int32_t *cclu_new,
-    int64_t cap, unsigned long long *error) {
-    constexpr int PER = 2;  // sub-chunks of WR_THREADS entry pairs per chunk
+// compaction of the non-zero entries) and
+// u = s * (2^-shift / ||s||) as FP32. Other clusters copy their row.
+__global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows2(
+    int32_t k, const int64_t *flag, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
+    const int64_t *acc, const uint32_t *bits, const int64_t *bit_off, int64_t avg_len, double inv_scale, const int64_t *coff_old, const int32_t *cterm_old,
+    const float *cval_old, const double *snorm_new, const int64_t *coff_new, int32_t *cterm_new, float *cval_new,
+    int32_t *cclu_new, int64_t cap, unsigned long long *error) {
+    constexpr int PER = 2;  // whole rows: sub-chunks of WR_THREADS entry pairs per chunk
     constexpr int NWR = WR_THREADS / 32;
     __shared__ int warp_n[PER][NWR];
     const int j = blockIdx.x;
     if (j >= k) return;
     const bool over = coff_new[k] > cap;  // more entries than the buffers hold: write nothing, report
     if (over && j == 0 && threadIdx.x == 0) atomicOr(error, 1ull);
+    if (over) return;
     const int64_t o0 = coff_new[j];
+    const int64_t cb = coff_old[j], ce = coff_old[j + 1];
     if (!flag[j]) {
-        if (over) return;
-        const int64_t cb = coff_old[j], ce = coff_old[j + 1];
         for (int64_t q = cb + threadIdx.x; q < ce; q += WR_THREADS) {
             cterm_new[o0 + (q - cb)] = cterm_old[q];
             cval_new[o0 + (q - cb)] = cval_old[q];
@@ -627,8 +689,7 @@ __global__ void __launch_bounds__(WR_THREADS) k_acc_rows2(
         }
         return;
     }
-    const int64_t base = acc_off[j], L2 = (acc_off[j + 1] - base) >> 1;  // entry pairs (even rows)
-    const longlong2 *row = reinterpret_cast<const longlong2 *>(acc + base);
+    const int64_t base = acc_off[j], L = acc_off[j + 1] - base;
     const int32_t doff = clu_doff[j];
     // u = S * (2^-shift / ||s_j||) in FP32 from the integer sum S (split in
     // 32-bit halves, each converted with one rounding): at most 4 roundings,
@@ -641,6 +702,43 @@ __global__ void __launch_bounds__(WR_THREADS) k_acc_rows2(
     };
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t o = o0;
+    if (through_map(bits, ce - cb, cnt[j], avg_len, L)) {  // as pass 1 decided, which left the bits of the non-zero entries
+        const uint32_t *map = bits + bit_off[j];
+        const int64_t nw = (L + 31) >> 5;
+        int turn = 0;
+        for (int64_t w0 = 0; w0 < nw; w0 += WR_THREADS, turn ^= 1) {
+            const int64_t w = w0 + threadIdx.x;
+            uint32_t b = w < nw ? map[w] : 0u;
+            const int64_t *e = acc + base + 32 * w;
+            const int n = __popc(b);
+            int inc = n;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= d) inc += y;
+            }
+            if (lane == 31) warp_n[turn][warp] = inc;
+            __syncthreads();  // the counts of the turn before the last are rewritten only behind this
+            int pre = 0, total = 0;
+#pragma unroll
+            for (int v = 0; v < NWR; ++v) {
+                const int c = warp_n[turn][v];
+                if (v < warp) pre += c;
+                total += c;
+            }
+            int64_t pos = o + pre + (inc - n);
+            for (; b; b &= b - 1, ++pos) {
+                const int t = __ffs(b) - 1;
+                cterm_new[pos] = (int32_t)(32 * w + t) + doff;
+                cval_new[pos] = value(e[t]);
+                cclu_new[pos] = j;
+            }
+            o += total;
+        }
+        return;
+    }
+    const longlong2 *row = reinterpret_cast<const longlong2 *>(acc + base);
+    const int64_t L2 = L >> 1;  // entry pairs (even rows)
     for (int64_t c0 = 0; c0 < L2; c0 += (int64_t)WR_THREADS * PER) {
         // sub-chunk m holds pairs c0 + m*WR_THREADS + tid (coalesced 16-byte loads);
         // entries keep their order: pair by pair, and x before y inside a pair
@@ -679,11 +777,9 @@ __global__ void __launch_bounds__(WR_THREADS) k_acc_rows2(
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 if (!pv[e]) continue;
-                if (!over) {
-                    cterm_new[pos] = (int32_t)(t + e) + doff;
-                    cval_new[pos] = value(pv[e]);
-                    cclu_new[pos] = j;
-                }
+                cterm_new[pos] = (int32_t)(t + e) + doff;
+                cval_new[pos] = value(pv[e]);
+                cclu_new[pos] = j;
                 ++pos;
             }
         }
@@ -992,7 +1088,17 @@ cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev) {
     SIVF_CUDA_TRY(cudaMemsetAsync(c->moving, 1, k, c->stream));
     SIVF_CUDA_TRY(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), c->stream));
     if (c->dense) {  // no member has been added yet
-        SIVF_CUDA_TRY(cudaMemsetAsync(c->acc, 0, sizeof(int64_t) * (size_t)c->acc_total, c->stream));
+        if (c->acc_bits && c->acc_ready) {
+            k_acc_clear<<<(unsigned)std::min<int32_t>(k, 65535), TPB, 0, c->stream>>>(k, c->acc_off, c->acc_bit_off,
+                                                                                     c->acc, c->acc_bits);
+            note_launch();
+            SIVF_CUDA_TRY(cudaGetLastError());
+        } else {
+            SIVF_CUDA_TRY(cudaMemsetAsync(c->acc, 0, sizeof(int64_t) * (size_t)c->acc_total, c->stream));
+            if (c->acc_bits)
+                SIVF_CUDA_TRY(cudaMemsetAsync(c->acc_bits, 0, sizeof(uint32_t) * (size_t)c->acc_words, c->stream));
+            c->acc_ready = true;
+        }
         SIVF_CUDA_TRY(cudaMemsetAsync(c->acc_lab, 0xFF, sizeof(int32_t) * N, c->stream));
     }
     c->iter = 1;  // finalize below marks every cluster moving
@@ -1133,17 +1239,19 @@ cudaError_t run_update_dense(sivf_ctx *c) {
     k_recompute_flags<<<blocks_for(k), TPB, 0, s>>>(k, c->lam, cnt, flag);
     const float fscale = ldexpf(1.0f, c->acc_shift);
     const double inv_scale = ldexp(1.0, -c->acc_shift);
+    const int64_t avg_len = c->nnz / N + 1;  // entries of an object
     k_acc_scatter<<<blocks_gs(N * 32), TPB, 0, s>>>(N, c->labels, c->acc_lab, c->row_ptr, c->idx, c->val,
-                                                     c->clu_doff, c->acc_off, fscale, c->acc, moved_d);
-    k_acc_rows1<<<(unsigned)k, WR_THREADS, 0, s>>>(k, flag, cnt, c->acc_off, c->clu_doff, c->acc, inv_scale,
-                                                   c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm, sz,
+                                                     c->clu_doff, c->acc_off, fscale, c->acc, c->acc_bits,
+                                                     c->acc_bit_off, moved_d);
+    k_acc_rows1<<<(unsigned)k, WR_THREADS, 0, s>>>(k, flag, cnt, c->acc_off, c->clu_doff, c->acc, c->acc_bits,
+                                                   c->acc_bit_off, avg_len, inv_scale, c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm, sz,
                                                    c->snorm_new, jAd, jUd);
     note_launch(4);
     SIVF_CUDA_TRY(cudaGetLastError());
     SIVF_CUDA_TRY(scan_exclusive_i64(sz, c->coff[nw], k, newn_d, ws, s));
     SIVF_CUDA_TRY(cudaMemcpyAsync(c->coff[nw] + k, newn_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    k_acc_rows2<<<(unsigned)k, WR_THREADS, 0, s>>>(k, flag, c->acc_off, c->clu_doff, c->acc, inv_scale, c->coff[cur],
-                                                   c->cterm[cur], c->cval[cur], c->snorm_new, c->coff[nw],
+    k_acc_rows2<<<(unsigned)k, WR_THREADS, 0, s>>>(k, flag, cnt, c->acc_off, c->clu_doff, c->acc, c->acc_bits,
+                                                   c->acc_bit_off, avg_len, inv_scale, c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm_new, c->coff[nw],
                                                    c->cterm[nw], c->cval[nw], c->cclu, c->cap_c, &c->ctr->error);
     k_sum_inst<<<(unsigned)c->n_inst, 1024, 0, s>>>(c->inst_k, jAd, jUd, c->obj_dev);
     k_copy_back<<<blocks_gs(c->cap_c), TPB, 0, s>>>(k, c->cap_c, c->coff[nw], c->cterm[nw], c->cval[nw],

@@ -106,74 +106,6 @@ struct AssignParams {
     unsigned long long *inst_changed;
 };
 
-// (value, index) ordering: larger value first, then lower index.
-struct Top2 {
-    uint32_t bv;
-    int32_t bi;       // INT32_MAX = none
-    long long sv;     // -1 = none
-};
-
-__device__ __forceinline__ void top2_push(Top2 &t, uint32_t v, int32_t j) {
-    if (t.bi == INT32_MAX || v > t.bv || (v == t.bv && j < t.bi)) {
-        if (t.bi != INT32_MAX) t.sv = max(t.sv, (long long)t.bv);
-        t.bv = v;
-        t.bi = j;
-    } else {
-        t.sv = max(t.sv, (long long)v);
-    }
-}
-
-__device__ __forceinline__ Top2 top2_merge(Top2 a, Top2 b) {
-    Top2 r;
-    bool a_wins = a.bi != INT32_MAX && (b.bi == INT32_MAX || a.bv > b.bv || (a.bv == b.bv && a.bi < b.bi));
-    Top2 w = a_wins ? a : b, l = a_wins ? b : a;
-    r.bv = w.bv;
-    r.bi = w.bi;
-    r.sv = max(w.sv, l.sv);
-    if (l.bi != INT32_MAX) r.sv = max(r.sv, (long long)l.bv);
-    return r;
-}
-
-// One thread's running top-2 over score positions: the best score with its
-// position (-1: none) and the second score. A cluster id is looked up only
-// when two scores tie (lowest id wins), and once for the winner at the end,
-// instead of at every new best: those lookups are dependent global loads.
-struct PosTop2 {
-    uint32_t bv;
-    int bp;
-    long long sv;
-};
-
-template <typename IdAt>
-__device__ __forceinline__ void pos_push(PosTop2 &t, uint32_t v, int p, const IdAt &id_at) {
-    if (t.bp < 0 || v > t.bv) {
-        if (t.bp >= 0) t.sv = max(t.sv, (long long)t.bv);
-        t.bv = v;
-        t.bp = p;
-    } else {
-        t.sv = max(t.sv, (long long)v);
-        if (v == t.bv && id_at(p) < id_at(t.bp)) t.bp = p;
-    }
-}
-
-// the same top-2 as top2_push over the same scores, with the winner's id
-template <typename IdAt>
-__device__ __forceinline__ Top2 pos_top2(const PosTop2 &t, const IdAt &id_at) {
-    Top2 r;
-    r.bv = t.bv;
-    r.bi = t.bp >= 0 ? id_at(t.bp) : INT32_MAX;
-    r.sv = t.sv;
-    return r;
-}
-
-__device__ __forceinline__ Top2 top2_shfl(Top2 t, int o) {
-    Top2 r;
-    r.bv = __shfl_xor_sync(0xffffffffu, t.bv, o);
-    r.bi = __shfl_xor_sync(0xffffffffu, t.bi, o);
-    r.sv = __shfl_xor_sync(0xffffffffu, t.sv, o);
-    return r;
-}
-
 // FP64 dot product of object rows [rb, re) with centroid j's master row
 // (binary search of each object term in the centroid's ascending terms).
 // Fixed lane assignment plus a butterfly reduction: deterministic, and every
@@ -1051,16 +983,19 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
 // dense chain and every fixed-point add as that kernel does, so both compute
 // the same scores, labels and own scores.
 
-// 8 warps per CTA, 1,472 score slots each (the moving clusters' scores), so
-// that a CTA's static shared memory is 48 KB; 4 CTAs per SM. On the
+// 8 warps per CTA, 1,472 score slots each (the moving clusters' scores) and
+// room for 128 staged terms, so that 4 CTAs reside on an SM. On the
 // 8M x 140K, k = 20,000 corpus one warp per object beat one CTA per object
 // up to about 1,500 moving clusters (1,156: 553 vs 623 ms, 1,284: 623 vs
 // 648 ms per assignment) and lost above (1,802: 800 vs 726 ms).
 constexpr int LIGHT_WARPS = 8;
-constexpr int LIGHT_MAX = 1472;  // the largest moving count of a light object
+constexpr int LIGHT_MAX = 1472;   // the largest moving count of a light object
+constexpr int LIGHT_TERMS = 128;  // terms staged at once
+constexpr int LIGHT_SMEM = LIGHT_WARPS * (LIGHT_MAX * 4 + LIGHT_TERMS * 8);
 static_assert(LIGHT_MAX % 8 == 0, "vector accesses of a slice");
-static_assert(LIGHT_WARPS * (LIGHT_MAX * 4 + 32 * 8) <= 48 * 1024, "static shared memory of the light kernel");
+static_assert(4 * (LIGHT_SMEM + 1024) <= 228 * 1024, "four CTAs on an SM");
 
+// instance of object i: largest m with inst_obj[m] <= i
 __device__ __forceinline__ int instance_of(const AssignParams &P, int64_t i) {
     int lo = 0, hi = P.n_inst - 1;
     while (lo < hi) {
@@ -1104,152 +1039,219 @@ __global__ void k_classify(AssignParams P, int light_max, int32_t *heavy_ids, in
     }
 }
 
+// The dense terms of [s0, s0 + LIGHT_TERMS) of the object's row into dn, in
+// staging (term) order; returns their number. With `first`, the fronts of the
+// other terms are added to the scores and the postings counted. Fronts of 32
+// postings and more are added one after the other by the whole warp; shorter
+// ones are laid end to end, 32 postings at a time, a lane finding its front by
+// bisection over the lanes' prefix sums.
+template <int PREC, bool CID16>
+__device__ __forceinline__ int light_stage(const AssignParams &P, uint32_t *rho, int2 *dn, int s0, int ce, int lane,
+                                           bool first, unsigned long long &c_post, unsigned long long &c_dpost) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const unsigned below = (1u << lane) - 1u;
+    int nd = 0;
+    const int s1 = min(ce, s0 + LIGHT_TERMS);
+    for (int s = s0; s < s1; s += 32) {
+        const int h = s + lane;
+        int4 td = make_int4(0, 0, 0, -1);
+        float vs = 0.f;
+        if (h < s1) {
+            const int t = P.idx[h];
+            vs = P.val[h] * FIX_SCALE;
+            if (P.checked && (t < 0 || t >= P.D)) atomicOr(&P.ctr->error, 2ull);
+            else td = __ldg(P.tdesc + t);
+        }
+        const bool dense = td.w >= 0;
+        const unsigned m = __ballot_sync(FULL, dense);
+        if (dense) {
+            // FP16 rows hold u * 2^14 (exact)
+            dn[nd + __popc(m & below)] =
+                make_int2(td.w, __float_as_int(PREC == SIVF_FP16 ? vs * FP16_INV_SCALE : vs));
+        }
+        nd += __popc(m);
+        if (!first) continue;
+        c_post += (unsigned long long)td.y;
+        if (dense) c_dpost += (unsigned long long)td.y;
+        const int len = dense ? 0 : td.y;
+        unsigned big = __ballot_sync(FULL, len >= 32);
+        while (big) {
+            const int src = __ffs(big) - 1;
+            big &= big - 1;
+            const int L = __shfl_sync(FULL, len, src);
+            const size_t at = (size_t)(unsigned)__shfl_sync(FULL, td.x, src) * 4;
+            const float v = __shfl_sync(FULL, vs, src);
+            for (int o = lane; o < L; o += 32) {
+                int id;
+                float u;
+                load_one<PREC, CID16>(P, at + o, id, u);
+                atomicAdd(rho + id, __float2uint_ru(v * u));
+            }
+        }
+        const int small = len < 32 ? len : 0;
+        int incl = small;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int total = __shfl_sync(FULL, incl, 31);
+        for (int q0 = 0; q0 < total; q0 += 32) {
+            const int q = q0 + lane;
+            int src = 0;  // first lane whose prefix sum exceeds q
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(FULL, incl, src + step - 1) <= q) src += step;
+            src = min(src, 31);
+            const int o = q - __shfl_sync(FULL, incl - small, src);
+            const size_t at = (size_t)(unsigned)__shfl_sync(FULL, td.x, src) * 4;
+            const float v = __shfl_sync(FULL, vs, src);
+            if (q < total) {
+                int id;
+                float u;
+                load_one<PREC, CID16>(P, at + o, id, u);
+                atomicAdd(rho + id, __float2uint_ru(v * u));
+            }
+        }
+    }
+    __syncwarp();
+    return nd;
+}
+
+// One warp per object. The next object's entry of the list and its row bounds
+// are fetched behind the current object's work, so that of the chain of
+// dependent loads only the terms and their descriptors are waited for.
 template <int PREC, bool CID16>
 __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(AssignParams P) {
-    __shared__ __align__(16) uint32_t s_rho[LIGHT_WARPS][LIGHT_MAX];
-    __shared__ int2 s_dn[LIGHT_WARPS][32];
+    extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned FULL = 0xffffffffu, below = (1u << lane) - 1u;
-    uint32_t *rho = s_rho[w];
-    int2 *dn = s_dn[w];
-    // counters kept by lane 0: filtered, sim-calcs, changed, re-scored, candidates, dense entries
+    constexpr unsigned FULL = 0xffffffffu;
+    uint32_t *rho = smem + w * LIGHT_MAX;
+    int2 *dn = reinterpret_cast<int2 *>(smem + LIGHT_WARPS * LIGHT_MAX) + w * LIGHT_TERMS;
+    // counters kept by lane 0: filtered, sim-calcs, re-scored, candidates, dense entries; any lane: changed
     unsigned long long c_filt = 0, c_sim = 0, c_chg = 0, c_resc = 0, c_cand = 0, c_dent = 0;
     unsigned long long c_post = 0, c_dpost = 0;  // every lane
-    const long long n_obj = (long long)P.ctr->n_light;
-    for (;;) {
-        long long li = 0;
-        if (lane == 0) li = (long long)atomicAdd(&P.ctr->work_light, 1ull);
-        li = __shfl_sync(FULL, li, 0);
-        if (li >= n_obj) break;
-        const int64_t i = P.light_ids[li];
-        int64_t rb = P.row_ptr[i], re = P.row_ptr[i + 1];
-        if (P.checked && (rb < 0 || re < rb || re > P.nnz)) {
+    const unsigned n_obj = P.ctr->n_light;
+    auto bounds = [&](int i, int &rb, int &re) {
+        int64_t b = P.row_ptr[i], e = P.row_ptr[i + 1];
+        if (P.checked && (b < 0 || e < b || e > P.nnz)) {
             if (lane == 0) atomicOr(&P.ctr->error, 1ull);
-            rb = re = 0;
+            b = e = 0;
         }
+        rb = (int)b;
+        re = (int)e;
+    };
+    unsigned li = 0;
+    if (lane == 0) li = atomicAdd(&P.ctr->work_light, 1u);
+    li = __shfl_sync(FULL, li, 0);
+    int i = li < n_obj ? P.light_ids[li] : -1;
+    int rb = 0, re = 0;
+    if (i >= 0) bounds(i, rb, re);
+    while (i >= 0) {
+        if (lane == 0) li = atomicAdd(&P.ctr->work_light, 1u);
+        const int32_t a_prev = P.labels_prev[i];
+        const uint32_t own_q = P.own[i];
         const int inst = instance_of(P, i);
         const int k_off = P.inst_k[inst];
         const int n_mov = P.mov_beg[inst + 1] - P.mov_beg[inst];
-        const int32_t a_prev = P.labels_prev[i];
         const int a_loc = a_prev - k_off;
-        const uint32_t own_q = P.own[i];
+        const int n_terms = re - rb;
         if (lane == 0) {
             ++c_filt;
             c_sim += (unsigned long long)n_mov;
         }
+        int i_next = -1;
         if (n_mov == 0) {  // the own cluster is the only candidate: label and own score stay
             if (lane == 0) P.labels[i] = a_prev;
-            continue;
-        }
-        for (int p = lane; p < ((n_mov + 7) & ~7); p += 32) rho[p] = 0u;
-        __syncwarp();
-        int nd_obj = 0;
-        for (int64_t cb = rb; cb < re; cb += P.chunk) {
-            const int64_t ce = min(re, cb + (int64_t)P.chunk);
-            // dense rows: the front (positions below n_mov) of each dense term of the chunk
-            for (int base = 0; base < n_mov; base += 256) {
-                const int p = PREC == SIVF_FP32 ? base + 4 * lane : base + 8 * lane;
-                constexpr int HALF = PREC == SIVF_FP32 ? 128 : 4;
-                const bool second = p + HALF < n_mov;
-                const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * (PREC == SIVF_FP32 ? 4 : 2);
-                float acc[8];
-#pragma unroll
-                for (int m = 0; m < 8; ++m) acc[m] = 0.f;
-                int nd_chunk = 0;
-                for (int64_t s0 = cb; s0 < ce; s0 += 32) {
-                    const int64_t h = s0 + lane;
-                    int2 e = make_int2(-1, 0);
-                    if (h < ce) {
-                        int t = P.idx[h];
-                        if (P.checked && (t < 0 || t >= P.D)) {
-                            atomicOr(&P.ctr->error, 2ull);
-                            t = -1;
-                        }
-                        const int dr = t >= 0 ? P.tdesc[t].w : -1;
-                        if (dr >= 0) {
-                            float vs = P.val[h] * FIX_SCALE;
-                            if constexpr (PREC == SIVF_FP16) vs *= FP16_INV_SCALE;
-                            e = make_int2(dr, __float_as_int(vs));
-                        }
-                    }
-                    const unsigned m = __ballot_sync(FULL, e.x >= 0);
-                    if (e.x >= 0) dn[__popc(m & below)] = e;
-                    __syncwarp();
-                    const int cnt = __popc(m);
-                    if (p < n_mov)
-                        for (int d = 0; d < cnt; ++d) {  // staging (term) order
-                            const int2 x = dn[d];
-                            fma_raw8<PREC>(load_raw8<PREC>(e0, x.x, HALF, second), __int_as_float(x.y), acc);
-                        }
-                    nd_chunk += cnt;
-                    __syncwarp();
-                }
-                if (p < n_mov) rho_put4<false>(rho, p, acc, false);  // LIGHT_MAX is a multiple of 8: stays in the slice
-                if (second) rho_put4<false>(rho, p + HALF, acc + 4, false);
-                if (base == 0) {
-                    nd_obj += nd_chunk;
-                    if (lane == 0) c_dent += (unsigned long long)nd_chunk * (unsigned long long)n_mov;
-                }
-            }
+        } else {
+            const int n8 = (n_mov + 7) & ~7;
+            for (int p = 4 * lane; p < n8; p += 128) rho_st4<false>(rho + p, make_uint4(0u, 0u, 0u, 0u));
             __syncwarp();
-            // sparse fronts of the chunk's other terms, one segment at a time, lane-strided
-            for (int64_t s0 = cb; s0 < ce; s0 += 32) {
-                const int64_t h = s0 + lane;
-                int len = 0, sb = 0;
-                float vs = 0.f;
-                if (h < ce) {
-                    int t = P.idx[h];
-                    if (P.checked && (t < 0 || t >= P.D)) t = -1;
-                    if (t >= 0) {
-                        const int4 td = __ldg(P.tdesc + t);
-                        len = td.y;
-                        c_post += (unsigned long long)len;
-                        if (td.w >= 0) {
-                            c_dpost += (unsigned long long)len;
-                            len = 0;
-                        } else {
-                            sb = td.x;
-                            vs = P.val[h] * FIX_SCALE;
-                        }
-                    }
-                }
-                unsigned m = __ballot_sync(FULL, len > 0);
-                while (m) {
-                    const int src = __ffs(m) - 1;
-                    m &= m - 1;
-                    const int L = __shfl_sync(FULL, len, src), b = __shfl_sync(FULL, sb, src);
-                    const float v = __shfl_sync(FULL, vs, src);
-                    for (int o = lane; o < L; o += 32) {
-                        int id;
-                        float u;
-                        load_one<PREC, CID16>(P, (size_t)(unsigned)b * 4 + o, id, u);
-                        atomicAdd(rho + id, __float2uint_ru(v * u));
-                    }
-                }
-            }
-            __syncwarp();
-        }
-        // argmax over the moving clusters plus the own cluster (carried score)
-        auto id_at = [&](int p) { return P.pos_clu[k_off + p]; };
-        PosTop2 pt;
-        pt.bv = 0u;
-        pt.bp = -1;
-        pt.sv = -1;
-        for (int p = lane; p < n_mov; p += 32) pos_push(pt, rho[score_slot(p)], p, id_at);
-        Top2 t = pos_top2(pt, id_at);
-        if (lane == 0) top2_push(t, own_q, a_loc);
+            for (int cb = rb; cb < re; cb += P.chunk) {
+                const int ce = min(re, cb + P.chunk);
+                // positions 256 at a time; a chunk of more terms than are staged
+                // at once is staged again for every 256
+                int nd = 0;
+                for (int base = 0; base < n_mov; base += 256) {
+                    constexpr int W = PREC == SIVF_FP32 ? 4 : 8, HALF = PREC == SIVF_FP32 ? 128 : 4;
+                    constexpr int U = PREC == SIVF_FP32 ? 2 : 4;
+                    const int p = base + W * lane;
+                    const bool in = p < n_mov, second = p + HALF < n_mov;
+                    const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * (PREC == SIVF_FP32 ? 4 : 2);
+                    float acc[8];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t = top2_merge(t, top2_shfl(t, o));
-        int winner = t.bi;
-        if (t.bv > 0u && t.sv >= 0) {
+                    for (int m = 0; m < 8; ++m) acc[m] = 0.f;
+                    for (int s0 = cb; s0 < ce; s0 += LIGHT_TERMS) {
+                        if (base == 0 || ce - cb > LIGHT_TERMS)
+                            nd = light_stage<PREC, CID16>(P, rho, dn, s0, ce, lane, base == 0, c_post, c_dpost);
+                        if (base == 0 && lane == 0) c_dent += (unsigned long long)nd * (unsigned long long)n_mov;
+                        if (in) {
+                            int d = 0;
+                            for (; d + U <= nd; d += U) {
+                                Raw8<PREC> r[U];
+                                float vs[U];
+#pragma unroll
+                                for (int q = 0; q < U; ++q) {
+                                    const int2 x = dn[d + q];
+                                    r[q] = load_raw8<PREC>(e0, x.x, HALF, second);
+                                    vs[q] = __int_as_float(x.y);
+                                }
+#pragma unroll
+                                for (int q = 0; q < U; ++q) fma_raw8<PREC>(r[q], vs[q], acc);
+                            }
+                            for (; d < nd; ++d) {
+                                const int2 x = dn[d];
+                                fma_raw8<PREC>(load_raw8<PREC>(e0, x.x, HALF, second), __int_as_float(x.y), acc);
+                            }
+                        }
+                        __syncwarp();
+                    }
+                    if (in) rho_put4<false>(rho, p, acc, false);  // LIGHT_MAX is a multiple of 8: stays in the slice
+                    if (second) rho_put4<false>(rho, p + HALF, acc + 4, false);
+                }
+                __syncwarp();
+            }
+            li = __shfl_sync(FULL, li, 0);
+            if (li < n_obj) i_next = P.light_ids[li];
+            // argmax over the moving clusters plus the own cluster (carried
+            // score), as in the CTA kernel
+            auto id_at = [&](int p) { return P.pos_clu[k_off + p]; };
+            uint32_t bv = 0u, sv = 0u;
+            for (int p = 4 * lane; (p & ~7) < n_mov; p += 128) {
+                const uint4 q = rho_ld4<false>(rho + p);
+                if (score_slot(p) < n_mov) top2_add(bv, sv, q.x);
+                if (score_slot(p + 1) < n_mov) top2_add(bv, sv, q.y);
+                if (score_slot(p + 2) < n_mov) top2_add(bv, sv, q.z);
+                if (score_slot(p + 3) < n_mov) top2_add(bv, sv, q.w);
+            }
+            const uint32_t mine = bv;
+            warp_top2(bv, sv);
+            const uint32_t top = bv;
+            top2_add(bv, sv, own_q);
             // the carried own score may come from a scan with other dense terms:
             // count every term as dense
-            const double best = (double)t.bv * FIX_QUANTUM;
-            const double E = error_bound(best, re - rb, (int)(re - rb), (double)P.sumv[i], P.eps, P.eta);
-            const double gap = (double)((long long)t.bv - t.sv) * FIX_QUANTUM;
-            if (gap <= 2.0 * E) {
+            bool flag = bv > 0u && !clear_of_bound(bv, bv - sv, n_terms, n_terms, P.eps_f,
+                                                   P.eta_q != 0.f ? P.eta_q * P.sumv[i] : 0.f);
+            uint32_t thr = 0;
+            if (flag) {  // warp-uniform: the exact form of the bound
+                const double E = error_bound((double)bv * FIX_QUANTUM, n_terms, n_terms, (double)P.sumv[i], P.eps,
+                                             P.eta);
+                flag = (double)(bv - sv) * FIX_QUANTUM <= 2.0 * E;
                 const double span = ceil(2.0 * E / FIX_QUANTUM);
-                const uint32_t thr = span >= (double)t.bv ? 0u : t.bv - (uint32_t)span;
+                thr = span >= (double)bv ? 0u : bv - (uint32_t)span;
+            }
+            auto finish = [&](int al, uint32_t q) {  // by the one lane that knows the label
+                const int a = k_off + al;
+                P.labels[i] = a;
+                P.own[i] = q;
+                if (a != a_prev) {
+                    ++c_chg;
+                    P.moving[a] = 1;
+                    P.moving[a_prev] = 1;
+                    if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
+                }
+            };
+            if (flag) {
                 double wbest = -1.0;
                 int wj = INT32_MAX, ncand = 0;
                 for (int base = 0; base < n_mov; base += 32) {
@@ -1276,30 +1278,43 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
                         wj = a_loc;
                     }
                 }
-                if (wj != INT32_MAX) winner = wj;
                 if (lane == 0) {
                     ++c_resc;
                     c_cand += (unsigned long long)ncand;
+                    finish(wj, wj == a_loc ? own_q : rho[score_slot(P.clu_pos[k_off + wj])]);
+                }
+            } else if (bv == 0u || own_q == bv) {
+                // all scores zero: the lowest id among the candidates; else the own
+                // cluster, which no scanned score reaches
+                if (lane == 0) finish(bv == 0u ? min(a_loc, id_at(0)) : a_loc, bv);
+            } else if (mine == top) {  // one lane: a second one would make the gap zero
+                for (int p = 4 * lane; (p & ~7) < n_mov; p += 128) {
+                    const uint4 q = rho_ld4<false>(rho + p);
+                    int e = -1;
+                    if (q.x == top && score_slot(p) < n_mov) e = score_slot(p);
+                    if (q.y == top && score_slot(p + 1) < n_mov) e = score_slot(p + 1);
+                    if (q.z == top && score_slot(p + 2) < n_mov) e = score_slot(p + 2);
+                    if (q.w == top && score_slot(p + 3) < n_mov) e = score_slot(p + 3);
+                    if (e >= 0) {
+                        finish(id_at(e), top);
+                        break;
+                    }
                 }
             }
+            __syncwarp();
         }
-        if (lane == 0) {
-            const int a = k_off + winner;
-            P.labels[i] = a;
-            P.own[i] = winner == a_loc ? own_q : rho[score_slot(P.clu_pos[a])];
-            if (a != a_prev) {
-                ++c_chg;
-                P.moving[a] = 1;
-                P.moving[a_prev] = 1;
-                if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
-            }
+        if (n_mov == 0) {
+            li = __shfl_sync(FULL, li, 0);
+            if (li < n_obj) i_next = P.light_ids[li];
         }
-        __syncwarp();
+        i = i_next;
+        if (i >= 0) bounds(i, rb, re);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         c_post += __shfl_xor_sync(FULL, c_post, o);
         c_dpost += __shfl_xor_sync(FULL, c_dpost, o);
+        c_chg += __shfl_xor_sync(FULL, c_chg, o);
     }
     if (lane == 0) {
         if (c_post) atomicAdd(&P.ctr->postings, c_post);
@@ -1411,8 +1426,12 @@ template <int PREC>
 cudaError_t launch_light(sivf_ctx *c, const AssignParams &P) {
     const bool ids16 = P.sc_id16 || P.sc_pack;
     const unsigned grid = (unsigned)c->num_sms * 4;  // one wave of resident CTAs
-    if (ids16) assign_light_kernel<PREC, true><<<grid, LIGHT_WARPS * 32, 0, c->stream>>>(P);
-    else assign_light_kernel<PREC, false><<<grid, LIGHT_WARPS * 32, 0, c->stream>>>(P);
+    auto kern = ids16 ? assign_light_kernel<PREC, true> : assign_light_kernel<PREC, false>;
+    if (!c->light_ready) {  // a host call that a stream capture refuses: made on the first, host-launched step
+        SIVF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LIGHT_SMEM));
+        c->light_ready = true;
+    }
+    kern<<<grid, LIGHT_WARPS * 32, LIGHT_SMEM, c->stream>>>(P);
     note_launch();
     return cudaGetLastError();
 }

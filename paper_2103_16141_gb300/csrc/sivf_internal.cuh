@@ -99,7 +99,7 @@ struct DevCounters {
     unsigned long long dense_postings;  // postings of the scanned segments held in dense rows
     long long dense_terms;              // terms with a dense row (last inverted-file build)
     long long dense_used;               // dense-row entries in use / 8 (last build)
-    unsigned long long work_light;   // object work counter of the light (warp-per-object) kernel
+    unsigned int work_light, pad;    // object work counter of the light (warp-per-object) kernel
     unsigned int n_heavy, n_light;   // objects in the two lists of the assignment
     long long sparse_entries;        // entries of the sparse scan copy (last build)
 };
@@ -214,6 +214,7 @@ struct sivf_ctx {
     int assign_threads = 0, assign_ctas_per_sm = 0;
     int64_t assign_grid = 0;  // cached launch grid of the assignment kernel (0 = not yet chosen)
     int assign_global = 0;    // 1: score vectors in global memory (grho), else shared memory
+    bool light_ready = false; // the warp-per-object kernel's shared memory has been set
     bool tuned = false;       // the autotuner has picked the assignment configuration
     uint32_t *grho = nullptr; // global score vectors: grho_ctas slabs of kmax (zero between objects)
     int64_t grho_ctas = 0;

@@ -58,7 +58,7 @@ void free_all(sivf_ctx *c) {
     for (void *p : ptrs)
         if (p) cudaFree(p);
     destroy_loop_graph(c);
-    void *pins[] = {c->ctr_host, c->inst_changed_pin, c->obj_pin, c->nmov_pin, c->loop_pin, c->objf_pin};
+    void *pins[] = {c->ctr_host, c->inst_changed_pin, c->obj_pin, c->loop_pin, c->objf_pin};
     for (void *p : pins)
         if (p) cudaFreeHost(p);
     for (auto &e : c->ev)
@@ -289,7 +289,6 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     INIT_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c->inst_changed_pin), sizeof(unsigned long long) * ni),
               "alloc host");
     INIT_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c->obj_pin), sizeof(double) * 2 * ni), "alloc host");
-    INIT_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c->nmov_pin), sizeof(int32_t)), "alloc host");
     INIT_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c->loop_pin), sizeof(int32_t) * (4 + (size_t)ni)), "alloc host");
     INIT_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c->objf_pin), sizeof(double) * ni), "alloc host");
     if (c->assign_global || c->cfg.autotune) {
@@ -629,24 +628,16 @@ namespace sivf {
 // pinned host mirrors; a graph body is captured without either.
 cudaError_t enqueue_assign(sivf_ctx *c, bool timing) {
     cudaStream_t s = c->stream;
-    // a^[r-1] <- a^[r], lambda^[r-1] <- lambda^[r] (copies keep every buffer
-    // address fixed from one iteration to the next)
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->labels_prev, c->labels, sizeof(int32_t) * c->N, cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->lam_prev, c->lam, c->k, cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), s));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->moving, 0, c->k, s));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->inst_changed, 0, sizeof(unsigned long long) * c->n_inst, s));
-    if (timing) {
-        SIVF_CUDA_TRY(cudaMemcpyAsync(c->nmov_pin, c->n_mov_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        SIVF_CUDA_TRY(cudaEventRecord(c->ev[0], s));
-    }
+    SIVF_CUDA_TRY(launch_begin_assign(c));
+    if (timing) SIVF_CUDA_TRY(cudaEventRecord(c->ev[0], s));
     SIVF_CUDA_TRY(launch_assign(c));
     SIVF_CUDA_TRY(launch_finalize_assign(c));
     if (timing) {
         SIVF_CUDA_TRY(cudaEventRecord(c->ev[1], s));
         SIVF_CUDA_TRY(cudaMemcpyAsync(c->ctr_host, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
-        SIVF_CUDA_TRY(cudaMemcpyAsync(c->inst_changed_pin, c->inst_changed, sizeof(unsigned long long) * c->n_inst,
-                                      cudaMemcpyDeviceToHost, s));
+        if (c->n_inst > 1)  // one instance: the counters hold its count
+            SIVF_CUDA_TRY(cudaMemcpyAsync(c->inst_changed_pin, c->inst_changed,
+                                          sizeof(unsigned long long) * c->n_inst, cudaMemcpyDeviceToHost, s));
     }
     return cudaSuccess;
 }
@@ -683,7 +674,7 @@ sivf_status finish_assign(sivf_ctx *c, int64_t *n_changed, float ms) {
     st.iter = c->iter;
     st.changed = (int64_t)h.changed;
     st.n_moving = (int64_t)h.n_moving;
-    st.n_moving_prev = *c->nmov_pin;
+    st.n_moving_prev = h.n_moving_prev;
     st.filtered = (int64_t)h.filtered;
     st.simcalc = (int64_t)h.simcalc;
     st.postings = (int64_t)h.postings;
@@ -758,7 +749,6 @@ sivf_status graph_loop(sivf_ctx *c, int32_t max_total, std::vector<int32_t> &don
     API_CUDA(c, cudaMemcpyAsync(lp, c->loop_dev, sizeof(int32_t) * 4, cudaMemcpyDeviceToHost, s), "copy");
     API_CUDA(c, cudaMemcpyAsync(lp + 4, c->done_dev, sizeof(int32_t) * ni, cudaMemcpyDeviceToHost, s), "copy");
     API_CUDA(c, cudaMemcpyAsync(c->objf_pin, c->objf_dev, sizeof(double) * ni, cudaMemcpyDeviceToHost, s), "copy");
-    API_CUDA(c, cudaMemcpyAsync(c->nmov_pin, c->n_mov_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy");
     API_CUDA(c, cudaMemcpyAsync(c->ctr_host, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s), "copy");
     API_CUDA(c, cudaMemcpyAsync(c->inst_changed_pin, c->inst_changed, sizeof(unsigned long long) * ni,
                                 cudaMemcpyDeviceToHost, s), "copy");

@@ -1005,6 +1005,30 @@ __device__ __forceinline__ int instance_of(const AssignParams &P, int64_t i) {
     return lo;
 }
 
+// Start of a step: a^[r-1] <- a^[r], lambda^[r-1] <- lambda^[r] (copies keep
+// every buffer address fixed from one iteration to the next), the moving flags
+// and the counters cleared; the moving count of lambda^[r-1] is kept beside
+// the counters. One launch instead of five copies and fills.
+__global__ void k_begin(int64_t N, int32_t k, int32_t n_inst, const int32_t *labels, int32_t *labels_prev,
+                        const uint8_t *lam, uint8_t *lam_prev, uint8_t *moving, unsigned long long *inst_changed,
+                        const int32_t *n_mov, DevCounters *ctr) {
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+    const int4 *from = reinterpret_cast<const int4 *>(labels);
+    int4 *to = reinterpret_cast<int4 *>(labels_prev);
+    for (int64_t q = g; q < N >> 2; q += st) to[q] = from[q];
+    for (int64_t i = (N & ~(int64_t)3) + g; i < N; i += st) labels_prev[i] = labels[i];
+    for (int64_t j = g; j < k; j += st) {
+        lam_prev[j] = lam[j];
+        moving[j] = 0;
+    }
+    for (int64_t m = g; m < n_inst; m += st) inst_changed[m] = 0ull;
+    if (g == 0) {
+        DevCounters z = {};
+        z.n_moving_prev = (long long)*n_mov;
+        *ctr = z;
+    }
+}
+
 // Objects into the two lists: filtered objects of an instance with at most
 // light_max moving clusters to the light list, every other object to the
 // heavy list (warp-aggregated appends; the order inside a list changes no
@@ -1437,6 +1461,15 @@ cudaError_t launch_light(sivf_ctx *c, const AssignParams &P) {
 }
 
 }  // namespace
+
+cudaError_t launch_begin_assign(sivf_ctx *c) {
+    const unsigned blocks = (unsigned)std::min<int64_t>((std::max(c->N / 4, (int64_t)c->k) + 255) / 256 + 1,
+                                                        (int64_t)c->num_sms * 8);
+    k_begin<<<blocks, 256, 0, c->stream>>>(c->N, c->k, c->n_inst, c->labels, c->labels_prev, c->lam, c->lam_prev,
+                                           c->moving, c->inst_changed, c->n_mov_dev, c->ctr);
+    note_launch();
+    return cudaGetLastError();
+}
 
 cudaError_t launch_assign(sivf_ctx *c) {
     AssignParams P;

@@ -102,6 +102,7 @@ struct DevCounters {
     unsigned int work_light, pad;    // object work counter of the light (warp-per-object) kernel
     unsigned int n_heavy, n_light;   // objects in the two lists of the assignment
     long long sparse_entries;        // entries of the sparse scan copy (last build)
+    long long n_moving_prev;         // lambda^[r-1] = 0 count (written when the step begins)
 };
 
 // Bump allocator over one device block (scratch that lives for one step).
@@ -244,7 +245,6 @@ struct sivf_ctx {
     // pinned host mirrors (read after a stream synchronisation)
     unsigned long long *inst_changed_pin = nullptr;  // [n_inst]
     double *obj_pin = nullptr;                      // [2 * n_inst]
-    int32_t *nmov_pin = nullptr;                    // [1] moving count before the assignment
     // device-side Lloyd loop (use_graph): WHILE conditional node around one iteration
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
@@ -285,6 +285,7 @@ cudaError_t scan_exclusive_u32_dev(const uint32_t *in, uint32_t *out, int64_t nm
 int bits_for(uint64_t max_value);  // number of bits to hold values in [0, max_value]
 
 // ---- assign.cu ----
+cudaError_t launch_begin_assign(sivf_ctx *c);
 cudaError_t launch_assign(sivf_ctx *c);
 cudaError_t launch_finalize_assign(sivf_ctx *c);
 cudaError_t autotune_assign(sivf_ctx *c);

@@ -412,12 +412,48 @@ __global__ void __launch_bounds__(WR_THREADS) k_write_rows(
     }
 }
 
-// Copy the new rows back over the current ones (fixed buffers for graph replay).
-__global__ void k_copy_back(int32_t k, int64_t cap, const int64_t *coff_src, const int32_t *term_src,
-                            const float *val_src, const double *sn_src, int64_t *coff_dst, int32_t *term_dst,
-                            float *val_dst, double *sn_dst) {
+// Last kernel of the centroid step. Blocks below n_inst: the objective sums of
+// an instance, in a fixed order (per-thread strided partial sums, then a
+// tree). The others copy the new rows back over the current ones (fixed
+// buffers for graph replay). Block 0 leaves the step's counts.
+__global__ void __launch_bounds__(1024) k_finish_rows(int32_t k, int64_t cap, int32_t n_inst, const int32_t *inst_k,
+                                                      const double *jA, const double *jU, double *out,
+                                                      const int64_t *coff_src, const int32_t *term_src,
+                                                      const float *val_src, const double *sn_src, int64_t *coff_dst,
+                                                      int32_t *term_dst, float *val_dst, double *sn_dst,
+                                                      const int64_t *moved, DevCounters *ctr) {
+    if ((int)blockIdx.x < n_inst) {
+        __shared__ double sa[1024], sb[1024];
+        const int m = blockIdx.x;
+        const int j0 = inst_k[m], j1 = inst_k[m + 1];
+        double x = 0.0, y = 0.0;
+        for (int j = j0 + threadIdx.x; j < j1; j += 1024) {
+            x += jA[j];
+            y += jU[j];
+        }
+        sa[threadIdx.x] = x;
+        sb[threadIdx.x] = y;
+        __syncthreads();
+        for (int s = 512; s > 0; s >>= 1) {
+            if ((int)threadIdx.x < s) {
+                sa[threadIdx.x] += sa[threadIdx.x + s];
+                sb[threadIdx.x] += sb[threadIdx.x + s];
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            out[2 * m] = sa[0];
+            out[2 * m + 1] = sb[0];
+            if (m == 0) {
+                ctr->moved = *moved;
+                ctr->c_nnz = coff_src[k];
+            }
+        }
+        return;
+    }
     const int64_t n = min(coff_src[k], cap);
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+    const int64_t g = (blockIdx.x - n_inst) * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t st = (int64_t)(gridDim.x - n_inst) * blockDim.x;
     for (int64_t e = g; e < n; e += st) {
         term_dst[e] = term_src[e];
         val_dst[e] = val_src[e];
@@ -426,32 +462,46 @@ __global__ void k_copy_back(int32_t k, int64_t cap, const int64_t *coff_src, con
     for (int64_t j = g; j < k; j += st) sn_dst[j] = sn_src[j];
 }
 
-// Per-instance objective sums (one CTA per instance), fixed order:
-// per-thread strided partial sums, then a tree.
-__global__ void __launch_bounds__(1024) k_sum_inst(const int32_t *inst_k, const double *a, const double *b,
-                                                   double *out) {
-    __shared__ double sa[1024], sb[1024];
-    const int m = blockIdx.x;
-    const int j0 = inst_k[m], j1 = inst_k[m + 1];
-    double x = 0.0, y = 0.0;
-    for (int j = j0 + threadIdx.x; j < j1; j += 1024) {
-        x += a[j];
-        y += b[j];
-    }
-    sa[threadIdx.x] = x;
-    sb[threadIdx.x] = y;
-    __syncthreads();
-    for (int s = 512; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) {
-            sa[threadIdx.x] += sa[threadIdx.x + s];
-            sb[threadIdx.x] += sb[threadIdx.x + s];
+// Offsets of the new rows: exclusive sums of sz[0..k) into coff[0..k], one CTA.
+__global__ void __launch_bounds__(1024) k_row_offsets(int32_t k, const int64_t *sz, int64_t *coff) {
+    constexpr int PER = 4;
+    __shared__ int64_t warp_s[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t carry = 0;
+    for (int64_t b = 0; b < k; b += 1024 * PER) {
+        const int64_t j0 = b + (int64_t)threadIdx.x * PER;
+        int64_t v[PER], sum = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            v[q] = j0 + q < k ? sz[j0 + q] : 0;
+            sum += v[q];
         }
+        int64_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) warp_s[warp] = inc;
+        __syncthreads();
+        int64_t w = warp_s[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        const int64_t total = __shfl_sync(0xffffffffu, w, 31);
+        const int64_t before = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+        int64_t at = carry + (warp ? before : 0) + inc - sum;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            if (j0 + q < k) coff[j0 + q] = at;
+            at += v[q];
+        }
+        carry += total;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        out[2 * m] = sa[0];
-        out[2 * m + 1] = sb[0];
-    }
+    if (threadIdx.x == 0) coff[k] = carry;
 }
 
 // ---------------- u2-u4, dense accumulator form ----------------
@@ -467,42 +517,55 @@ __global__ void __launch_bounds__(1024) k_sum_inst(const int32_t *inst_k, const 
 // 2^-shift per member. The clusters touched are exactly the moving ones; their
 // rows are then read in ascending term order.
 
-__global__ void k_label_counts(int64_t N, const int32_t *labels, int64_t *cnt) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(reinterpret_cast<unsigned long long *>(cnt + labels[i]), 1ull);
-}
-
-// One warp per object whose label changed since it was last added: its q
-// values move from the old cluster's row to the new one's, and every entry
-// added to has its bit set in the occupancy map (bits, 32 entries per word;
-// null: no map).
-__global__ void k_acc_scatter(int64_t N, const int32_t *labels, int32_t *acc_lab, const int64_t *row_ptr,
+// Member counts of the labels, and the objects whose label changed since they
+// were last added: a changed object's q values move from the old cluster's row
+// to the new one's, and every entry added to has its bit set in the occupancy
+// map (bits, 32 entries per word; null: no map). A warp looks at `per` (at
+// most 32) objects at once and takes the changed ones of them one by one, all
+// lanes on an object's entries: one warp per object, changed or not, spent
+// most of its warps on finding nothing to do.
+__global__ void k_acc_scatter(int64_t N, int per, const int32_t *labels, int32_t *acc_lab, const int64_t *row_ptr,
                               const int32_t *idx, const float *val, const int32_t *clu_doff, const int64_t *acc_off,
-                              float fscale, int64_t *acc, uint32_t *bits, const int64_t *bit_off, int64_t *moved) {
+                              float fscale, int64_t *acc, uint32_t *bits, const int64_t *bit_off, int64_t *cnt,
+                              int64_t *moved) {
+    constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t stride = (((int64_t)gridDim.x * blockDim.x) >> 5) * per;
     long long mv = 0;
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < N; i += nw) {
-        const int32_t jn = labels[i], jo = acc_lab[i];
-        if (jn == jo) continue;
-        const int64_t rb = row_ptr[i], re = row_ptr[i + 1];
-        const int32_t dn = clu_doff[jn];
-        unsigned long long *rn = reinterpret_cast<unsigned long long *>(acc + acc_off[jn] - dn);
-        uint32_t *bn = bits ? bits + bit_off[jn] : nullptr;
-        unsigned long long *ro =
-            jo >= 0 ? reinterpret_cast<unsigned long long *>(acc + acc_off[jo] - clu_doff[jo]) : nullptr;
-        for (int64_t h = rb + lane; h < re; h += 32) {
-            const unsigned long long q = (unsigned long long)__float2ll_ru(val[h] * fscale);
-            const int32_t t = idx[h];
-            atomicAdd(rn + t, q);
-            if (ro) atomicAdd(ro + t, 0ull - q);  // two's complement: subtracts q
-            const uint32_t bit = 1u << ((t - dn) & 31);
-            if (bn && !(bn[(t - dn) >> 5] & bit)) atomicOr(bn + ((t - dn) >> 5), bit);
+    for (int64_t i0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * per; i0 < N; i0 += stride) {
+        const int64_t i = i0 + lane;
+        const bool valid = lane < per && i < N;
+        const int32_t jn = valid ? labels[i] : -1, jo = valid ? acc_lab[i] : -1;
+        if (valid) atomicAdd(reinterpret_cast<unsigned long long *>(cnt + jn), 1ull);
+        const bool changed = valid && jn != jo;
+        int64_t rb = 0, re = 0;
+        if (changed) {
+            rb = row_ptr[i];
+            re = row_ptr[i + 1];
+            acc_lab[i] = jn;
+            mv += (re - rb) * (jo >= 0 ? 2 : 1);
         }
-        mv += (re - rb) * (jo >= 0 ? 2 : 1);
-        __syncwarp();
-        if (lane == 0) acc_lab[i] = jn;
+        for (unsigned todo = __ballot_sync(FULL, changed); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int32_t n = __shfl_sync(FULL, jn, src), o = __shfl_sync(FULL, jo, src);
+            const int64_t b = __shfl_sync(FULL, rb, src), e = __shfl_sync(FULL, re, src);
+            const int32_t dn = clu_doff[n];
+            unsigned long long *rn = reinterpret_cast<unsigned long long *>(acc + acc_off[n] - dn);
+            uint32_t *bn = bits ? bits + bit_off[n] : nullptr;
+            unsigned long long *ro =
+                o >= 0 ? reinterpret_cast<unsigned long long *>(acc + acc_off[o] - clu_doff[o]) : nullptr;
+            for (int64_t h = b + lane; h < e; h += 32) {
+                const unsigned long long q = (unsigned long long)__float2ll_ru(val[h] * fscale);
+                const int32_t t = idx[h];
+                atomicAdd(rn + t, q);
+                if (ro) atomicAdd(ro + t, 0ull - q);  // two's complement: subtracts q
+                const uint32_t bit = 1u << ((t - dn) & 31);
+                if (bn && !(bn[(t - dn) >> 5] & bit)) atomicOr(bn + ((t - dn) >> 5), bit);
+            }
+        }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mv += __shfl_xor_sync(FULL, mv, o);
     if (lane == 0 && mv) atomicAdd(reinterpret_cast<unsigned long long *>(moved), (unsigned long long)mv);
 }
 
@@ -574,7 +637,7 @@ __device__ __forceinline__ void block_sum_u128(unsigned long long &hi, unsigned 
 // its map, the bits of entries that became zero are cleared.
 // Other clusters keep their row (sizes and objective pieces as in k_write_rows).
 __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
-    int32_t k, const int64_t *flag, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
+    int32_t k, const uint8_t *lam, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
     const int64_t *acc, uint32_t *bits, const int64_t *bit_off, int64_t avg_len, double inv_scale,
     const int64_t *coff_old, const int32_t *cterm_old, const float *cval_old, const double *snorm_old, int64_t *sz, double *snorm_new,
     double *jA, double *jU) {
@@ -584,7 +647,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     const int j = blockIdx.x;
     if (j >= k) return;
     const int64_t cb = coff_old[j], ce = coff_old[j + 1];
-    if (!flag[j]) {
+    if (lam[j] != 0 || cnt[j] == 0) {  // invariant or empty
         if (threadIdx.x == 0) {
             const double sn = cnt[j] > 0 ? snorm_old[j] : 0.0;
             sz[j] = ce - cb;
@@ -667,7 +730,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
 // compaction of the non-zero entries) and
 // u = s * (2^-shift / ||s||) as FP32. Other clusters copy their row.
 __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows2(
-    int32_t k, const int64_t *flag, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
+    int32_t k, const uint8_t *lam, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
     const int64_t *acc, const uint32_t *bits, const int64_t *bit_off, int64_t avg_len, double inv_scale, const int64_t *coff_old, const int32_t *cterm_old,
     const float *cval_old, const double *snorm_new, const int64_t *coff_new, int32_t *cterm_new, float *cval_new,
     int32_t *cclu_new, int64_t cap, unsigned long long *error) {
@@ -681,7 +744,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows2(
     if (over) return;
     const int64_t o0 = coff_new[j];
     const int64_t cb = coff_old[j], ce = coff_old[j + 1];
-    if (!flag[j]) {
+    if (lam[j] != 0 || cnt[j] == 0) {  // invariant or empty
         for (int64_t q = cb + threadIdx.x; q < ce; q += WR_THREADS) {
             cterm_new[o0 + (q - cb)] = cterm_old[q];
             cval_new[o0 + (q - cb)] = cval_old[q];
@@ -803,17 +866,6 @@ __global__ void k_if_keys(const int64_t *n_dev, int64_t cap, const int32_t *cter
     }
 }
 
-__global__ void k_if_lens(int32_t D, const uint32_t *cnt2, int64_t *len, int64_t *slen, int32_t *mf0) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < D) {
-        const int64_t l = (int64_t)cnt2[2 * t] + (int64_t)cnt2[2 * t + 1];
-        len[t] = l;
-        // scan copy: fronts and backs take whole quads of 4 entries
-        slen[t] = (((int64_t)cnt2[2 * t] + 3) & ~(int64_t)3) + (((int64_t)cnt2[2 * t + 1] + 3) & ~(int64_t)3);
-        mf0[t] = (int32_t)cnt2[2 * t];
-    }
-}
-
 // Canonical arrays (if_cid: global cluster ids, if_val) in sorted order.
 __global__ void k_if_fill(const int64_t *n_dev, int64_t cap, const uint32_t *order, const int32_t *cclu,
                           const float *cval, int32_t *if_cid, float *if_val) {
@@ -827,13 +879,56 @@ __global__ void k_if_fill(const int64_t *n_dev, int64_t cap, const uint32_t *ord
 
 // ---------------- scan order and dense head rows ----------------
 
-// Scan position of every cluster: within its instance, the moving clusters of
-// lambda^[r] (mov_list, ascending) take positions 0 .. n_mov - 1 and the
-// invariant ones follow in ascending id; id_order (IVF-CBICP) keeps the ids.
-__global__ void k_positions(int32_t k, int32_t n_inst, const int32_t *inst_k, const uint8_t *lam,
-                            const int32_t *mov_list, const int32_t *mov_beg, int id_order, int32_t *clu_pos,
-                            int32_t *pos_clu) {
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < k; g += (int64_t)gridDim.x * blockDim.x) {
+constexpr int DENSE_BINS = 64;      // list length / k in steps of 1/64
+constexpr int DENSE_MIN_LEN = 32;   // shorter lists stay sparse whatever k
+
+// instance of term t, its k, and the 1/64 bin of its list length
+__device__ __forceinline__ void term_bin(int32_t t, int32_t n_inst, const int32_t *inst_d, const int32_t *inst_k,
+                                         int64_t L, int32_t *kin, int *bin) {
+    int lo = 0, hi = n_inst - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (inst_d[mid] <= t) lo = mid; else hi = mid - 1;
+    }
+    const int32_t km = inst_k[lo + 1] - inst_k[lo];
+    *kin = km;
+    const int64_t q = (L * DENSE_BINS) / (km > 0 ? km : 1);
+    *bin = (int)(q < DENSE_BINS ? q : DENSE_BINS);
+}
+
+// First pass over the terms of the build: list lengths and front lengths from
+// the per-part counts, the slot cursors cleared, and the histogram of the
+// dense-row entries each length bin would take (lists of at least min_len
+// postings; formed per block, then added). The scan position of every cluster
+// is found beside it: within its instance, the moving clusters of lambda^[r]
+// (mov_list, ascending) take positions 0 .. n_mov - 1 and the invariant ones
+// follow in ascending id; id_order (IVF-CBICP) keeps the ids.
+__global__ void __launch_bounds__(TPB) k_if_lists(int32_t D, int32_t k, int32_t n_inst, const int32_t *inst_d,
+                                                  const int32_t *inst_k, const uint32_t *cnt2, int64_t min_len,
+                                                  int dense, int64_t *len, int32_t *mf0, uint32_t *cursor,
+                                                  unsigned long long *hist, const uint8_t *lam,
+                                                  const int32_t *mov_list, const int32_t *mov_beg, int id_order,
+                                                  int32_t *clu_pos, int32_t *pos_clu, DevCounters *ctr) {
+    __shared__ unsigned long long sh[DENSE_BINS + 1];
+    for (int b = threadIdx.x; b <= DENSE_BINS; b += TPB) sh[b] = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->dense_terms = 0;
+    __syncthreads();
+    const int64_t g0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = g0; t < D; t += st) {
+        const uint32_t f = cnt2[2 * t], b = cnt2[2 * t + 1];
+        const int64_t L = (int64_t)f + (int64_t)b;
+        len[t] = L;
+        mf0[t] = (int32_t)f;
+        cursor[2 * t] = 0u;
+        cursor[2 * t + 1] = 0u;
+        if (dense && L >= min_len) {
+            int32_t km;
+            int bin;
+            term_bin((int32_t)t, n_inst, inst_d, inst_k, L, &km, &bin);
+            atomicAdd(sh + bin, (unsigned long long)((km + 7) & ~7));
+        }
+    }
+    for (int64_t g = g0; g < k; g += st) {
         const int32_t j = (int32_t)g;
         int lo = 0, hi = n_inst - 1;  // instance: largest m with inst_k[m] <= j
         while (lo < hi) {
@@ -854,80 +949,106 @@ __global__ void k_positions(int32_t k, int32_t n_inst, const int32_t *inst_k, co
         clu_pos[j] = p;
         pos_clu[koff + p] = jl;
     }
+    __syncthreads();
+    for (int b = threadIdx.x; b <= DENSE_BINS; b += TPB)
+        if (sh[b]) atomicAdd(hist + b, sh[b]);
 }
 
-constexpr int DENSE_BINS = 64;      // list length / k in steps of 1/64
-constexpr int DENSE_MIN_LEN = 32;   // shorter lists stay sparse whatever k
+// The terms in tiles of IF_TILE: second pass, the width of a dense row (in
+// 8-entry units) or the room of a sparse list for every term, and each tile's
+// sums of list lengths, sparse entries and row widths. Every block finds the
+// dense threshold from the histogram: the smallest bin >= bmin whose rows
+// (with every longer bin's) fit in cap entries; DENSE_BINS + 1 = no dense rows.
+constexpr int IF_TILE = 4 * TPB;
 
-// instance of term t, its k, and the 1/64 bin of its list length
-__device__ __forceinline__ void term_bin(int32_t t, int32_t n_inst, const int32_t *inst_d, const int32_t *inst_k,
-                                         int64_t L, int32_t *kin, int *bin) {
-    int lo = 0, hi = n_inst - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (inst_d[mid] <= t) lo = mid; else hi = mid - 1;
+struct IfSums {
+    long long len, room, w8;
+};
+
+__device__ __forceinline__ IfSums if_add(IfSums a, IfSums b) {
+    return {a.len + b.len, a.room + b.room, a.w8 + b.w8};
+}
+
+// inclusive scan over the block; total for every thread (two barriers)
+__device__ __forceinline__ IfSums if_block_scan(IfSums v, IfSums *warp_s, IfSums &total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const IfSums y = {__shfl_up_sync(0xffffffffu, v.len, o), __shfl_up_sync(0xffffffffu, v.room, o),
+                          __shfl_up_sync(0xffffffffu, v.w8, o)};
+        if (lane >= o) v = if_add(v, y);
     }
-    const int32_t km = inst_k[lo + 1] - inst_k[lo];
-    *kin = km;
-    const int64_t q = (L * DENSE_BINS) / (km > 0 ? km : 1);
-    *bin = (int)(q < DENSE_BINS ? q : DENSE_BINS);
-}
-
-// Histogram of the dense-row entries each length bin would take (lists of at
-// least min_len postings).
-__global__ void k_dense_hist(int32_t D, int32_t n_inst, const int32_t *inst_d, const int32_t *inst_k,
-                             const int64_t *len, int64_t min_len, unsigned long long *hist) {
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D; g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t L = len[g];
-        if (L < min_len) continue;
-        int32_t km;
-        int bin;
-        term_bin((int32_t)g, n_inst, inst_d, inst_k, L, &km, &bin);
-        atomicAdd(hist + bin, (unsigned long long)((km + 7) & ~7));
+    __syncthreads();
+    if (lane == 31) warp_s[warp] = v;
+    __syncthreads();
+    IfSums before = {0, 0, 0};
+    total = {0, 0, 0};
+#pragma unroll
+    for (int w = 0; w < TPB / 32; ++w) {
+        if (w < warp) before = if_add(before, warp_s[w]);
+        total = if_add(total, warp_s[w]);
     }
+    return if_add(before, v);
 }
 
-// Smallest bin >= bmin whose rows (with every longer bin's) fit in cap
-// entries; DENSE_BINS + 1 = no dense rows.
-__global__ void k_dense_threshold(const unsigned long long *hist, int bmin, unsigned long long cap, int32_t *thr) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    unsigned long long acc = 0;
-    int b = DENSE_BINS + 1;
-    for (int q = DENSE_BINS; q >= bmin; --q) {
-        acc += hist[q];
-        if (acc > cap) break;
-        b = q;
-    }
-    *thr = b;
-}
+__device__ __forceinline__ int64_t quads4(int64_t n) { return (n + 3) & ~(int64_t)3; }
 
-// Dense-row width (in 8-entry units) of every term; the sparse scan copy
-// gives dense terms no room.
-__global__ void k_dense_width(int32_t D, int32_t n_inst, const int32_t *inst_d, const int32_t *inst_k,
-                              const int64_t *len, int64_t min_len, const int32_t *thr, int64_t *w8, int64_t *slen) {
-    const int b = *thr;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D; g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t L = len[g];
-        int64_t w = 0;
-        if (L >= min_len) {
-            int32_t km;
-            int bin;
-            term_bin((int32_t)g, n_inst, inst_d, inst_k, L, &km, &bin);
-            if (bin >= b) w = (km + 7) >> 3;
+__global__ void __launch_bounds__(TPB) k_if_tiles(int32_t D, int32_t n_inst, const int32_t *inst_d,
+                                                  const int32_t *inst_k, const int64_t *len, const int32_t *mf0,
+                                                  int64_t min_len, const unsigned long long *hist, int bmin,
+                                                  unsigned long long cap, int32_t *thr, int32_t *w8, IfSums *tiles) {
+    __shared__ IfSums warp_s[TPB / 32];
+    __shared__ unsigned long long sh[DENSE_BINS + 1];
+    __shared__ int s_thr;
+    for (int b = threadIdx.x; b <= DENSE_BINS; b += TPB) sh[b] = hist[b];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long acc = 0;
+        int b = DENSE_BINS + 1;
+        for (int q = DENSE_BINS; q >= bmin; --q) {
+            acc += sh[q];
+            if (acc > cap) break;
+            b = q;
         }
-        w8[g] = w;
-        if (w) slen[g] = 0;
+        s_thr = b;
+        if (blockIdx.x == 0) *thr = b;
+    }
+    __syncthreads();
+    const int64_t n_tiles = ((int64_t)D + IF_TILE - 1) / IF_TILE;
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        IfSums v = {0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < IF_TILE / TPB; ++q) {
+            const int64_t t = tile * IF_TILE + (int64_t)q * TPB + threadIdx.x;
+            if (t >= D) break;
+            const int64_t L = len[t];
+            int64_t w = 0;
+            if (L >= min_len && s_thr <= DENSE_BINS) {
+                int32_t km;
+                int bin;
+                term_bin((int32_t)t, n_inst, inst_d, inst_k, L, &km, &bin);
+                if (bin >= s_thr) w = (km + 7) >> 3;
+            }
+            w8[t] = (int32_t)w;
+            const int64_t f = mf0[t];
+            v = if_add(v, {L, w ? 0 : quads4(f) + quads4(L - f), w});
+        }
+        IfSums total;
+        if_block_scan(v, warp_s, total);
+        if (threadIdx.x == 0) tiles[tile] = total;
     }
 }
 
-// What the assignment reads about a term, in one 16-byte load: where its list
-// starts in the scan copy, its front and list lengths, and its dense row. The
-// last quads of a sparse list's front and back are filled up with zero
-// postings here (they add 0 to a score).
-__global__ void k_term_desc(int32_t D, const int64_t *w8, const int64_t *base8, const int64_t *sc_off,
-                            const int32_t *mf0, const int64_t *len, int4 *tdesc, uint16_t *sc_id16, int32_t *sc_id32,
-                            float *sc_val, uint32_t *sc_pack, uint16_t *sc_lp, DevCounters *ctr) {
-    long long n = 0;
+// Third pass: the offsets (sums of the earlier tiles, then within the tile)
+// and what the assignment reads about a term, in one 16-byte descriptor: the
+// first quad of its list in the scan copy, its front and list lengths, and its
+// dense row. The last quads of a sparse list's front and back are filled up
+// with zero postings here (they add 0 to a score).
+__global__ void __launch_bounds__(TPB) k_if_offsets(int32_t D, const int64_t *len, const int32_t *mf0,
+                                                    const int32_t *w8, const IfSums *tiles, int64_t *if_off,
+                                                    int4 *tdesc, uint16_t *sc_id16, int32_t *sc_id32, float *sc_val,
+                                                    uint32_t *sc_pack, uint16_t *sc_lp, DevCounters *ctr) {
+    __shared__ IfSums warp_s[TPB / 32];
     auto fill = [&](int64_t from, int64_t to) {
         for (int64_t p = from; p < to; ++p) {
             if (sc_id16) sc_id16[p] = 0;
@@ -937,23 +1058,51 @@ __global__ void k_term_desc(int32_t D, const int64_t *w8, const int64_t *base8, 
             if (sc_lp) sc_lp[p] = 0;
         }
     };
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D; g += (int64_t)gridDim.x * blockDim.x) {
-        const bool d = w8[g] > 0;
-        const int64_t at = sc_off[g], f = mf0[g], l = len[g];
-        tdesc[g] = make_int4((int)(at >> 2), (int)f, (int)l, d ? (int)base8[g] : -1);
-        n += d;
-        if (!d) {
-            const int64_t f4 = (f + 3) & ~(int64_t)3, b4 = (l - f + 3) & ~(int64_t)3;
-            fill(at + f, at + f4);
-            fill(at + f4 + (l - f), at + f4 + b4);
+    const int64_t n_tiles = ((int64_t)D + IF_TILE - 1) / IF_TILE;
+    long long n_dense = 0;
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        IfSums base = {0, 0, 0};
+        for (int64_t q = threadIdx.x; q < tile; q += TPB) base = if_add(base, tiles[q]);
+        IfSums unused;
+        if_block_scan(base, warp_s, unused);
+        base = unused;  // every earlier tile
+#pragma unroll
+        for (int q = 0; q < IF_TILE / TPB; ++q) {
+            const int64_t t = tile * IF_TILE + (int64_t)q * TPB + threadIdx.x;
+            int64_t L = 0, f = 0, w = 0;
+            if (t < D) {
+                L = len[t];
+                f = mf0[t];
+                w = w8[t];
+            }
+            const IfSums v = {L, w ? 0 : quads4(f) + quads4(L - f), w};
+            IfSums total;
+            const IfSums inc = if_block_scan(v, warp_s, total);
+            if (t < D) {
+                const int64_t at = base.room + inc.room - v.room;
+                if_off[t] = base.len + inc.len - L;
+                tdesc[t] = make_int4((int)(at >> 2), (int)f, (int)L, w ? (int)(base.w8 + inc.w8 - w) : -1);
+                if (w) {
+                    ++n_dense;
+                } else {
+                    fill(at + f, at + quads4(f));
+                    fill(at + quads4(f) + (L - f), at + v.room);
+                }
+            }
+            base = if_add(base, total);
+        }
+        if (tile == n_tiles - 1 && threadIdx.x == 0) {
+            if_off[D] = base.len;
+            ctr->sparse_entries = base.room;
+            ctr->dense_used = base.w8;
         }
     }
-    if (n) atomicAdd(reinterpret_cast<unsigned long long *>(&ctr->dense_terms), (unsigned long long)n);
+    if (n_dense) atomicAdd(reinterpret_cast<unsigned long long *>(&ctr->dense_terms), (unsigned long long)n_dense);
 }
 
 // zero the entries in use (16 bytes at a time; rows are multiples of 8 entries)
-__global__ void k_dense_zero(const int64_t *used8, int esize, uint4 *dense) {
-    const int64_t n16 = used8[0] * 8 * esize / 16;
+__global__ void k_dense_zero(const DevCounters *ctr, int esize, uint4 *dense) {
+    const int64_t n16 = ctr->dense_used * 8 * esize / 16;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n16; q += (int64_t)gridDim.x * blockDim.x)
         dense[q] = make_uint4(0u, 0u, 0u, 0u);
 }
@@ -1122,66 +1271,49 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     const int32_t D = c->D;
     Workspace &ws = c->ws;
     size_t mark = ws.used;
-    uint32_t *cnt2 = ws.take<uint32_t>((size_t)2 * D);
-    int64_t *len = ws.take<int64_t>((size_t)D + 1);
-    int64_t *slen = ws.take<int64_t>((size_t)D + 1);
-    int64_t *w8 = ws.take<int64_t>((size_t)D + 1);
-    int64_t *base8 = ws.take<int64_t>((size_t)D + 1);
-    unsigned long long *hist = ws.take<unsigned long long>(DENSE_BINS + 1);
-    int64_t *total = ws.take<int64_t>(3);
-    if (!cnt2 || !len || !slen || !w8 || !base8 || !hist || !total) return cudaErrorMemoryAllocation;
+    const int64_t n_tiles = ((int64_t)D + IF_TILE - 1) / IF_TILE;
+    // the counts and the histogram are cleared together
+    uint32_t *cnt2 = ws.take<uint32_t>((size_t)2 * D + 2 * (DENSE_BINS + 1));
+    uint32_t *cursor = ws.take<uint32_t>((size_t)2 * D);
+    int64_t *len = ws.take<int64_t>((size_t)D);
+    int32_t *w8 = ws.take<int32_t>((size_t)D);
+    IfSums *tiles = ws.take<IfSums>((size_t)n_tiles);
+    if (!cnt2 || !cursor || !len || !w8 || !tiles) return cudaErrorMemoryAllocation;
+    unsigned long long *hist = reinterpret_cast<unsigned long long *>(cnt2 + 2 * (size_t)D);
     cudaStream_t s = c->stream;
     const bool cb = c->cfg.icp == 2;
     c->canon_stale = true;
-    SIVF_CUDA_TRY(cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * 2 * D, s));
+    SIVF_CUDA_TRY(cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * (2 * (size_t)D + 2 * (DENSE_BINS + 1)), s));
     k_if_count<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, c->cterm[cur], c->cclu, c->lam, cb ? 0 : 1, cnt2);
-    k_if_lens<<<blocks_for(D), TPB, 0, s>>>(D, cnt2, len, slen, c->if_mf0);
-    // scan order of lambda^[r] (mov_list and mov_beg were computed from it)
-    k_positions<<<blocks_gs(c->k), TPB, 0, s>>>(c->k, c->n_inst, c->inst_k, c->lam, c->mov_list, c->mov_beg,
-                                                 cb ? 1 : 0, c->clu_pos, c->pos_clu);
-    note_launch(3);
     // dense head rows: the longest lists (relative to their instance's k) that
     // fit in the row capacity, from dense_frac of k up; with dense_all every
     // list (the dense-mean variant: all of the centroids as dense rows)
-    SIVF_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (DENSE_BINS + 1), s));
     const bool all = c->cfg.dense_all != 0;
     const int bmin = all ? 0 : std::max(1, (int)ceilf(c->dense_frac * DENSE_BINS));
     const int64_t min_len = all ? 1 : DENSE_MIN_LEN;
     const bool dense = c->cap_dense > 0 && !cb && bmin <= DENSE_BINS;
-    if (dense) {
-        k_dense_hist<<<blocks_gs(D), TPB, 0, s>>>(D, c->n_inst, c->inst_d, c->inst_k, len, min_len, hist);
-        k_dense_threshold<<<1, 32, 0, s>>>(hist, bmin, (unsigned long long)c->cap_dense, c->dense_thr);
-        note_launch(2);
-    } else {  // no bin qualifies: the threshold becomes DENSE_BINS + 1 (no rows)
-        k_dense_threshold<<<1, 32, 0, s>>>(hist, DENSE_BINS + 1, 0ull, c->dense_thr);
-        note_launch();
-    }
-    k_dense_width<<<blocks_gs(D), TPB, 0, s>>>(D, c->n_inst, c->inst_d, c->inst_k, len, min_len, c->dense_thr, w8,
-                                                slen);
-    note_launch();
+    const unsigned tile_blocks = (unsigned)std::min<int64_t>(n_tiles, GS_MAX_BLOCKS);
+    // (mov_list and mov_beg belong to the current lambda^[r])
+    k_if_lists<<<(unsigned)std::min<int64_t>(blocks_for(std::max(D, c->k)), 1024), TPB, 0, s>>>(
+        D, c->k, c->n_inst, c->inst_d, c->inst_k, cnt2, min_len, dense ? 1 : 0, len, c->if_mf0, cursor, hist, c->lam,
+        c->mov_list, c->mov_beg, cb ? 1 : 0, c->clu_pos, c->pos_clu, c->ctr);
+    k_if_tiles<<<tile_blocks, TPB, 0, s>>>(D, c->n_inst, c->inst_d, c->inst_k, len, c->if_mf0, min_len, hist,
+                                           dense ? bmin : DENSE_BINS + 1, (unsigned long long)c->cap_dense,
+                                           c->dense_thr, w8, tiles);
+    k_if_offsets<<<tile_blocks, TPB, 0, s>>>(D, len, c->if_mf0, w8, tiles, c->if_off, c->tdesc, c->sc_id16, c->sc_id32,
+                                             c->sc_val, c->sc_pack, c->sc_lp, c->ctr);
+    note_launch(4);
     SIVF_CUDA_TRY(cudaGetLastError());
-    SIVF_CUDA_TRY(scan_exclusive_i64(len, c->if_off, D, total, ws, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->if_off + D, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(scan_exclusive_i64(slen, slen, D, total + 1, ws, s));
-    SIVF_CUDA_TRY(scan_exclusive_i64(w8, base8, D, total + 2, ws, s));
-    SIVF_CUDA_TRY(cudaMemsetAsync(&c->ctr->dense_terms, 0, sizeof(long long), s));
-    k_term_desc<<<blocks_gs(D), TPB, 0, s>>>(D, w8, base8, slen, c->if_mf0, len, c->tdesc, c->sc_id16, c->sc_id32,
-                                              c->sc_val, c->sc_pack, c->sc_lp, c->ctr);
-    note_launch();
     if (dense) {
         const int esize = c->cfg.prec == SIVF_FP32 ? 4 : 2;
-        k_dense_zero<<<blocks_gs(c->cap_dense * esize / 16), TPB, 0, s>>>(total + 2, esize,
+        k_dense_zero<<<blocks_gs(c->cap_dense * esize / 16), TPB, 0, s>>>(c->ctr, esize,
                                                                             static_cast<uint4 *>(c->dense_val));
         note_launch();
     }
-    // the counts are consumed: the same array now hands out the slots
-    SIVF_CUDA_TRY(cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * 2 * D, s));
     k_scan_fill<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, c->cterm[cur], c->cclu, c->cval[cur], c->lam, cb ? 0 : 1,
-                                                c->clu_pos, c->tdesc, cnt2, (int)c->cfg.prec, c->dense_val, c->sc_id16, c->sc_id32, c->sc_val,
-                                                c->sc_pack, c->sc_lp);
+                                                c->clu_pos, c->tdesc, cursor, (int)c->cfg.prec, c->dense_val,
+                                                c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp);
     note_launch();
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->dense_used, total + 2, sizeof(long long), cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->sparse_entries, total + 1, sizeof(long long), cudaMemcpyDeviceToDevice, s));
     SIVF_CUDA_TRY(cudaGetLastError());
     ws.used = mark;
     return cudaSuccess;
@@ -1220,6 +1352,32 @@ cudaError_t build_canonical_if(sivf_ctx *c) {
     return cudaSuccess;
 }
 
+namespace {
+
+// coff of the new buffer from the row sizes
+cudaError_t row_offsets(sivf_ctx *c, const int64_t *sz, int nw) {
+    cudaStream_t s = c->stream;
+    if (c->k <= 1 << 18) {  // one CTA, 4096 rows a turn
+        k_row_offsets<<<1, 1024, 0, s>>>(c->k, sz, c->coff[nw]);
+        note_launch();
+        return cudaGetLastError();
+    }
+    return scan_exclusive_i64(sz, c->coff[nw], c->k, c->coff[nw] + c->k, c->ws, s);
+}
+
+// objective sums, rows into the current buffer, counts of the step
+cudaError_t finish_rows(sivf_ctx *c, const double *jA, const double *jU, const int64_t *moved) {
+    const int cur = c->cur, nw = 1 - c->cur;
+    const unsigned copy = (unsigned)std::min<int64_t>((c->cap_c + 1023) / 1024, 1024);
+    k_finish_rows<<<(unsigned)c->n_inst + copy, 1024, 0, c->stream>>>(
+        c->k, c->cap_c, c->n_inst, c->inst_k, jA, jU, c->obj_dev, c->coff[nw], c->cterm[nw], c->cval[nw],
+        c->snorm_new, c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm, moved, c->ctr);
+    note_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 // Update step with the dense accumulator (u1: member counts only; u2-u4 as
 // above; u5 as in the sort form).
 cudaError_t run_update_dense(sivf_ctx *c) {
@@ -1229,38 +1387,29 @@ cudaError_t run_update_dense(sivf_ctx *c) {
     const int64_t N = c->N;
     const int32_t k = c->k;
     const int cur = c->cur, nw = 1 - c->cur;
-    int64_t *cnt = ws.take<int64_t>(k), *flag = ws.take<int64_t>(k);
-    int64_t *sz = ws.take<int64_t>((size_t)k + 1), *newn_d = ws.take<int64_t>(1), *moved_d = ws.take<int64_t>(1);
+    int64_t *cnt = ws.take<int64_t>((size_t)k + 1), *sz = ws.take<int64_t>((size_t)k + 1);
     double *jAd = ws.take<double>(k), *jUd = ws.take<double>(k);
-    if (!cnt || !flag || !sz || !newn_d || !moved_d || !jAd || !jUd) return cudaErrorMemoryAllocation;
-    SIVF_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * k, s));
-    SIVF_CUDA_TRY(cudaMemsetAsync(moved_d, 0, sizeof(int64_t), s));
-    k_label_counts<<<blocks_gs(N), TPB, 0, s>>>(N, c->labels, cnt);
-    k_recompute_flags<<<blocks_for(k), TPB, 0, s>>>(k, c->lam, cnt, flag);
+    if (!cnt || !sz || !jAd || !jUd) return cudaErrorMemoryAllocation;
+    int64_t *moved_d = cnt + k;  // cleared with the counts
+    SIVF_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * ((size_t)k + 1), s));
     const float fscale = ldexpf(1.0f, c->acc_shift);
     const double inv_scale = ldexp(1.0, -c->acc_shift);
     const int64_t avg_len = c->nnz / N + 1;  // entries of an object
-    k_acc_scatter<<<blocks_gs(N * 32), TPB, 0, s>>>(N, c->labels, c->acc_lab, c->row_ptr, c->idx, c->val,
-                                                     c->clu_doff, c->acc_off, fscale, c->acc, c->acc_bits,
-                                                     c->acc_bit_off, moved_d);
-    k_acc_rows1<<<(unsigned)k, WR_THREADS, 0, s>>>(k, flag, cnt, c->acc_off, c->clu_doff, c->acc, c->acc_bits,
-                                                   c->acc_bit_off, avg_len, inv_scale, c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm, sz,
-                                                   c->snorm_new, jAd, jUd);
-    note_launch(4);
-    SIVF_CUDA_TRY(cudaGetLastError());
-    SIVF_CUDA_TRY(scan_exclusive_i64(sz, c->coff[nw], k, newn_d, ws, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->coff[nw] + k, newn_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    k_acc_rows2<<<(unsigned)k, WR_THREADS, 0, s>>>(k, flag, cnt, c->acc_off, c->clu_doff, c->acc, c->acc_bits,
-                                                   c->acc_bit_off, avg_len, inv_scale, c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm_new, c->coff[nw],
-                                                   c->cterm[nw], c->cval[nw], c->cclu, c->cap_c, &c->ctr->error);
-    k_sum_inst<<<(unsigned)c->n_inst, 1024, 0, s>>>(c->inst_k, jAd, jUd, c->obj_dev);
-    k_copy_back<<<blocks_gs(c->cap_c), TPB, 0, s>>>(k, c->cap_c, c->coff[nw], c->cterm[nw], c->cval[nw],
-                                                     c->snorm_new, c->coff[cur], c->cterm[cur], c->cval[cur],
-                                                     c->snorm);
+    int per = 1;  // objects a warp looks at together: as many as still leave every SM 64 warps
+    while (per < 32 && N / (2 * per) >= (int64_t)c->num_sms * 64) per *= 2;
+    k_acc_scatter<<<blocks_gs((N + per - 1) / per * 32), TPB, 0, s>>>(
+        N, per, c->labels, c->acc_lab, c->row_ptr, c->idx, c->val, c->clu_doff, c->acc_off, fscale, c->acc,
+        c->acc_bits, c->acc_bit_off, cnt, moved_d);
+    k_acc_rows1<<<(unsigned)k, WR_THREADS, 0, s>>>(k, c->lam, cnt, c->acc_off, c->clu_doff, c->acc, c->acc_bits,
+                                                   c->acc_bit_off, avg_len, inv_scale, c->coff[cur], c->cterm[cur],
+                                                   c->cval[cur], c->snorm, sz, c->snorm_new, jAd, jUd);
+    SIVF_CUDA_TRY(row_offsets(c, sz, nw));
+    k_acc_rows2<<<(unsigned)k, WR_THREADS, 0, s>>>(k, c->lam, cnt, c->acc_off, c->clu_doff, c->acc, c->acc_bits,
+                                                   c->acc_bit_off, avg_len, inv_scale, c->coff[cur], c->cterm[cur],
+                                                   c->cval[cur], c->snorm_new, c->coff[nw], c->cterm[nw], c->cval[nw],
+                                                   c->cclu, c->cap_c, &c->ctr->error);
     note_launch(3);
-    SIVF_CUDA_TRY(cudaGetLastError());
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->moved, moved_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->c_nnz, newn_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    SIVF_CUDA_TRY(finish_rows(c, jAd, jUd, moved_d));
     ws.reset();
     SIVF_CUDA_TRY(build_inverted_file(c));
     ws.reset();
@@ -1284,13 +1433,13 @@ cudaError_t run_update(sivf_ctx *c) {
     uint32_t *lk0 = ws.take<uint32_t>(N), *lv0 = ws.take<uint32_t>(N);
     uint32_t *lk1 = ws.take<uint32_t>(N), *lv1 = ws.take<uint32_t>(N);
     int64_t *cnt = ws.take<int64_t>(k), *flag = ws.take<int64_t>(k), *rrank = ws.take<int64_t>(k);
-    int64_t *nrec_d = ws.take<int64_t>(1), *T_d = ws.take<int64_t>(1), *newn_d = ws.take<int64_t>(1);
+    int64_t *nrec_d = ws.take<int64_t>(1), *T_d = ws.take<int64_t>(1);
     uint32_t *U_d = ws.take<uint32_t>(1);
     int64_t *sz = ws.take<int64_t>((size_t)k + 1);
     double *jAd = ws.take<double>(k), *jUd = ws.take<double>(k);
     int64_t *tc = ws.take<int64_t>(N), *toff = ws.take<int64_t>(N);
     int64_t *ubeg = ws.take<int64_t>((size_t)k + 1), *uend = ws.take<int64_t>((size_t)k + 1);
-    if (!lk0 || !lv0 || !lk1 || !lv1 || !cnt || !flag || !rrank || !nrec_d || !T_d || !newn_d || !U_d || !sz ||
+    if (!lk0 || !lv0 || !lk1 || !lv1 || !cnt || !flag || !rrank || !nrec_d || !T_d || !U_d || !sz ||
         !jAd || !jUd || !tc || !toff || !ubeg || !uend)
         return cudaErrorMemoryAllocation;
     SIVF_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * k, s));
@@ -1366,19 +1515,12 @@ cudaError_t run_update(sivf_ctx *c) {
     // u3/u4: new cluster-major rows (into the second buffer), copied back
     k_new_sizes<<<blocks_for(k), TPB, 0, s>>>(k, flag, rrank, ubeg, uend, c->coff[cur], sz);
     note_launch();
-    SIVF_CUDA_TRY(scan_exclusive_i64(sz, c->coff[nw], k, newn_d, ws, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->coff[nw] + k, newn_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    SIVF_CUDA_TRY(row_offsets(c, sz, nw));
     k_write_rows<<<(unsigned)k, WR_THREADS, 0, s>>>(
         k, flag, rrank, ubeg, uend, uterm, usum, cnt, c->coff[cur], c->cterm[cur], c->cval[cur], c->snorm,
         c->coff[nw], c->cterm[nw], c->cval[nw], c->cclu, c->snorm_new, jAd, jUd, c->cap_c, &c->ctr->error);
-    k_sum_inst<<<(unsigned)c->n_inst, 1024, 0, s>>>(c->inst_k, jAd, jUd, c->obj_dev);
-    k_copy_back<<<blocks_gs(c->cap_c), TPB, 0, s>>>(k, c->cap_c, c->coff[nw], c->cterm[nw], c->cval[nw],
-                                                     c->snorm_new, c->coff[cur], c->cterm[cur], c->cval[cur],
-                                                     c->snorm);
-    note_launch(3);
-    SIVF_CUDA_TRY(cudaGetLastError());
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->moved, T_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&c->ctr->c_nnz, newn_d, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    note_launch();
+    SIVF_CUDA_TRY(finish_rows(c, jAd, jUd, T_d));
     ws.reset();
 
     // u5: rebuild the structured inverted file with lambda^[r]

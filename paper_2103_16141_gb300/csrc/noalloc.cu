@@ -39,8 +39,8 @@ constexpr size_t kMaxTerms = SIVF_NOALLOC_MAX_TERMS;
 constexpr size_t kMaxClusters = SIVF_NOALLOC_MAX_CLUSTERS;
 
 // scratch layout, taken by a bump allocator in this order (256-byte aligned):
-// check flag, cluster id, keys, values, keys', values' (4 B x entries each),
-// per (term, part) counts (2 x terms x 4 B), list lengths ((terms + 1) x 8 B),
+// cluster id, keys, values, keys', values' (4 B x entries each), per (term,
+// part) counts (2 x terms x 4 B) and the check flag, list lengths ((terms + 1) x 8 B),
 // radix histogram (at most 1 MiB at the limits) and scan partials.
 constexpr size_t kScratchBytes = SIVF_NOALLOC_SCRATCH_BYTES;
 static_assert(kScratchBytes >= 256 + 5 * 4 * kMaxEntries + 2 * 4 * kMaxTerms + 8 * (kMaxTerms + 1) + (1u << 20),
@@ -152,20 +152,18 @@ extern "C" sivf_status sivf_build_inverted_file_noalloc(int32_t k, int32_t D, in
     ws.base = static_cast<char *>(base);
     ws.cap = kScratchBytes;
     const size_t n = (size_t)n_entries;
-    int *bad = ws.take<int>(1);
     int32_t *clu = ws.take<int32_t>(n + 1);
     uint32_t *k0 = ws.take<uint32_t>(n + 1), *v0 = ws.take<uint32_t>(n + 1);
     uint32_t *k1 = ws.take<uint32_t>(n + 1), *v1 = ws.take<uint32_t>(n + 1);
-    uint32_t *cnt2 = ws.take<uint32_t>(2 * (size_t)D);
+    uint32_t *cnt2 = ws.take<uint32_t>(2 * (size_t)D + 1);
     int64_t *len = ws.take<int64_t>((size_t)D + 1);
-    int64_t *total = ws.take<int64_t>(1);
-    if (!bad || !clu || !k0 || !v0 || !k1 || !v1 || !cnt2 || !len || !total) return SIVF_ERR_INVALID_ARG;
+    if (!clu || !k0 || !v0 || !k1 || !v1 || !cnt2 || !len) return SIVF_ERR_INVALID_ARG;
+    int *bad = reinterpret_cast<int *>(cnt2 + 2 * (size_t)D);  // the flag, cleared with the counts
 
     int bits_t = bits_for((uint64_t)(D - 1));
     if (bits_t < 1) bits_t = 1;
     // the scratch keeps the previous call's contents: clear the flag and the counters
-    if (cudaMemsetAsync(bad, 0, sizeof(int), s) != cudaSuccess) return SIVF_ERR_CUDA;
-    if (cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * 2 * (size_t)D, s) != cudaSuccess) return SIVF_ERR_CUDA;
+    if (cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * (2 * (size_t)D + 1), s) != cudaSuccess) return SIVF_ERR_CUDA;
     na_check<<<grid_for(k, 256), 256, 0, s>>>(k, n_entries, coff, bad);
     na_cluster_of<<<grid_for((int64_t)k * 32, 256), 256, 0, s>>>(k, n_entries, coff, clu, bad);
     if (n_entries > 0)
@@ -173,9 +171,7 @@ extern "C" sivf_status sivf_build_inverted_file_noalloc(int32_t k, int32_t D, in
     na_lens<<<grid_for(D, 256), 256, 0, s>>>(D, cnt2, len, if_mf0);
     note_launch(n_entries > 0 ? 4 : 3);
     if (cudaGetLastError() != cudaSuccess) return SIVF_ERR_CUDA;
-    if (scan_exclusive_i64(len, if_off, D, total, ws, s) != cudaSuccess) return SIVF_ERR_CUDA;
-    if (cudaMemcpyAsync(if_off + D, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return SIVF_ERR_CUDA;
+    if (scan_exclusive_i64(len, if_off, D, if_off + D, ws, s) != cudaSuccess) return SIVF_ERR_CUDA;
     bool alt = false;
     if (radix_sort_pairs(k0, v0, k1, v1, n_entries, bits_t + 1, &alt, ws, s) != cudaSuccess) return SIVF_ERR_CUDA;
     if (n_entries > 0) {

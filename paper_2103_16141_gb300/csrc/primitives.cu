@@ -1,8 +1,11 @@
 // Device-wide primitives used by the update step: exclusive prefix sums and a
 // stable LSD radix sort of (uint32 key, uint32 value) pairs.
 //
-// Scan: reduce-then-scan in three launches (tile sums, one-CTA scan of the
-// tile sums, tile-local scan plus carry-in).
+// Scan: reduce-then-scan in two launches (tile sums, then a tile-local scan
+// whose block first adds up the sums of the earlier tiles), one when there is
+// a single tile, and three (a one-CTA scan of the tile sums in between) when
+// there are so many tiles that adding them up in every block would cost more
+// than a launch.
 // Every tile kernel loops over tiles with a grid of at most TILE_GRID blocks,
 // and when the element count is on the device it stops at the live tiles, so
 // a launch sized by a capacity costs no empty blocks.
@@ -98,14 +101,30 @@ __global__ void __launch_bounds__(1024) scan_single_block(T *data, int64_t n, co
     if (threadIdx.x == 0 && total_out) *total_out = carry;
 }
 
-template <typename T>
+// tile_sums: scanned offsets of the tiles (SUMMED = false), or their plain
+// sums, of which a block adds up those before its tile (null: one tile); the
+// block of the last tile then leaves the total.
+template <typename T, bool SUMMED>
 __global__ void __launch_bounds__(SCAN_THREADS) scan_tiles(const T *in, T *out, int64_t n, const int64_t *n_dev,
-                                                           const T *tile_offs) {
+                                                           const T *tile_sums, T *total_out) {
     __shared__ T warp_s[32];
     __shared__ T total;
     if (n_dev) n = min(*n_dev, n);  // never past the launch bound
     const int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+    if (SUMMED && tiles == 0 && blockIdx.x == 0 && threadIdx.x == 0 && total_out) *total_out = T(0);
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {  // block-uniform
+        T before = T(0);
+        if constexpr (SUMMED) {
+            if (tile_sums) {
+                T part = T(0);
+                for (int64_t q = threadIdx.x; q < t; q += SCAN_THREADS) part += tile_sums[q];
+                block_exclusive_scan<T>(part, warp_s, &total);
+                before = total;
+                __syncthreads();
+            }
+        } else {
+            before = tile_sums[t];
+        }
         const int64_t base = t * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
         T v[SCAN_ITEMS];
         T s = 0;
@@ -114,12 +133,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_tiles(const T *in, T *out, 
             v[i] = base + i < n ? in[base + i] : T(0);
             s += v[i];
         }
-        T ex = block_exclusive_scan<T>(s, warp_s, &total) + tile_offs[t];
+        T ex = block_exclusive_scan<T>(s, warp_s, &total) + before;
 #pragma unroll
         for (int i = 0; i < SCAN_ITEMS; ++i) {
             if (base + i < n) out[base + i] = ex;
             ex += v[i];
         }
+        if (SUMMED && t == tiles - 1 && threadIdx.x == 0 && total_out) *total_out = before + total;
         __syncthreads();
     }
 }
@@ -133,13 +153,23 @@ cudaError_t scan_exclusive_impl(const T *in, T *out, int64_t n, T *total, Worksp
         return cudaSuccess;
     }
     int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+    if (tiles == 1) {
+        scan_tiles<T, true><<<1, SCAN_THREADS, 0, s>>>(in, out, n, n_dev, nullptr, total);
+        note_launch();
+        return cudaGetLastError();
+    }
     size_t mark = ws.used;
     T *sums = ws.take<T>((size_t)tiles);
     if (!sums) return cudaErrorMemoryAllocation;
     scan_tile_sums<T><<<tile_grid(tiles), SCAN_THREADS, 0, s>>>(in, n, n_dev, sums);
-    scan_single_block<T><<<1, 1024, 0, s>>>(sums, tiles, n_dev, n, total);
-    scan_tiles<T><<<tile_grid(tiles), SCAN_THREADS, 0, s>>>(in, out, n, n_dev, sums);
-    note_launch(3);
+    if (tiles <= 1024) {  // at most four sums per thread
+        scan_tiles<T, true><<<tile_grid(tiles), SCAN_THREADS, 0, s>>>(in, out, n, n_dev, sums, total);
+        note_launch(2);
+    } else {
+        scan_single_block<T><<<1, 1024, 0, s>>>(sums, tiles, n_dev, n, total);
+        scan_tiles<T, false><<<tile_grid(tiles), SCAN_THREADS, 0, s>>>(in, out, n, n_dev, sums, nullptr);
+        note_launch(3);
+    }
     ws.used = mark;
     return cudaGetLastError();
 }

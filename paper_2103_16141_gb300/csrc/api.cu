@@ -71,11 +71,14 @@ sivf_status check_usable(sivf_ctx *c) {
     return SIVF_OK;
 }
 
-// Dense-row counters of the inverted file built by sivf_init / sivf_reseed
-// (later builds report them through the update step's counters).
+// Counts of the centroids and the inverted file made by sivf_init /
+// sivf_reseed (later builds report them through the update step's counters).
+// Waits for the stream.
 cudaError_t read_file_counters(sivf_ctx *c) {
     SIVF_CUDA_TRY(cudaMemcpyAsync(c->ctr_host, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, c->stream));
     SIVF_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    c->c_nnz = c->ctr_host->c_nnz;
+    c->if_nnz = c->c_nnz;
     c->dense_terms_h = c->ctr_host->dense_terms;
     c->dense_used_h = c->ctr_host->dense_used * 8;
     c->sparse_entries_h = c->ctr_host->sparse_entries;
@@ -417,7 +420,6 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
         // the first inverted file
         INIT_CUDA(reseed_dev(c, ids_dev), "seed");
     }
-    INIT_CUDA(cudaStreamSynchronize(c->stream), "sync");
     INIT_CUDA(read_file_counters(c), "counters");
     c->ws.reset();
     c->stats.centroid_nnz = c->c_nnz;
@@ -607,7 +609,6 @@ sivf_status sivf_reseed(sivf_ctx *c, const int32_t *init_ids) {
     API_CUDA(c, cudaMemcpyAsync(ids_dev, init_ids, sizeof(int32_t) * c->k, cudaMemcpyHostToDevice, c->stream), "copy");
     c->launch_base = g_launches;
     API_CUDA(c, reseed_dev(c, ids_dev), "reseed");
-    API_CUDA(c, cudaStreamSynchronize(c->stream), "sync");
     API_CUDA(c, read_file_counters(c), "counters");
     c->ws.reset();
     c->stats = sivf_stats{};

@@ -303,7 +303,6 @@ cudaError_t run_update(sivf_ctx *c);
 cudaError_t build_inverted_file(sivf_ctx *c);
 cudaError_t build_canonical_if(sivf_ctx *c);
 cudaError_t validate_csr(sivf_ctx *c, int *bad);
-cudaError_t init_centroids(sivf_ctx *c, const int32_t *init_ids_dev);
 cudaError_t set_labels_dev(sivf_ctx *c, const int32_t *src_dev);
 cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev);
 

@@ -94,16 +94,34 @@ __global__ void k_validate(int64_t N, int32_t D, int64_t nnz, const int64_t *row
     }
 }
 
-__global__ void k_seed_sizes(int32_t k, const int32_t *init_ids, const int64_t *row_ptr, int64_t *sz) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < k) {
-        int64_t d = init_ids[j];
+// State before the first assignment: no labels, no own scores, nothing added
+// to the accumulator, every cluster moving, no sums behind the centroids; and
+// the sizes of the seed rows.
+__global__ void k_reset(int64_t N, int32_t k, int32_t *labels, int32_t *labels_prev, uint32_t *own, int32_t *acc_lab,
+                        uint8_t *lam, uint8_t *lam_prev, uint8_t *moving, double *snorm, const int32_t *init_ids,
+                        const int64_t *row_ptr, int64_t *sz, DevCounters *ctr) {
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = g; i < N; i += st) {
+        labels[i] = -1;
+        labels_prev[i] = -1;
+        own[i] = OWN_INVALID;
+        if (acc_lab) acc_lab[i] = -1;
+    }
+    for (int64_t j = g; j < k; j += st) {
+        lam[j] = 0;
+        lam_prev[j] = 0;
+        moving[j] = 1;
+        snorm[j] = 0.0;
+        const int64_t d = init_ids[j];
         sz[j] = row_ptr[d + 1] - row_ptr[d];
     }
+    if (g == 0) *ctr = DevCounters{};
 }
 
+// The seed rows, one warp each; their total is left in the counters.
 __global__ void k_seed_rows(int32_t k, const int32_t *init_ids, const int64_t *row_ptr, const int32_t *idx,
-                            const float *val, const int64_t *coff, int32_t *cterm, float *cval, int32_t *cclu) {
+                            const float *val, const int64_t *coff, int32_t *cterm, float *cval, int32_t *cclu,
+                            DevCounters *ctr) {
     const int lane = threadIdx.x & 31;
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (wid >= k) return;
@@ -115,6 +133,7 @@ __global__ void k_seed_rows(int32_t k, const int32_t *init_ids, const int64_t *r
         cval[o + (h - b)] = val[h];
         cclu[o + (h - b)] = j;
     }
+    if (wid == 0 && lane == 0) ctr->c_nnz = coff[k];
 }
 
 // Replace a^[r] by src. lambda^[r] is recomputed against a^[r-1] (every
@@ -1179,31 +1198,6 @@ cudaError_t validate_csr(sivf_ctx *c, int *bad_host) {
     return cudaSuccess;
 }
 
-cudaError_t init_centroids(sivf_ctx *c, const int32_t *init_ids_dev) {
-    const int cur = c->cur;
-    int64_t *sz = c->ws.take<int64_t>((size_t)c->k + 1);
-    int64_t *total = c->ws.take<int64_t>(1);
-    if (!sz || !total) return cudaErrorMemoryAllocation;
-    k_seed_sizes<<<blocks_for(c->k), TPB, 0, c->stream>>>(c->k, init_ids_dev, c->row_ptr, sz);
-    note_launch();
-    SIVF_CUDA_TRY(scan_exclusive_i64(sz, c->coff[cur], c->k, total, c->ws, c->stream));
-    SIVF_CUDA_TRY(cudaMemcpyAsync(c->coff[cur] + c->k, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, c->stream));
-    int64_t tot = 0;
-    SIVF_CUDA_TRY(cudaMemcpyAsync(&tot, total, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
-    SIVF_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    if (tot > c->cap_c) return cudaErrorMemoryAllocation;
-    c->c_nnz = tot;
-    c->if_nnz = tot;
-    k_seed_rows<<<blocks_for((int64_t)c->k * 32), TPB, 0, c->stream>>>(c->k, init_ids_dev, c->row_ptr, c->idx,
-                                                                       c->val, c->coff[cur], c->cterm[cur],
-                                                                       c->cval[cur], c->cclu);
-    note_launch();
-    SIVF_CUDA_TRY(cudaGetLastError());
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->snorm, 0, sizeof(double) * c->k, c->stream));
-    c->ws.reset();
-    return cudaSuccess;
-}
-
 cudaError_t set_labels_dev(sivf_ctx *c, const int32_t *src) {
     // src must not live in the workspace region taken below
     int *bad = c->ws.take<int>(1);
@@ -1221,41 +1215,6 @@ cudaError_t set_labels_dev(sivf_ctx *c, const int32_t *src) {
     SIVF_CUDA_TRY(cudaGetLastError());
     if (c->iter == 0) c->iter = 1;  // first membership: every cluster is moving
     SIVF_CUDA_TRY(launch_finalize_assign(c));
-    return cudaSuccess;
-}
-
-// Restart from new seeds: no labels, no own scores, every cluster moving,
-// mu^[0] = seed rows, first inverted file.
-cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev) {
-    const int64_t N = c->N;
-    const int32_t k = c->k;
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->labels, 0xFF, sizeof(int32_t) * N, c->stream));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->labels_prev, 0xFF, sizeof(int32_t) * N, c->stream));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->own, 0xFF, sizeof(uint32_t) * N, c->stream));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->lam, 0, k, c->stream));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->lam_prev, 0, k, c->stream));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->moving, 1, k, c->stream));
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), c->stream));
-    if (c->dense) {  // no member has been added yet
-        if (c->acc_bits && c->acc_ready) {
-            k_acc_clear<<<(unsigned)std::min<int32_t>(k, 65535), TPB, 0, c->stream>>>(k, c->acc_off, c->acc_bit_off,
-                                                                                     c->acc, c->acc_bits);
-            note_launch();
-            SIVF_CUDA_TRY(cudaGetLastError());
-        } else {
-            SIVF_CUDA_TRY(cudaMemsetAsync(c->acc, 0, sizeof(int64_t) * (size_t)c->acc_total, c->stream));
-            if (c->acc_bits)
-                SIVF_CUDA_TRY(cudaMemsetAsync(c->acc_bits, 0, sizeof(uint32_t) * (size_t)c->acc_words, c->stream));
-            c->acc_ready = true;
-        }
-        SIVF_CUDA_TRY(cudaMemsetAsync(c->acc_lab, 0xFF, sizeof(int32_t) * N, c->stream));
-    }
-    c->iter = 1;  // finalize below marks every cluster moving
-    SIVF_CUDA_TRY(launch_finalize_assign(c));
-    c->iter = 0;
-    SIVF_CUDA_TRY(init_centroids(c, init_ids_dev));
-    SIVF_CUDA_TRY(build_inverted_file(c));
-    c->needs_update = false;
     return cudaSuccess;
 }
 
@@ -1377,6 +1336,48 @@ cudaError_t finish_rows(sivf_ctx *c, const double *jA, const double *jU, const i
 }
 
 }  // namespace
+
+// Restart from new seeds: no labels, no own scores, every cluster moving,
+// mu^[0] = seed rows (distinct documents, so they fit the centroid buffers),
+// first inverted file. No host synchronisation; the counts are in the counters.
+cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev) {
+    const int64_t N = c->N;
+    const int32_t k = c->k;
+    const int cur = c->cur;
+    cudaStream_t s = c->stream;
+    const size_t mark = c->ws.used;
+    int64_t *sz = c->ws.take<int64_t>((size_t)k + 1);
+    if (!sz) return cudaErrorMemoryAllocation;
+    if (c->dense) {  // no member has been added yet
+        if (c->acc_bits && c->acc_ready) {
+            k_acc_clear<<<(unsigned)std::min<int32_t>(k, 65535), TPB, 0, s>>>(k, c->acc_off, c->acc_bit_off, c->acc,
+                                                                              c->acc_bits);
+            note_launch();
+        } else {
+            SIVF_CUDA_TRY(cudaMemsetAsync(c->acc, 0, sizeof(int64_t) * (size_t)c->acc_total, s));
+            if (c->acc_bits)
+                SIVF_CUDA_TRY(cudaMemsetAsync(c->acc_bits, 0, sizeof(uint32_t) * (size_t)c->acc_words, s));
+            c->acc_ready = true;
+        }
+    }
+    k_reset<<<blocks_gs(std::max<int64_t>(N, k)), TPB, 0, s>>>(N, k, c->labels, c->labels_prev, c->own,
+                                                               c->dense ? c->acc_lab : nullptr, c->lam, c->lam_prev,
+                                                               c->moving, c->snorm, init_ids_dev, c->row_ptr, sz,
+                                                               c->ctr);
+    note_launch();
+    c->iter = 1;  // finalize below marks every cluster moving
+    SIVF_CUDA_TRY(launch_finalize_assign(c));
+    c->iter = 0;
+    SIVF_CUDA_TRY(row_offsets(c, sz, cur));
+    k_seed_rows<<<blocks_for((int64_t)k * 32), TPB, 0, s>>>(k, init_ids_dev, c->row_ptr, c->idx, c->val, c->coff[cur],
+                                                            c->cterm[cur], c->cval[cur], c->cclu, c->ctr);
+    note_launch();
+    SIVF_CUDA_TRY(cudaGetLastError());
+    SIVF_CUDA_TRY(build_inverted_file(c));
+    c->ws.used = mark;
+    c->needs_update = false;
+    return cudaSuccess;
+}
 
 // Update step with the dense accumulator (u1: member counts only; u2-u4 as
 // above; u5 as in the sort form).

@@ -53,8 +53,7 @@ void free_all(sivf_ctx *c) {
                     c->ctr, c->obj_dev, c->ws.base, c->inst_obj, c->inst_k, c->mov_beg, c->clu_koff,
                     c->inst_changed, c->own_row_ptr, c->own_idx, c->own_val, c->clu_doff,
                     c->loop_dev, c->done_dev, c->objf_dev, c->grho, c->acc, c->acc_off, c->acc_lab, c->acc_bits, c->acc_bit_off,
-                    c->clu_pos, c->pos_clu, c->dense_val, c->inst_d, c->dense_thr,
-                    c->heavy_ids, c->light_ids};
+                    c->clu_pos, c->pos_clu, c->dense_val, c->inst_d, c->dense_thr};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     destroy_loop_graph(c);
@@ -218,8 +217,6 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     const int64_t capc = c->cap_c;
     const int32_t ni = c->n_inst;
     INIT_CUDA(dmalloc(c, &c->labels, N), "alloc");
-    INIT_CUDA(dmalloc(c, &c->heavy_ids, N), "alloc");
-    INIT_CUDA(dmalloc(c, &c->light_ids, N), "alloc");
     INIT_CUDA(dmalloc(c, &c->labels_prev, N), "alloc");
     INIT_CUDA(dmalloc(c, &c->own, N), "alloc");
     INIT_CUDA(dmalloc(c, &c->sumv, N), "alloc");
@@ -683,7 +680,8 @@ sivf_status finish_assign(sivf_ctx *c, int64_t *n_changed, float ms) {
     st.rescore_cands = (int64_t)h.rescore_cands;
     st.dense_entries = (int64_t)h.dense_entries;
     st.dense_postings = (int64_t)h.dense_postings;
-    st.light_objects = (int64_t)h.n_light;
+    const bool light_on = (c->cfg.icp == 1 || c->cfg.icp == 3) && c->cfg.light_max_moving >= 0;
+    st.light_objects = (int64_t)h.n_light + (light_on ? (int64_t)h.n_done : 0);
     if (ms >= 0.f) st.ms_assign = ms;
     if (n_changed) *n_changed = st.changed;
     return SIVF_OK;

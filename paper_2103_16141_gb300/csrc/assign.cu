@@ -78,8 +78,10 @@ struct AssignParams {
     const int32_t *clu_pos;    // cluster (global id) -> scan position in its instance
     const int32_t *pos_clu;    // instance cluster offset + scan position -> local id
     const void *dense;         // dense rows: u16 (BF16, FP16 x 2^14) or f32
-    const int32_t *heavy_ids;  // objects of the CTA-per-object kernel (ctr->n_heavy of them)
-    const int32_t *light_ids;  // objects of the warp-per-object kernel (ctr->n_light of them)
+    // objects to score, {object, first entry, entries | filtered << 31, previous
+    // label}: those of the CTA kernel from the front (ctr->n_heavy), those of
+    // the warp kernel from the back (ctr->n_light; entry N - 1 - j)
+    int4 *objs;
     int chunk;                 // terms staged per chunk by the CTA kernel (its block size)
     int stream_sparse;         // 1: the sparse scan copy exceeds L2; its loads are streamed
     uint32_t *grho;            // global score vectors, one kmax slab per CTA (global score-buffer variant)
@@ -519,6 +521,16 @@ __device__ __forceinline__ void dense_tile(const AssignParams &P, uint32_t *rho,
     }
 }
 
+// instance of object i: largest m with inst_obj[m] <= i
+__device__ __forceinline__ int instance_of(const AssignParams &P, int64_t i) {
+    int lo = 0, hi = P.n_inst - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (P.inst_obj[mid] <= i) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
 // Sparse phase: the rows [w0, w1) of 32 quads, by one warp. The quads of the
 // chunk's segments lie end to end; a lane finds the segment of its first quad
 // by bisection and walks forward from there. Several rows are in flight.
@@ -595,7 +607,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
     int2 *s_dense = reinterpret_cast<int2 *>(s_seg + T);
     uint32_t *s_lam = reinterpret_cast<uint32_t *>(s_dense + T);  // CB: lambda^[r-1] bits of all clusters
     __shared__ int2 warp_i2[NW];
-    __shared__ long long s_obj;
+    __shared__ int4 s_next;  // the object after the current one (x = -1: none)
     __shared__ uint32_t warp_b[NW], warp_s[NW];
     __shared__ double warp_d[NW];
     __shared__ int warp_j[NW];
@@ -619,41 +631,33 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
     unsigned long long c_post_obj = 0, c_dpost = 0;  // per thread
     __syncthreads();
 
-    const long long n_obj = (long long)P.ctr->n_heavy;
+    // Fetching an object is a chain of dependent loads. Its first links (the
+    // work counter, the object's entry) run one object ahead: thread 0 asks the
+    // counter when an object starts and reads the next object's entry behind
+    // the object's first dense and sparse work, and its row is then asked into
+    // L2, so that an object starts with its terms' loads.
+    const unsigned n_obj = P.ctr->n_heavy;
+    if (tid == 0) {
+        const unsigned n = atomicAdd(&P.ctr->work, 1u);
+        s_next = n < n_obj ? P.objs[n] : make_int4(-1, 0, 0, 0);
+    }
     for (;;) {
-        if (tid == 0) s_obj = (long long)atomicAdd(&P.ctr->work, 1ull);
         __syncthreads();
-        if (s_obj >= n_obj) break;
-        const int i = P.heavy_ids[s_obj];
+        const int4 ob = s_next;
+        if (ob.x < 0) break;
+        unsigned ahead = 0;
+        if (tid == 0) ahead = atomicAdd(&P.ctr->work, 1u);
+        const int i = ob.x;
+        const int rb = ob.y, re = ob.y + (ob.z & 0x7FFFFFFF);
+        const bool filt = ob.z < 0;
+        const int32_t a_prev = ob.w;  // global id, -1 before the first assignment
         if constexpr (!GRHO)  // cleared while the object's first loads are in flight
             for (int p = 4 * tid; p < dirty; p += 4 * T) rho_st4<GRHO>(rho + p, make_uint4(0u, 0u, 0u, 0u));
-        int rb, re;  // nnz < 2^31
-        {
-            int64_t b = P.row_ptr[i], e = P.row_ptr[i + 1];
-            if (P.checked && (b < 0 || e < b || e > P.nnz)) {
-                // the borrowed CSR changed since it was validated: record it, read nothing
-                if (tid == 0) atomicOr(&P.ctr->error, 1ull);
-                b = e = 0;
-            }
-            rb = (int)b;
-            re = (int)e;
-        }
-        // instance of object i: largest m with inst_obj[m] <= i
-        int inst = 0;
-        {
-            int lo = 0, hi = P.n_inst - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (P.inst_obj[mid] <= i) lo = mid; else hi = mid - 1;
-            }
-            inst = lo;
-        }
+        const int inst = instance_of(P, i);
         const int k_off = P.inst_k[inst];
         const int km = P.inst_k[inst + 1] - k_off;
-        const int32_t a_prev = P.labels_prev[i];  // global id, -1 before the first assignment
         const int a_loc = a_prev >= 0 ? a_prev - k_off : -1;
         const uint32_t own_q = P.own[i];
-        const bool filt = P.icp && a_prev >= 0 && own_q != OWN_INVALID && P.lam_prev[a_prev] != 0;
         const int mb = P.mov_beg[inst];
         const int n_mov_inst = P.mov_beg[inst + 1] - mb;
         // score index of the m-th moving cluster, and cluster id of a score index
@@ -663,19 +667,6 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         // the instance's clusters are moving; decided after the front scan
         bool relax = P.icp == 3 && !filt && a_prev >= 0 && own_q != OWN_INVALID && 2 * n_mov_inst <= km;
         bool wasted = false;  // a relaxed front scan that was rejected
-        dirty = 0;
-        if (!CB && filt && n_mov_inst == 0) {
-            // an invariant cluster in an instance with no moving cluster (it
-            // has converged; only batches run on): the only candidate is the
-            // own cluster and every front is empty, so the label and the own
-            // score stay as they are
-            if (tid == 0) {
-                P.labels[i] = a_prev;
-                s_cnt[0] += 1;
-            }
-            __syncthreads();
-            continue;
-        }
         // rho[id] += q; under CB a filtered object skips invariant centroids
         const bool cbf = CB && filt;
         auto add = [&](int id, float prod) {
@@ -765,6 +756,8 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
                     if (step == 0) __syncthreads();
                 }
             }
+            if (tid == 0 && pass == 0 && cb == rb)
+                s_next = ahead < n_obj ? P.objs[ahead] : make_int4(-1, 0, 0, 0);
             __syncthreads();
         }
         if (!relax) break;
@@ -792,6 +785,15 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
         }
         const bool sub = filt || relax;  // candidates: the moving clusters (plus the carried own one if filt)
         const int n_mov = sub ? n_mov_inst : 0;
+
+        if (tid < 8) {  // the next object's first 256 terms and values
+            const int4 nx = s_next;
+            const int e = nx.y + 32 * tid;
+            if (nx.x >= 0 && 32 * tid < (nx.z & 0x7FFFFFFF)) {
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(P.idx + e));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(P.val + e));
+            }
+        }
 
         // ---- argmax over the candidates (Algorithm 4, lines 14-16) ----
         // The two largest scores, without ids: an object whose gap is clear of
@@ -947,7 +949,6 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
                 finish(bj, (filt && bj == a_loc) ? own_q : rho_ld<GRHO>(rho + (CB ? bj : slot(P.clu_pos[k_off + bj]))));
             }
         }
-        __syncthreads();
     }
 
     // every thread staged a share of the terms: sum the posting counts
@@ -995,16 +996,6 @@ constexpr int LIGHT_SMEM = LIGHT_WARPS * (LIGHT_MAX * 4 + LIGHT_TERMS * 8);
 static_assert(LIGHT_MAX % 8 == 0, "vector accesses of a slice");
 static_assert(4 * (LIGHT_SMEM + 1024) <= 228 * 1024, "four CTAs on an SM");
 
-// instance of object i: largest m with inst_obj[m] <= i
-__device__ __forceinline__ int instance_of(const AssignParams &P, int64_t i) {
-    int lo = 0, hi = P.n_inst - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (P.inst_obj[mid] <= i) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
 // Start of a step: a^[r-1] <- a^[r], lambda^[r-1] <- lambda^[r] (copies keep
 // every buffer address fixed from one iteration to the next), the moving flags
 // and the counters cleared; the moving count of lambda^[r-1] is kept beside
@@ -1032,23 +1023,40 @@ __global__ void k_begin(int64_t N, int32_t k, int32_t n_inst, const int32_t *lab
 // Objects into the two lists: filtered objects of an instance with at most
 // light_max moving clusters to the light list, every other object to the
 // heavy list (warp-aggregated appends; the order inside a list changes no
-// result, every object is scored on its own).
-__global__ void k_classify(AssignParams P, int light_max, int32_t *heavy_ids, int32_t *light_ids) {
+// result, every object is scored on its own). A filtered object of an instance
+// with no moving cluster (a batch's converged instance) goes to neither: its
+// own cluster is the only candidate and every front is empty, so its label and
+// own score stay as they are. IVF-CBICP still walks its lists. In checked mode
+// the row offsets are checked here, before anything is read through them.
+__global__ void k_classify(AssignParams P, int light_max) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    unsigned n_done = 0;
     for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < P.N; i0 += stride) {
         const int64_t i = i0 + lane;
         const bool valid = i < P.N;
-        bool light = false;
-        if (valid && light_max > 0) {
-            const int32_t a = P.labels_prev[i];
-            if (a >= 0 && P.own[i] != OWN_INVALID && P.lam_prev[a] != 0) {
-                const int m = instance_of(P, i);
-                light = P.mov_beg[m + 1] - P.mov_beg[m] <= light_max;
+        bool light = false, done = false;
+        int4 e = make_int4(0, 0, 0, 0);
+        if (valid) {
+            int64_t b = P.row_ptr[i], z = P.row_ptr[i + 1];
+            if (P.checked && (b < 0 || z < b || z > P.nnz)) {
+                // the borrowed CSR changed since it was validated: record it, read nothing
+                atomicOr(&P.ctr->error, 1ull);
+                b = z = 0;
             }
+            const int32_t a = P.labels_prev[i];
+            const bool filt = P.icp && a >= 0 && P.own[i] != OWN_INVALID && P.lam_prev[a] != 0;
+            if (filt && P.icp != 2) {
+                const int m = instance_of(P, i);
+                const int n_mov = P.mov_beg[m + 1] - P.mov_beg[m];
+                done = n_mov == 0;
+                light = !done && n_mov <= light_max;
+            }
+            e = make_int4((int)i, (int)b, (int)(z - b) | (filt ? (int)0x80000000 : 0), a);
         }
         const unsigned ml = __ballot_sync(0xffffffffu, valid && light);
-        const unsigned mh = __ballot_sync(0xffffffffu, valid && !light);
+        const unsigned mh = __ballot_sync(0xffffffffu, valid && !light && !done);
+        n_done += __popc(__ballot_sync(0xffffffffu, done));
         unsigned bl = 0, bh = 0;
         if (lane == 0) {
             if (ml) bl = atomicAdd(&P.ctr->n_light, (unsigned)__popc(ml));
@@ -1057,9 +1065,13 @@ __global__ void k_classify(AssignParams P, int light_max, int32_t *heavy_ids, in
         bl = __shfl_sync(0xffffffffu, bl, 0);
         bh = __shfl_sync(0xffffffffu, bh, 0);
         const unsigned below = (1u << lane) - 1u;
-        if (!valid) continue;
-        if (light) light_ids[bl + __popc(ml & below)] = (int32_t)i;
-        else heavy_ids[bh + __popc(mh & below)] = (int32_t)i;
+        if (!valid || done) continue;
+        if (light) P.objs[P.N - 1 - (int64_t)(bl + __popc(ml & below))] = e;
+        else P.objs[bh + __popc(mh & below)] = e;
+    }
+    if (lane == 0 && n_done) {
+        atomicAdd(&P.ctr->n_done, n_done);
+        atomicAdd(&P.ctr->filtered, (unsigned long long)n_done);
     }
 }
 
@@ -1156,24 +1168,15 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
     unsigned long long c_filt = 0, c_sim = 0, c_chg = 0, c_resc = 0, c_cand = 0, c_dent = 0;
     unsigned long long c_post = 0, c_dpost = 0;  // every lane
     const unsigned n_obj = P.ctr->n_light;
-    auto bounds = [&](int i, int &rb, int &re) {
-        int64_t b = P.row_ptr[i], e = P.row_ptr[i + 1];
-        if (P.checked && (b < 0 || e < b || e > P.nnz)) {
-            if (lane == 0) atomicOr(&P.ctr->error, 1ull);
-            b = e = 0;
-        }
-        rb = (int)b;
-        re = (int)e;
-    };
     unsigned li = 0;
     if (lane == 0) li = atomicAdd(&P.ctr->work_light, 1u);
     li = __shfl_sync(FULL, li, 0);
-    int i = li < n_obj ? P.light_ids[li] : -1;
-    int rb = 0, re = 0;
-    if (i >= 0) bounds(i, rb, re);
-    while (i >= 0) {
+    const int4 none = make_int4(-1, 0, 0, 0);
+    int4 ob = li < n_obj ? P.objs[P.N - 1 - (int64_t)li] : none;
+    while (ob.x >= 0) {
         if (lane == 0) li = atomicAdd(&P.ctr->work_light, 1u);
-        const int32_t a_prev = P.labels_prev[i];
+        const int i = ob.x, rb = ob.y, re = ob.y + (ob.z & 0x7FFFFFFF);
+        const int32_t a_prev = ob.w;
         const uint32_t own_q = P.own[i];
         const int inst = instance_of(P, i);
         const int k_off = P.inst_k[inst];
@@ -1184,155 +1187,144 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
             ++c_filt;
             c_sim += (unsigned long long)n_mov;
         }
-        int i_next = -1;
-        if (n_mov == 0) {  // the own cluster is the only candidate: label and own score stay
-            if (lane == 0) P.labels[i] = a_prev;
-        } else {
-            const int n8 = (n_mov + 7) & ~7;
-            for (int p = 4 * lane; p < n8; p += 128) rho_st4<false>(rho + p, make_uint4(0u, 0u, 0u, 0u));
-            __syncwarp();
-            for (int cb = rb; cb < re; cb += P.chunk) {
-                const int ce = min(re, cb + P.chunk);
-                // positions 256 at a time; a chunk of more terms than are staged
-                // at once is staged again for every 256
-                int nd = 0;
-                for (int base = 0; base < n_mov; base += 256) {
-                    constexpr int W = PREC == SIVF_FP32 ? 4 : 8, HALF = PREC == SIVF_FP32 ? 128 : 4;
-                    constexpr int U = PREC == SIVF_FP32 ? 2 : 4;
-                    const int p = base + W * lane;
-                    const bool in = p < n_mov, second = p + HALF < n_mov;
-                    const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * (PREC == SIVF_FP32 ? 4 : 2);
-                    float acc[8];
+        const int n8 = (n_mov + 7) & ~7;
+        for (int p = 4 * lane; p < n8; p += 128) rho_st4<false>(rho + p, make_uint4(0u, 0u, 0u, 0u));
+        __syncwarp();
+        for (int cb = rb; cb < re; cb += P.chunk) {
+            const int ce = min(re, cb + P.chunk);
+            // positions 256 at a time; a chunk of more terms than are staged
+            // at once is staged again for every 256
+            int nd = 0;
+            for (int base = 0; base < n_mov; base += 256) {
+                constexpr int W = PREC == SIVF_FP32 ? 4 : 8, HALF = PREC == SIVF_FP32 ? 128 : 4;
+                constexpr int U = PREC == SIVF_FP32 ? 2 : 4;
+                const int p = base + W * lane;
+                const bool in = p < n_mov, second = p + HALF < n_mov;
+                const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * (PREC == SIVF_FP32 ? 4 : 2);
+                float acc[8];
 #pragma unroll
-                    for (int m = 0; m < 8; ++m) acc[m] = 0.f;
-                    for (int s0 = cb; s0 < ce; s0 += LIGHT_TERMS) {
-                        if (base == 0 || ce - cb > LIGHT_TERMS)
-                            nd = light_stage<PREC, CID16>(P, rho, dn, s0, ce, lane, base == 0, c_post, c_dpost);
-                        if (base == 0 && lane == 0) c_dent += (unsigned long long)nd * (unsigned long long)n_mov;
-                        if (in) {
-                            int d = 0;
-                            for (; d + U <= nd; d += U) {
-                                Raw8<PREC> r[U];
-                                float vs[U];
+                for (int m = 0; m < 8; ++m) acc[m] = 0.f;
+                for (int s0 = cb; s0 < ce; s0 += LIGHT_TERMS) {
+                    if (base == 0 || ce - cb > LIGHT_TERMS)
+                        nd = light_stage<PREC, CID16>(P, rho, dn, s0, ce, lane, base == 0, c_post, c_dpost);
+                    if (base == 0 && lane == 0) c_dent += (unsigned long long)nd * (unsigned long long)n_mov;
+                    if (in) {
+                        int d = 0;
+                        for (; d + U <= nd; d += U) {
+                            Raw8<PREC> r[U];
+                            float vs[U];
 #pragma unroll
-                                for (int q = 0; q < U; ++q) {
-                                    const int2 x = dn[d + q];
-                                    r[q] = load_raw8<PREC>(e0, x.x, HALF, second);
-                                    vs[q] = __int_as_float(x.y);
-                                }
-#pragma unroll
-                                for (int q = 0; q < U; ++q) fma_raw8<PREC>(r[q], vs[q], acc);
+                            for (int q = 0; q < U; ++q) {
+                                const int2 x = dn[d + q];
+                                r[q] = load_raw8<PREC>(e0, x.x, HALF, second);
+                                vs[q] = __int_as_float(x.y);
                             }
-                            for (; d < nd; ++d) {
-                                const int2 x = dn[d];
-                                fma_raw8<PREC>(load_raw8<PREC>(e0, x.x, HALF, second), __int_as_float(x.y), acc);
-                            }
+#pragma unroll
+                            for (int q = 0; q < U; ++q) fma_raw8<PREC>(r[q], vs[q], acc);
                         }
-                        __syncwarp();
+                        for (; d < nd; ++d) {
+                            const int2 x = dn[d];
+                            fma_raw8<PREC>(load_raw8<PREC>(e0, x.x, HALF, second), __int_as_float(x.y), acc);
+                        }
                     }
-                    if (in) rho_put4<false>(rho, p, acc, false);  // LIGHT_MAX is a multiple of 8: stays in the slice
-                    if (second) rho_put4<false>(rho, p + HALF, acc + 4, false);
+                    __syncwarp();
                 }
-                __syncwarp();
+                if (in) rho_put4<false>(rho, p, acc, false);  // LIGHT_MAX is a multiple of 8: stays in the slice
+                if (second) rho_put4<false>(rho, p + HALF, acc + 4, false);
             }
-            li = __shfl_sync(FULL, li, 0);
-            if (li < n_obj) i_next = P.light_ids[li];
-            // argmax over the moving clusters plus the own cluster (carried
-            // score), as in the CTA kernel
-            auto id_at = [&](int p) { return P.pos_clu[k_off + p]; };
-            uint32_t bv = 0u, sv = 0u;
+            __syncwarp();
+        }
+        li = __shfl_sync(FULL, li, 0);
+        ob = li < n_obj ? P.objs[P.N - 1 - (int64_t)li] : none;
+        // argmax over the moving clusters plus the own cluster (carried
+        // score), as in the CTA kernel
+        auto id_at = [&](int p) { return P.pos_clu[k_off + p]; };
+        uint32_t bv = 0u, sv = 0u;
+        for (int p = 4 * lane; (p & ~7) < n_mov; p += 128) {
+            const uint4 q = rho_ld4<false>(rho + p);
+            if (score_slot(p) < n_mov) top2_add(bv, sv, q.x);
+            if (score_slot(p + 1) < n_mov) top2_add(bv, sv, q.y);
+            if (score_slot(p + 2) < n_mov) top2_add(bv, sv, q.z);
+            if (score_slot(p + 3) < n_mov) top2_add(bv, sv, q.w);
+        }
+        const uint32_t mine = bv;
+        warp_top2(bv, sv);
+        const uint32_t top = bv;
+        top2_add(bv, sv, own_q);
+        // the carried own score may come from a scan with other dense terms:
+        // count every term as dense
+        bool flag = bv > 0u && !clear_of_bound(bv, bv - sv, n_terms, n_terms, P.eps_f,
+                                               P.eta_q != 0.f ? P.eta_q * P.sumv[i] : 0.f);
+        uint32_t thr = 0;
+        if (flag) {  // warp-uniform: the exact form of the bound
+            const double E = error_bound((double)bv * FIX_QUANTUM, n_terms, n_terms, (double)P.sumv[i], P.eps,
+                                         P.eta);
+            flag = (double)(bv - sv) * FIX_QUANTUM <= 2.0 * E;
+            const double span = ceil(2.0 * E / FIX_QUANTUM);
+            thr = span >= (double)bv ? 0u : bv - (uint32_t)span;
+        }
+        auto finish = [&](int al, uint32_t q) {  // by the one lane that knows the label
+            const int a = k_off + al;
+            P.labels[i] = a;
+            P.own[i] = q;
+            if (a != a_prev) {
+                ++c_chg;
+                P.moving[a] = 1;
+                P.moving[a_prev] = 1;
+                if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
+            }
+        };
+        if (flag) {
+            double wbest = -1.0;
+            int wj = INT32_MAX, ncand = 0;
+            for (int base = 0; base < n_mov; base += 32) {
+                const int p = base + lane;
+                const int j = (p < n_mov && rho[score_slot(p)] >= thr) ? P.pos_clu[k_off + p] : -1;
+                unsigned bal = __ballot_sync(FULL, j >= 0);
+                while (bal) {
+                    const int src = __ffs(bal) - 1;
+                    bal &= bal - 1;
+                    const int jc = __shfl_sync(FULL, j, src);
+                    const double x = exact_score(P, rb, re, k_off + jc, lane);
+                    ++ncand;
+                    if (x > wbest || (x == wbest && jc < wj)) {
+                        wbest = x;
+                        wj = jc;
+                    }
+                }
+            }
+            if (own_q >= thr) {
+                const double x = exact_score(P, rb, re, a_prev, lane);
+                ++ncand;
+                if (x > wbest || (x == wbest && a_loc < wj)) {
+                    wbest = x;
+                    wj = a_loc;
+                }
+            }
+            if (lane == 0) {
+                ++c_resc;
+                c_cand += (unsigned long long)ncand;
+                finish(wj, wj == a_loc ? own_q : rho[score_slot(P.clu_pos[k_off + wj])]);
+            }
+        } else if (bv == 0u || own_q == bv) {
+            // all scores zero: the lowest id among the candidates; else the own
+            // cluster, which no scanned score reaches
+            if (lane == 0) finish(bv == 0u ? min(a_loc, id_at(0)) : a_loc, bv);
+        } else if (mine == top) {  // one lane: a second one would make the gap zero
             for (int p = 4 * lane; (p & ~7) < n_mov; p += 128) {
                 const uint4 q = rho_ld4<false>(rho + p);
-                if (score_slot(p) < n_mov) top2_add(bv, sv, q.x);
-                if (score_slot(p + 1) < n_mov) top2_add(bv, sv, q.y);
-                if (score_slot(p + 2) < n_mov) top2_add(bv, sv, q.z);
-                if (score_slot(p + 3) < n_mov) top2_add(bv, sv, q.w);
-            }
-            const uint32_t mine = bv;
-            warp_top2(bv, sv);
-            const uint32_t top = bv;
-            top2_add(bv, sv, own_q);
-            // the carried own score may come from a scan with other dense terms:
-            // count every term as dense
-            bool flag = bv > 0u && !clear_of_bound(bv, bv - sv, n_terms, n_terms, P.eps_f,
-                                                   P.eta_q != 0.f ? P.eta_q * P.sumv[i] : 0.f);
-            uint32_t thr = 0;
-            if (flag) {  // warp-uniform: the exact form of the bound
-                const double E = error_bound((double)bv * FIX_QUANTUM, n_terms, n_terms, (double)P.sumv[i], P.eps,
-                                             P.eta);
-                flag = (double)(bv - sv) * FIX_QUANTUM <= 2.0 * E;
-                const double span = ceil(2.0 * E / FIX_QUANTUM);
-                thr = span >= (double)bv ? 0u : bv - (uint32_t)span;
-            }
-            auto finish = [&](int al, uint32_t q) {  // by the one lane that knows the label
-                const int a = k_off + al;
-                P.labels[i] = a;
-                P.own[i] = q;
-                if (a != a_prev) {
-                    ++c_chg;
-                    P.moving[a] = 1;
-                    P.moving[a_prev] = 1;
-                    if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
-                }
-            };
-            if (flag) {
-                double wbest = -1.0;
-                int wj = INT32_MAX, ncand = 0;
-                for (int base = 0; base < n_mov; base += 32) {
-                    const int p = base + lane;
-                    const int j = (p < n_mov && rho[score_slot(p)] >= thr) ? P.pos_clu[k_off + p] : -1;
-                    unsigned bal = __ballot_sync(FULL, j >= 0);
-                    while (bal) {
-                        const int src = __ffs(bal) - 1;
-                        bal &= bal - 1;
-                        const int jc = __shfl_sync(FULL, j, src);
-                        const double x = exact_score(P, rb, re, k_off + jc, lane);
-                        ++ncand;
-                        if (x > wbest || (x == wbest && jc < wj)) {
-                            wbest = x;
-                            wj = jc;
-                        }
-                    }
-                }
-                if (own_q >= thr) {
-                    const double x = exact_score(P, rb, re, a_prev, lane);
-                    ++ncand;
-                    if (x > wbest || (x == wbest && a_loc < wj)) {
-                        wbest = x;
-                        wj = a_loc;
-                    }
-                }
-                if (lane == 0) {
-                    ++c_resc;
-                    c_cand += (unsigned long long)ncand;
-                    finish(wj, wj == a_loc ? own_q : rho[score_slot(P.clu_pos[k_off + wj])]);
-                }
-            } else if (bv == 0u || own_q == bv) {
-                // all scores zero: the lowest id among the candidates; else the own
-                // cluster, which no scanned score reaches
-                if (lane == 0) finish(bv == 0u ? min(a_loc, id_at(0)) : a_loc, bv);
-            } else if (mine == top) {  // one lane: a second one would make the gap zero
-                for (int p = 4 * lane; (p & ~7) < n_mov; p += 128) {
-                    const uint4 q = rho_ld4<false>(rho + p);
-                    int e = -1;
-                    if (q.x == top && score_slot(p) < n_mov) e = score_slot(p);
-                    if (q.y == top && score_slot(p + 1) < n_mov) e = score_slot(p + 1);
-                    if (q.z == top && score_slot(p + 2) < n_mov) e = score_slot(p + 2);
-                    if (q.w == top && score_slot(p + 3) < n_mov) e = score_slot(p + 3);
-                    if (e >= 0) {
-                        finish(id_at(e), top);
-                        break;
-                    }
+                int e = -1;
+                if (q.x == top && score_slot(p) < n_mov) e = score_slot(p);
+                if (q.y == top && score_slot(p + 1) < n_mov) e = score_slot(p + 1);
+                if (q.z == top && score_slot(p + 2) < n_mov) e = score_slot(p + 2);
+                if (q.w == top && score_slot(p + 3) < n_mov) e = score_slot(p + 3);
+                if (e >= 0) {
+                    finish(id_at(e), top);
+                    break;
                 }
             }
-            __syncwarp();
         }
-        if (n_mov == 0) {
-            li = __shfl_sync(FULL, li, 0);
-            if (li < n_obj) i_next = P.light_ids[li];
-        }
-        i = i_next;
-        if (i >= 0) bounds(i, rb, re);
+        __syncwarp();
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1521,8 +1513,11 @@ cudaError_t launch_assign(sivf_ctx *c) {
     }
     P.eps_f = (float)P.eps;                    // powers of two: exact
     P.eta_q = (float)(P.eta / FIX_QUANTUM);
-    P.heavy_ids = c->heavy_ids;
-    P.light_ids = c->light_ids;
+    // the object lists live in the step workspace, which only the update uses
+    const size_t mark = c->ws.used;
+    P.objs = c->ws.take<int4>((size_t)c->N);
+    c->ws.used = mark;
+    if (!P.objs) return cudaErrorMemoryAllocation;
     P.chunk = c->assign_threads;
     {
         const int64_t b_post = c->cfg.prec == SIVF_FP32 ? 6 : 4;
@@ -1532,7 +1527,7 @@ cudaError_t launch_assign(sivf_ctx *c) {
     const int cap = c->cfg.light_max_moving;
     const int light_max = (c->cfg.icp == 1 || c->cfg.icp == 3) && cap >= 0 ? (cap == 0 ? LIGHT_MAX : cap) : 0;
     k_classify<<<(unsigned)std::min<int64_t>((c->N + 255) / 256, (int64_t)c->num_sms * 8), 256, 0, c->stream>>>(
-        P, light_max, c->heavy_ids, c->light_ids);
+        P, light_max);
     note_launch();
     SIVF_CUDA_TRY(cudaGetLastError());
     if (light_max > 0) {

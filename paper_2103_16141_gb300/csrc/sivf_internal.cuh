@@ -45,8 +45,10 @@
 //                                        q(x) = ceil(x 2^shift) of the current members,
 //                                        kept across iterations; acc_bits: a bit per entry
 //                                        that may be non-zero (1/64 of acc)
-//   object lists          heavy_ids, light_ids int32[N]: the objects of the CTA and the
-//                                        warp-per-object assignment kernels
+//   object lists          int4[N] in the step workspace during an assignment:
+//                                        {object, first entry, entries | filtered << 31,
+//                                        previous label}, the CTA kernel's objects from the
+//                                        front, the warp kernel's from the back
 #pragma once
 
 #include <cuda_runtime.h>
@@ -91,7 +93,7 @@ struct DevCounters {
     unsigned long long rescored;
     unsigned long long rescore_cands;
     unsigned long long n_moving;     // lambda^[r] = 0 count (written by finalize)
-    unsigned long long work;         // object work counter of the assignment kernel
+    unsigned int work, work_light;   // object work counters of the CTA and the warp kernel
     unsigned long long error;        // nonzero: device-side check failed (code)
     long long moved;                 // object non-zeros gathered by the last update
     long long c_nnz;                 // centroid non-zeros after the last update
@@ -99,8 +101,8 @@ struct DevCounters {
     unsigned long long dense_postings;  // postings of the scanned segments held in dense rows
     long long dense_terms;              // terms with a dense row (last inverted-file build)
     long long dense_used;               // dense-row entries in use / 8 (last build)
-    unsigned int work_light, pad;    // object work counter of the light (warp-per-object) kernel
     unsigned int n_heavy, n_light;   // objects in the two lists of the assignment
+    unsigned int n_done, pad;        // filtered objects of instances with no moving cluster (in neither)
     long long sparse_entries;        // entries of the sparse scan copy (last build)
     long long n_moving_prev;         // lambda^[r-1] = 0 count (written when the step begins)
 };
@@ -220,10 +222,6 @@ struct sivf_ctx {
     uint32_t *grho = nullptr; // global score vectors: grho_ctas slabs of kmax (zero between objects)
     int64_t grho_ctas = 0;
     unsigned long long launch_base = 0;  // g_launches at init / reseed
-    // object lists of the assignment: filtered objects of instances with few
-    // moving clusters take the warp-per-object kernel (light), the rest the
-    // CTA-per-object kernel (heavy)
-    int32_t *heavy_ids = nullptr, *light_ids = nullptr;
     long long sparse_entries_h = 0;  // entries of the sparse scan copy (host copy, for the L2 hint)
 
     // independent instances sharing one context: objects [inst_obj[m],

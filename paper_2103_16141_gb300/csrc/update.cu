@@ -1207,8 +1207,8 @@ __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *ct
         if (td.w >= 0) {
             const int64_t d = (int64_t)td.w * 8 + p;
             if (prec == SIVF_FP32) static_cast<float *>(dense)[d] = u;
-            else static_cast<uint16_t *>(dense)[d] = encode_lp(u, prec);
-            continue;
+            else if (prec == SIVF_FP16 || !(p & 1u)) static_cast<uint16_t *>(dense)[d] = encode_lp(u, prec);
+            continue;  // odd entries of BF16 rows: k_dense_odd
         }
         const uint32_t part = (structured && lam[j]) ? 1u : 0u;
         const int64_t pos = (int64_t)(unsigned)td.x * 4 + atomicAdd(cursor + (((uint32_t)t << 1) | part), 1u) +
@@ -1223,6 +1223,24 @@ __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *ct
         const uint16_t lp = encode_lp(u, prec);
         if (sc_pack) sc_pack[pos] = (id << 16) | (uint32_t)lp;
         else sc_lp[pos] = lp;
+    }
+}
+
+// Odd entries of the BF16 dense rows. The scan reads a word (even entry below,
+// odd entry above) as FP32 for the odd one, so the upper half is chosen such
+// that the word is the nearest to u among those with its lower half: within
+// half of the upper half's step, as rounding u to BF16 is (2^-8 relative).
+__global__ void k_dense_odd(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
+                            const float *cval, const int32_t *clu_pos, const int4 *tdesc, uint16_t *dense) {
+    const int64_t n = min(*n_dev, cap);
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t p = clu_pos[cclu[e]];
+        if (!(p & 1)) continue;
+        const int32_t row = tdesc[cterm[e]].w;
+        if (row < 0) continue;
+        uint16_t *at = dense + (int64_t)row * 8 + p;
+        const uint32_t u = max(__float_as_uint(cval[e]), 0x00800000u);  // at least the smallest normal
+        *at = (uint16_t)((u - at[-1] + 0x8000u) >> 16);
     }
 }
 
@@ -1317,6 +1335,11 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
                                                 c->clu_pos, c->tdesc, cursor, (int)c->cfg.prec, c->dense_val,
                                                 c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp);
     note_launch();
+    if (dense && c->cfg.prec == SIVF_BF16) {
+        k_dense_odd<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, c->cterm[cur], c->cclu, c->cval[cur], c->clu_pos,
+                                                   c->tdesc, static_cast<uint16_t *>(c->dense_val));
+        note_launch();
+    }
     SIVF_CUDA_TRY(cudaGetLastError());
     ws.used = mark;
     return cudaSuccess;

@@ -744,14 +744,14 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
             nd_obj += n_dense;
             if (tid == 0) s_cnt[5] += (unsigned long long)n_dense * (unsigned long long)npos;
             // Every warp has its share of the sparse rows and of the dense
-            // tiles. The sparse rows wait for the shared-memory atomics, the
-            // tiles for L2: even warps start with the one, odd warps with the
-            // other, so that a CTA has both under way (all warps in the same
-            // phase, with a barrier between the two, took 54.3 instead of
-            // 49.6 ms per assignment of 500,000 documents at k = 20,000, BF16;
-            // k = 10,000 23.3 and 20.8, k = 3001 FP16 2.13 and 1.88).
-            // A global score vector takes plain accesses, so its dense tiles
-            // come first, with a barrier behind them.
+            // tiles and goes from one to the other without a barrier: the rows
+            // wait for the shared-memory atomics, the tiles for L2, and warps
+            // drift apart (with a barrier between the two an assignment of
+            // 500,000 documents at k = 20,000, BF16, took 54.3 instead of 49.6
+            // ms, k = 10,000 23.3 and 20.8, k = 3001 FP16 2.13 and 1.88; which
+            // of the two a warp starts with made no difference). A global
+            // score vector takes plain accesses, so its dense tiles come
+            // first, with a barrier behind them.
             const int rows = (n_quads + 31) >> 5;
             const int per_warp = (rows + NW - 1) / NW;
             const int w0 = warp * per_warp, w1 = min(rows, w0 + per_warp);

@@ -347,14 +347,14 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
         // per-cluster arrays; u2 per tuple (sort mode only): 4 sort arrays,
         // term, rank, value, sorted value, 64-bit key, piece sum, unique term
         // and sum (60 B)
-        size_t phase1 = 4 * (size_t)N * 4 + 2 * n8 + 14 * k8 + (c->dense ? 0 : 64 * ((size_t)nnz + 1)) + 32 * 4096;
+        size_t phase1 = 4 * (size_t)N * 4 + 2 * n8 + 14 * k8 + (c->dense ? 0 : 60 * ((size_t)nnz + 1)) + 32 * 4096;
         // u5: sort arrays (16 B x entries), per-term counts, lengths, dense widths
         // and offsets (40 B x terms), the dense-length histogram
         // (per-term counts with the first, all of the second's arrays without it)
         size_t phase2 = std::max(16 * ((size_t)capc + 1) + 8 * ((size_t)D + 1), 40 * ((size_t)D + 1)) + 16 * 4096;
         size_t ws = phase1 > phase2 ? phase1 : phase2;
         size_t maxn = (size_t)(capc > N ? capc : N);
-        ws += (maxn / 4096 + 2) * 1024 * 4 + (maxn / 2048 + 2) * 16 + 64 * 256 + (1 << 20);
+        ws += (maxn / 4096 + 2) * 1024 * 4 + (maxn / 2048 + 2) * 16 + 64 * 256 + (1 << 19);
         c->ws_bytes = ws;
         INIT_CUDA(dmalloc(c, reinterpret_cast<char **>(&c->ws.base), ws), "alloc workspace");
         c->ws.cap = ws;

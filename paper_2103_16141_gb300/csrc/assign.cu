@@ -1007,7 +1007,7 @@ constexpr int LIGHT_MAX = 1472;   // the largest moving count of a light object
 constexpr int LIGHT_TERMS = 128;  // terms staged at once
 constexpr int LIGHT_SMEM = LIGHT_WARPS * (LIGHT_MAX * 4 + LIGHT_TERMS * 8);
 static_assert(LIGHT_MAX % 8 == 0, "vector accesses of a slice");
-static_assert(4 * (LIGHT_SMEM + 1024) <= 228 * 1024, "four CTAs on an SM");
+static_assert(4 * (LIGHT_SMEM + 1024 + 64) <= 228 * 1024, "four CTAs on an SM");
 
 // Start of a step: a^[r-1] <- a^[r], lambda^[r-1] <- lambda^[r] (copies keep
 // every buffer address fixed from one iteration to the next), the moving flags
@@ -1177,8 +1177,12 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
     constexpr unsigned FULL = 0xffffffffu;
     uint32_t *rho = smem + w * LIGHT_MAX;
     int2 *dn = reinterpret_cast<int2 *>(smem + LIGHT_WARPS * LIGHT_MAX) + w * LIGHT_TERMS;
-    // counters kept by lane 0: filtered, sim-calcs, re-scored, candidates, dense entries; any lane: changed
-    unsigned long long c_filt = 0, c_sim = 0, c_chg = 0, c_resc = 0, c_cand = 0, c_dent = 0;
+    // per-CTA counters in shared memory, which leaves the registers to the row
+    // loads: filtered, sim-calcs, changed, re-scored, candidates, dense entries
+    __shared__ unsigned long long s_cnt[6];
+    if (threadIdx.x < 6) s_cnt[threadIdx.x] = 0ull;
+    __syncthreads();
+    auto count = [&](int what, unsigned long long n) { atomicAdd(&s_cnt[what], n); };
     unsigned long long c_post = 0, c_dpost = 0;  // every lane
     const unsigned n_obj = P.ctr->n_light;
     unsigned li = 0;
@@ -1197,8 +1201,8 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
         const int a_loc = a_prev - k_off;
         const int n_terms = re - rb;
         if (lane == 0) {
-            ++c_filt;
-            c_sim += (unsigned long long)n_mov;
+            count(0, 1);
+            count(1, (unsigned long long)n_mov);
         }
         const int n8 = (n_mov + 7) & ~7;
         for (int p = 4 * lane; p < n8; p += 128) rho_st4<false>(rho + p, make_uint4(0u, 0u, 0u, 0u));
@@ -1210,7 +1214,7 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
             int nd = 0;
             for (int base = 0; base < n_mov; base += 256) {
                 constexpr int W = PREC == SIVF_FP32 ? 4 : 8, HALF = PREC == SIVF_FP32 ? 128 : 4;
-                constexpr int U = PREC == SIVF_FP32 ? 2 : 4;
+                constexpr int U = PREC == SIVF_FP32 ? 4 : 8;
                 const int p = base + W * lane;
                 const bool in = p < n_mov, second = p + HALF < n_mov;
                 const char *e0 = static_cast<const char *>(P.dense) + (size_t)p * (PREC == SIVF_FP32 ? 4 : 2);
@@ -1220,7 +1224,7 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
                 for (int s0 = cb; s0 < ce; s0 += LIGHT_TERMS) {
                     if (base == 0 || ce - cb > LIGHT_TERMS)
                         nd = light_stage<PREC, CID16>(P, rho, dn, s0, ce, lane, base == 0, c_post, c_dpost);
-                    if (base == 0 && lane == 0) c_dent += (unsigned long long)nd * (unsigned long long)n_mov;
+                    if (base == 0 && lane == 0) count(5, (unsigned long long)nd * (unsigned long long)n_mov);
                     if (in) {
                         int d = 0;
                         for (; d + U <= nd; d += U) {
@@ -1281,7 +1285,7 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
             P.labels[i] = a;
             P.own[i] = q;
             if (a != a_prev) {
-                ++c_chg;
+                count(2, 1);
                 P.moving[a] = 1;
                 P.moving[a_prev] = 1;
                 if (P.n_inst > 1) atomicAdd(P.inst_changed + inst, 1ull);
@@ -1315,8 +1319,8 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
                 }
             }
             if (lane == 0) {
-                ++c_resc;
-                c_cand += (unsigned long long)ncand;
+                count(3, 1);
+                count(4, (unsigned long long)ncand);
                 finish(wj, wj == a_loc ? own_q : rho[score_slot(P.clu_pos[k_off + wj])]);
             }
         } else if (bv == 0u || own_q == bv) {
@@ -1343,19 +1347,21 @@ __global__ void __launch_bounds__(LIGHT_WARPS * 32, 4) assign_light_kernel(Assig
     for (int o = 16; o > 0; o >>= 1) {
         c_post += __shfl_xor_sync(FULL, c_post, o);
         c_dpost += __shfl_xor_sync(FULL, c_dpost, o);
-        c_chg += __shfl_xor_sync(FULL, c_chg, o);
     }
     if (lane == 0) {
         if (c_post) atomicAdd(&P.ctr->postings, c_post);
         if (c_dpost) atomicAdd(&P.ctr->dense_postings, c_dpost);
-        if (c_filt) atomicAdd(&P.ctr->filtered, c_filt);
-        if (c_sim) atomicAdd(&P.ctr->simcalc, c_sim);
-        if (c_chg) atomicAdd(&P.ctr->changed, c_chg);
-        if (c_resc) {
-            atomicAdd(&P.ctr->rescored, c_resc);
-            atomicAdd(&P.ctr->rescore_cands, c_cand);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(&P.ctr->filtered, s_cnt[0]);
+        atomicAdd(&P.ctr->simcalc, s_cnt[1]);
+        atomicAdd(&P.ctr->changed, s_cnt[2]);
+        if (s_cnt[3]) {
+            atomicAdd(&P.ctr->rescored, s_cnt[3]);
+            atomicAdd(&P.ctr->rescore_cands, s_cnt[4]);
         }
-        if (c_dent) atomicAdd(&P.ctr->dense_entries, c_dent);
+        if (s_cnt[5]) atomicAdd(&P.ctr->dense_entries, s_cnt[5]);
     }
 }
 

@@ -1,8 +1,8 @@
 // Assignment step of SIVF (Algorithm 4, Section 4.1; Algorithm 2 when the
 // ICP filter is off; Algorithm 3, IVF-CBICP, as an ablation) on sm_103a.
 //
-// One CTA scores one object at a time (persistent CTAs pull object ids from a
-// global counter); filtered objects of instances with few moving clusters
+// One CTA scores one object at a time (persistent CTAs pull objects from a
+// global counter, one ahead); filtered objects of instances with few moving clusters
 // take a warp each instead (assign_light_kernel). The k similarities rho_j
 // live in shared memory as unsigned fixed-point sums with quantum 2^-31,
 // indexed by scan position (the moving clusters first):
@@ -12,6 +12,11 @@
 //    clusters) is read with 16-byte loads; for every chunk of staged terms the
 //    dense terms' products are chained in FP32 fused multiply-adds per score
 //    position, and the chain's ceil is added once.
+// What bounds the CTA kernel: the row stream into an SM (64 bytes per clock,
+// about 20 TB/s in all). k = 1000 FP32 reads 18.9 TB/s of rows over a whole
+// assignment, k = 3001 FP16 15.1, k = 20,000 BF16 13.7, where two CTAs per SM
+// leave part of the per-object latency uncovered and the L1 data pipe (76 %)
+// and the issue slots (64 %) are busy too.
 // Integer addition is associative, so the sums do not depend on the order in
 // which threads visit postings: the filtered and unfiltered modes produce
 // identical scores, and every run is deterministic.
@@ -345,13 +350,12 @@ __device__ __forceinline__ void load_one(const AssignParams &P, size_t pos, int 
 }
 
 // Register budget: 32 resident warps per SM asked of the compiler, so a
-// thread has 64 registers whatever the block size. The dense-row phase keeps
-// 16 FP32 accumulators per thread; with 40 registers (the earlier budget of
-// 48 warps) its loop spilled. 512-thread CTAs serve large k, whose score
-// vector (80 KB at k = 20,000) admits two CTAs per SM anyway: on the
-// 8M x 140K, k = 20,000 corpus (BF16, sparse scan only) asking for three (42
-// registers) took 4.2-4.6 s per assignment, two 3.1-3.3 s, one (128
-// registers, half the warps) 5.5-5.9 s.
+// thread has 64 registers whatever the block size: a dense tile holds 8 FP32
+// accumulators and 32 registers of rows in flight, four rows of sparse quads
+// 16 to 24. 512-thread CTAs serve large k, whose score vector (80 KB at
+// k = 20,000) admits two CTAs per SM anyway. With a sparse-only scan on the
+// 8M x 140K, k = 20,000 corpus, asking for three (42 registers) took 4.2-4.6 s
+// per assignment, two 3.1-3.3 s, one (128 registers, half the warps) 5.5-5.9 s.
 #ifndef SIVF_ASSIGN_WARPS_PER_SM
 #define SIVF_ASSIGN_WARPS_PER_SM 32
 #endif

@@ -219,7 +219,7 @@ struct sivf_ctx {
     int assign_global = 0;    // 1: score vectors in global memory (grho), else shared memory
     bool light_ready = false; // the warp-per-object kernel's shared memory has been set
     bool tuned = false;       // the autotuner has picked the assignment configuration
-    uint32_t *grho = nullptr; // global score vectors: grho_ctas slabs of kmax (zero between objects)
+    uint32_t *grho = nullptr; // global score vectors: grho_ctas slabs of kmax rounded up to 8 (set anew for every object)
     int64_t grho_ctas = 0;
     unsigned long long launch_base = 0;  // g_launches at init / reseed
     long long sparse_entries_h = 0;  // entries of the sparse scan copy (host copy, for the L2 hint)

@@ -12,7 +12,7 @@
 //      history, and the result is deterministic.
 //  u3  pass 1 (k_acc_rows1): new row sizes, ||s_j|| from the exact 128-bit
 //      sum of the squared integer sums (one rounding to FP64), and the
-//      objective pieces <s_j, mu_j^[r-1]>; pass 2 (k_acc_rows2): the row
+//      objective pieces <s_j, mu_j^[r-1]> the same way; pass 2 (k_acc_rows2): the row
 //      compacted in ascending term order, u = S (2^-shift / ||s_j||) in FP32.
 //      Dividing by |C_j| first cancels exactly and is skipped.
 //  u4  invariant and empty clusters keep their centroid row (copied).
@@ -678,19 +678,47 @@ __device__ __forceinline__ void block_sum_u128(unsigned long long &hi, unsigned 
 // held up the passes of a batch for 0.26 and 0.15 ms.
 constexpr int ILP = 4;
 
+// (hi, lo) += a * b.
+__device__ __forceinline__ void add_product(unsigned long long &hi, unsigned long long &lo, unsigned long long a,
+                                            unsigned long long b) {
+    const unsigned long long p = a * b;
+    lo += p;
+    hi += __umul64hi(a, b) + (lo < p ? 1ull : 0ull);
+}
+
+// x in [0, 2) in units of 2^-63, rounded down: exact from 2^-40 up.
+__device__ __forceinline__ unsigned long long fixed63(float x) {
+    const uint32_t b = __float_as_uint(x), e = b >> 23;  // a subnormal comes out as 0 either way
+    const unsigned long long m = (b & 0x7fffffu) | 0x800000u;
+    return e >= 87u ? m << (e - 87u) : e > 63u ? m >> (87u - e) : 0ull;
+}
+
+// Turns of a whole row's loop (ILP * WR_THREADS entry pairs each) after which
+// the entries just read are used for the objective's product with the previous
+// row, while they are in L2: 8192 entries, 80 MB for the CTAs of the chip. After
+// the whole row, those entries came from HBM again: 1.68 against 1.13 GB read at
+// 1000 rows of 100,000 entries, 1.38 against 1.31 ms for the update. Half or
+// twice the turns make no difference of more than 1 %.
+constexpr int DOT_TURNS = 4;
+// Previous entries in flight per thread there. The loop waits for a term, then
+// for its sum; two in flight took 1.52 ms, also with fewer row loads and spills.
+constexpr int DOT_ILP = 4;
+
 // Pass 1, one CTA per cluster: size of the new row, ||s_j|| (the squared
 // integer sums added exactly in 128 bits, one rounding to FP64) and
-// <s_j, mu_j^[r-1]> in FP64 over the previous row. The row's words (row_words)
-// are left with exactly its non-zero entries' bits: bits of entries that became
-// zero are cleared where the row is read through its map, all words are written
-// where it is read whole.
+// <s_j, mu_j^[r-1]> over the previous row, whose values are taken in units of
+// 2^-63 and multiplied and added exactly in 128 bits as well: conversions and
+// products in FP64 took longer than the reads (the pass 330 us, now 273 at 1000
+// rows of 100,000 entries, 17 % non-zero). By Cauchy-Schwarz that sum stays
+// below 2^63 times 2^63. The row's words (row_words) are left with exactly its
+// non-zero entries' bits: bits of entries that became zero are cleared where the
+// row is read through its map, all words are written where it is read whole.
 // Other clusters keep their row (sizes and objective pieces as in k_write_rows).
 __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     int32_t k, const uint8_t *lam, const int64_t *cnt, const int64_t *acc_off, const int32_t *clu_doff,
     const int64_t *acc, uint32_t *bits, const int64_t *bit_off, uint32_t *scratch, int64_t avg_len, double inv_scale,
     const int64_t *coff_old, const int32_t *cterm_old, const float *cval_old, const double *snorm_old, int64_t *sz, double *snorm_new,
     double *jA, double *jU) {
-    __shared__ double sh[WR_THREADS];
     __shared__ long long shl[WR_THREADS];
     __shared__ unsigned long long sh128[2][WR_THREADS];
     const int j = blockIdx.x;
@@ -707,7 +735,34 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
         return;
     }
     const int64_t base = acc_off[j], L = acc_off[j + 1] - base;
-    long long nz = 0;
+    // <s_j, mu_j^[r-1]> over the thread's entries of the previous row (every
+    // WR_THREADS-th) whose terms lie below a bound, from where it stopped last
+    const int32_t doff = clu_doff[j];
+    unsigned long long dot_hi = 0ull, dot_lo = 0ull;
+    const uint32_t old = (uint32_t)(ce - cb);  // a row has at most 2^31 entries
+    uint32_t at = threadIdx.x;
+    auto dot_upto = [&](uint32_t bound) {
+        for (bool more = at < old; more;) {
+            uint32_t t[DOT_ILP];
+#pragma unroll
+            for (int q = 0; q < DOT_ILP; ++q)
+                t[q] = at + q * WR_THREADS < old ? (uint32_t)(cterm_old[cb + (at + q * WR_THREADS)] - doff) : ~0u;
+            long long v[DOT_ILP];
+            float u[DOT_ILP];
+#pragma unroll
+            for (int q = 0; q < DOT_ILP; ++q) {
+                v[q] = t[q] < bound ? acc[base + t[q]] : 0;
+                u[q] = t[q] < bound ? cval_old[cb + (at + q * WR_THREADS)] : 0.f;
+            }
+            more = t[DOT_ILP - 1] < bound;
+#pragma unroll
+            for (int q = 0; q < DOT_ILP; ++q) {
+                add_product(dot_hi, dot_lo, (unsigned long long)v[q], fixed63(u[q]));
+                at += t[q] < bound ? WR_THREADS : 0;
+            }
+        }
+    };
+    uint32_t own_nz = 0;  // a row has at most 2^31 entries
     // ||S||^2 of the integer sums, exactly, as a 128-bit integer: the FP64 pipe
     // of this GPU retires about one operation per clock and SM, the integer
     // pipe dozens. Entries are non-negative (sums of positive member values)
@@ -716,11 +771,8 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     unsigned long long ss_hi = 0ull, ss_lo = 0ull;
     auto take = [&](long long v) {
         if (v) {
-            ++nz;
-            const unsigned long long u = (unsigned long long)v;
-            const unsigned long long lo = u * u;
-            ss_lo += lo;
-            ss_hi += __umul64hi(u, u) + (ss_lo < lo ? 1ull : 0ull);
+            ++own_nz;
+            add_product(ss_hi, ss_lo, (unsigned long long)v, (unsigned long long)v);
         }
     };
     if (through_map(bits, ce - cb, cnt[j], avg_len, L)) {
@@ -756,47 +808,45 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     } else {
         // rows start at even entries and have even lengths: 16-byte loads
         const longlong2 *row = reinterpret_cast<const longlong2 *>(acc + base);
-        const int64_t L2 = L >> 1;
-        const int64_t nw = (L + 31) >> 5;
-        const int lane = threadIdx.x & 31;
+        constexpr unsigned FULL = 0xffffffffu, TURN = ILP * WR_THREADS;
+        const uint32_t L2 = (uint32_t)(L >> 1), nw = (uint32_t)((L + 31) >> 5), lane = threadIdx.x & 31;
         uint32_t *words = row_words(bits, bit_off, scratch, base, j);
-        for (int64_t p0 = 0; p0 < L2; p0 += ILP * WR_THREADS) {
-            const int64_t p = p0 + threadIdx.x;
+        for (uint32_t p0 = 0; p0 < L2; p0 += TURN) {
             longlong2 v[ILP];
 #pragma unroll
-            for (int q = 0; q < ILP; ++q)
-                v[q] = p + q * WR_THREADS < L2 ? row[p + q * WR_THREADS] : make_longlong2(0, 0);
+            for (int q = 0; q < ILP; ++q) {
+                const uint32_t p = p0 + q * WR_THREADS + threadIdx.x;
+                v[q] = p < L2 ? row[p] : make_longlong2(0, 0);
+            }
+            if (words) {  // a load of the warp is 64 entries, two words: lanes 2q and 2q + 1 write those of load q
+                uint32_t x = 0, y = 0;
+#pragma unroll
+                for (int q = 0; q < ILP; ++q) {
+                    const uint32_t bx = __ballot_sync(FULL, v[q].x != 0), by = __ballot_sync(FULL, v[q].y != 0);
+                    if (lane >> 1 == q) {
+                        x = bx;
+                        y = by;
+                    }
+                }
+                const uint32_t w = ((p0 + (lane >> 1) * WR_THREADS + (threadIdx.x & ~31u)) >> 4) + (lane & 1);
+                const uint32_t half = (lane & 1) << 4;
+                if (lane < 2 * ILP && w < nw) words[w] = interleave16(x >> half, y >> half);
+            }
 #pragma unroll
             for (int q = 0; q < ILP; ++q) {
                 take(v[q].x);
                 take(v[q].y);
-                if (!words) continue;
-                const uint32_t x = __ballot_sync(0xffffffffu, v[q].x != 0), y = __ballot_sync(0xffffffffu, v[q].y != 0);
-                const int64_t w = ((p + q * WR_THREADS - lane) >> 4) + lane;  // the warp's 64 entries are two words
-                if (lane < 2 && w < nw) words[w] = interleave16(x >> (16 * lane), y >> (16 * lane));
             }
+            if ((p0 / TURN) % DOT_TURNS == DOT_TURNS - 1) dot_upto(min(2 * (p0 + TURN), (uint32_t)L));
         }
     }
-    nz = block_sum_ll(nz, shl);
+    const long long nz = block_sum_ll(own_nz, shl);
     block_sum_u128(ss_hi, ss_lo, sh128);
     // the exact sum to FP64 (one rounding of each half), then the power-of-two scale
     const double nrm = sqrt(((double)ss_hi * 18446744073709551616.0 + (double)ss_lo) * (inv_scale * inv_scale));
-    double dot = 0.0;
-    const int32_t doff = clu_doff[j];
-    for (int64_t q0 = cb + threadIdx.x; q0 < ce; q0 += ILP * WR_THREADS) {
-        long long v[ILP];
-        float u[ILP];
-#pragma unroll
-        for (int q = 0; q < ILP; ++q) {
-            const int64_t at = q0 + q * WR_THREADS;
-            const bool in = at < ce;
-            v[q] = in ? acc[base + (cterm_old[at] - doff)] : 0;
-            u[q] = in ? cval_old[at] : 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < ILP; ++q) dot += (double)v[q] * (double)u[q];
-    }
-    dot = block_sum_fixed(dot, sh) * inv_scale;
+    dot_upto((uint32_t)L);
+    block_sum_u128(dot_hi, dot_lo, sh128);
+    const double dot = ((double)dot_hi * 18446744073709551616.0 + (double)dot_lo) * inv_scale * 0x1p-63;
     if (threadIdx.x == 0) {
         sz[j] = nz;
         snorm_new[j] = nrm;

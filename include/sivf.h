@@ -251,9 +251,11 @@ sivf_status sivf_get_labels(sivf_ctx *ctx, int32_t *dst, int dst_is_device);
 /*
  * sivf_set_labels — replace the labels (resume from a checkpoint, or lockstep
  * resynchronisation). src: N labels in [0, k) (DEVICE if src_is_device).
- * Clusters whose membership changes become moving; objects whose label
- * changes lose their stored own-cluster score and take the unfiltered branch
- * at the next assignment. Call sivf_update afterwards to rebuild the means.
+ * Clusters whose membership changes become moving: against a^[r-1], and
+ * against the labels of the last update where one ran since assignment r.
+ * Objects whose label changes lose their stored own-cluster score and take the
+ * unfiltered branch at the next assignment. Call sivf_update afterwards to
+ * rebuild the means.
  */
 sivf_status sivf_set_labels(sivf_ctx *ctx, const int32_t *src, int src_is_device);
 

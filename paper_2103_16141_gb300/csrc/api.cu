@@ -718,6 +718,7 @@ sivf_status finish_update(sivf_ctx *c, float ms) {
     if (ms >= 0.f) c->stats.ms_update = ms;
     c->stats.centroid_nnz = c->c_nnz;
     c->needs_update = false;
+    c->assigned = false;
     return SIVF_OK;
 }
 
@@ -793,6 +794,7 @@ sivf_status sivf_assign(sivf_ctx *c, int64_t *n_changed) {
     // the inverted file still has the lambda^[r-1] layout: the next
     // assignment needs the update that rebuilds it with lambda^[r]
     c->needs_update = true;
+    c->assigned = true;
     return SIVF_OK;
 }
 

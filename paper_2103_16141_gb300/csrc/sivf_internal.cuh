@@ -137,6 +137,7 @@ struct sivf_ctx {
 
     bool latched = false;
     bool needs_update = false;  // an assignment or set_labels since the last update
+    bool assigned = false;      // an assignment since the last update: the centroids belong to a^[r-1]
     std::string err;
     int32_t iter = 0;
     int bits_t = 0;  // bits of a term id

@@ -137,15 +137,23 @@ __global__ void k_seed_rows(int32_t k, const int32_t *init_ids, const int64_t *r
 }
 
 // Replace a^[r] by src. lambda^[r] is recomputed against a^[r-1] (every
-// cluster moving before the second assignment); an object whose label
-// changes loses its stored own-cluster score.
-__global__ void k_set_labels(int64_t N, const int32_t *src, int32_t *labels, const int32_t *labels_prev,
+// cluster moving before the second assignment), whose centroids the stored own
+// scores belong to. Where the centroids have been rebuilt since (rebuilt = 1:
+// they belong to the labels replaced here, not to a^[r-1]), a cluster that loses
+// or gains a member against those labels is moving as well: its row would
+// otherwise stay that of the replaced labels. An object whose label changes
+// loses its stored own-cluster score.
+__global__ void k_set_labels(int64_t N, const int32_t *src, int32_t *labels, const int32_t *labels_prev, int rebuilt,
                              uint32_t *own, uint8_t *moving) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t a = src[i];
-        if (labels[i] != a) {
+        const int32_t a = src[i], old = labels[i];
+        if (old != a) {
             labels[i] = a;
             own[i] = OWN_INVALID;
+            if (rebuilt) {
+                moving[a] = 1;
+                if (old >= 0) moving[old] = 1;
+            }
         }
         const int32_t prev = labels_prev[i];
         if (a != prev) {
@@ -1395,8 +1403,12 @@ cudaError_t set_labels_dev(sivf_ctx *c, const int32_t *src) {
     SIVF_CUDA_TRY(cudaMemcpyAsync(&bad_h, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     SIVF_CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (bad_h) return cudaErrorInvalidValue;
-    SIVF_CUDA_TRY(cudaMemsetAsync(c->moving, 0, c->k, c->stream));
-    k_set_labels<<<blocks_gs(c->N), TPB, 0, c->stream>>>(c->N, src, c->labels, c->labels_prev, c->own, c->moving);
+    // labels set twice without an update in between: the centroids belong to
+    // those before the first call, so its marks stay
+    const bool rebuilt = !c->assigned;
+    if (!(rebuilt && c->needs_update)) SIVF_CUDA_TRY(cudaMemsetAsync(c->moving, 0, c->k, c->stream));
+    k_set_labels<<<blocks_gs(c->N), TPB, 0, c->stream>>>(c->N, src, c->labels, c->labels_prev, rebuilt ? 1 : 0, c->own,
+                                                         c->moving);
     note_launch();
     SIVF_CUDA_TRY(cudaGetLastError());
     if (c->iter == 0) c->iter = 1;  // first membership: every cluster is moving
@@ -1567,6 +1579,7 @@ cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev) {
     SIVF_CUDA_TRY(build_inverted_file(c));
     c->ws.used = mark;
     c->needs_update = false;
+    c->assigned = false;
     return cudaSuccess;
 }
 

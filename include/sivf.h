@@ -230,6 +230,9 @@ sivf_status sivf_assign(sivf_ctx *ctx, int64_t *n_changed);
  * clusters keep their centroid; the structured inverted file is rebuilt
  * (moving centroids in front, invariant behind, ascending ids in each part).
  * Requires at least one assignment (or sivf_set_labels) since sivf_init.
+ * Errors: SIVF_ERR_OOM, context latched, when the centroids outgrow their
+ * buffers (2 nnz + 1024 entries; empty clusters keep their rows); sivf_run and
+ * sivf_batch_run report it as well.
  */
 sivf_status sivf_update(sivf_ctx *ctx);
 

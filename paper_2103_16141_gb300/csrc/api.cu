@@ -664,15 +664,25 @@ cudaError_t enqueue_update(sivf_ctx *c, bool timing) {
 
 namespace {
 
+// What the device-side checks of a step found, from the pinned mirror.
+sivf_status device_error(sivf_ctx *c) {
+    const unsigned long long e = c->ctr_host->error;
+    if (!e) return SIVF_OK;
+    c->latched = true;
+    if (e & (ERR_ROW | ERR_TERM)) {
+        c->err = (e & ERR_ROW) ? "device-side check failed in the assignment: a row offset of the CSR is out of range"
+                               : "device-side check failed in the assignment: a term of the CSR is outside [0, D)";
+        return SIVF_ERR_STATE;
+    }
+    c->err = "the centroids outgrew their buffers (more than 2 nnz + 1024 entries)";
+    return SIVF_ERR_OOM;
+}
+
 // Host bookkeeping after an assignment whose counters are in the pinned mirrors.
 sivf_status finish_assign(sivf_ctx *c, int64_t *n_changed, float ms) {
     const DevCounters &h = *c->ctr_host;
-    if (h.error) {
-        c->latched = true;
-        c->err = (h.error & 1ull) ? "device-side check failed in the assignment: a row offset of the CSR is out of range"
-                                  : "device-side check failed in the assignment: a term of the CSR is outside [0, D)";
-        return SIVF_ERR_STATE;
-    }
+    const sivf_status e = device_error(c);
+    if (e != SIVF_OK) return e;
     for (int32_t m = 0; m < c->n_inst; ++m)
         c->inst_changed_h[(size_t)m] = c->n_inst == 1 ? h.changed : c->inst_changed_pin[m];
     sivf_stats &st = c->stats;
@@ -695,11 +705,8 @@ sivf_status finish_assign(sivf_ctx *c, int64_t *n_changed, float ms) {
 }
 
 sivf_status finish_update(sivf_ctx *c, float ms) {
-    if (c->ctr_host->error) {
-        c->latched = true;
-        c->err = "the centroids outgrew their buffers (more than 2 nnz + 1024 entries)";
-        return SIVF_ERR_OOM;
-    }
+    const sivf_status e = device_error(c);
+    if (e != SIVF_OK) return e;
     c->c_nnz = c->ctr_host->c_nnz;
     c->if_nnz = c->c_nnz;
     c->dense_terms_h = c->ctr_host->dense_terms;

@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(T, CB ? 8 : assign_min_blocks<T>()) assign_ker
             if (tid < cn) {
                 int t = P.idx[cb + tid];
                 if (P.checked && (t < 0 || t >= P.D)) {  // a term outside [0, D): record it, skip it
-                    atomicOr(&P.ctr->error, 2ull);
+                    atomicOr(&P.ctr->error, ERR_TERM);
                     t = -1;
                 }
                 const int4 td = t >= 0 ? __ldg(P.tdesc + t) : make_int4(0, 0, 0, -1);
@@ -1058,7 +1058,7 @@ __global__ void k_classify(AssignParams P, int light_max) {
             int64_t b = P.row_ptr[i], z = P.row_ptr[i + 1];
             if (P.checked && (b < 0 || z < b || z > P.nnz)) {
                 // the borrowed CSR changed since it was validated: record it, read nothing
-                atomicOr(&P.ctr->error, 1ull);
+                atomicOr(&P.ctr->error, ERR_ROW);
                 b = z = 0;
             }
             const int32_t a = P.labels_prev[i];
@@ -1112,7 +1112,7 @@ __device__ __forceinline__ int light_stage(const AssignParams &P, uint32_t *rho,
         if (h < s1) {
             const int t = P.idx[h];
             vs = P.val[h] * FIX_SCALE;
-            if (P.checked && (t < 0 || t >= P.D)) atomicOr(&P.ctr->error, 2ull);
+            if (P.checked && (t < 0 || t >= P.D)) atomicOr(&P.ctr->error, ERR_TERM);
             else td = __ldg(P.tdesc + t);
         }
         const bool dense = td.w >= 0;

@@ -11,6 +11,8 @@ namespace {
 // loop[0] = r of the last assignment, loop[1] = iteration cap, loop[2] = instances
 // still running. An instance converges at the first assignment r > 1 that changes
 // none of its labels (done[m] = r); until then objf[m] follows its update objective.
+// A failed check ends the loop, so that the host sees it: the next assignment
+// would clear the counters it is recorded in.
 __global__ void loop_control(cudaGraphConditionalHandle h, int32_t *loop, int32_t n_inst,
                              const unsigned long long *inst_changed, const DevCounters *ctr, const double *obj,
                              int32_t *done, double *objf) {
@@ -33,7 +35,7 @@ __global__ void loop_control(cudaGraphConditionalHandle h, int32_t *loop, int32_
     if (threadIdx.x == 0) {
         loop[0] = r;
         loop[2] = rem;
-        cudaGraphSetConditional(h, (rem > 0 && r < loop[1]) ? 1u : 0u);
+        cudaGraphSetConditional(h, (rem > 0 && r < loop[1] && ctr->error == 0) ? 1u : 0u);
     }
 }
 

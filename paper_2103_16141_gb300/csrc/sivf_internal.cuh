@@ -85,6 +85,11 @@ constexpr float FP16_INV_SCALE = 1.0f / 16384.0f;
 // (IVF-CBICP keeps cluster ids).
 __host__ __device__ __forceinline__ int score_slot(int p) { return p ^ ((p >> 5) & 7); }
 
+// What a device-side check found (DevCounters::error).
+constexpr unsigned long long ERR_ROW = 1;       // a row offset of the CSR is out of range
+constexpr unsigned long long ERR_TERM = 2;      // a term of the CSR is outside [0, D)
+constexpr unsigned long long ERR_CAPACITY = 4;  // more centroid entries than the buffers hold
+
 struct DevCounters {
     unsigned long long changed;
     unsigned long long filtered;
@@ -94,7 +99,7 @@ struct DevCounters {
     unsigned long long rescore_cands;
     unsigned long long n_moving;     // lambda^[r] = 0 count (written by finalize)
     unsigned int work, work_light;   // object work counters of the CTA and the warp kernel
-    unsigned long long error;        // nonzero: device-side check failed (code)
+    unsigned long long error;        // nonzero: device-side check failed (ERR_* bits)
     long long moved;                 // object non-zeros gathered by the last update
     long long c_nnz;                 // centroid non-zeros after the last update
     unsigned long long dense_entries;   // dense-row entries read by the assignment

@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(WR_THREADS) k_write_rows(
     const int64_t o = coff_new[j];
     const int64_t cb = coff_old[j], ce = coff_old[j + 1];
     if (coff_new[k] > cap) {  // more centroid entries than the buffers hold: write nothing, report
-        if (j == 0 && threadIdx.x == 0) atomicOr(error, 1ull);
+        if (j == 0 && threadIdx.x == 0) atomicOr(error, ERR_CAPACITY);
         return;
     }
     if (flag[j]) {
@@ -442,7 +442,9 @@ __global__ void __launch_bounds__(WR_THREADS) k_write_rows(
 // Last kernel of the centroid step. Blocks below n_inst: the objective sums of
 // an instance, in a fixed order (per-thread strided partial sums, then a
 // tree). The others copy the new rows back over the current ones (fixed
-// buffers for graph replay). Block 0 leaves the step's counts.
+// buffers for graph replay). Block 0 leaves the step's counts. New rows that
+// outgrew the buffers were not written: the current ones stay, whole and within
+// the buffers, for the file that is built next.
 __global__ void __launch_bounds__(1024) k_finish_rows(int32_t k, int64_t cap, int32_t n_inst, const int32_t *inst_k,
                                                       const double *jA, const double *jU, double *out,
                                                       const int64_t *coff_src, const int32_t *term_src,
@@ -478,7 +480,8 @@ __global__ void __launch_bounds__(1024) k_finish_rows(int32_t k, int64_t cap, in
         }
         return;
     }
-    const int64_t n = min(coff_src[k], cap);
+    const int64_t n = coff_src[k];
+    if (n > cap) return;
     const int64_t g = (blockIdx.x - n_inst) * (int64_t)blockDim.x + threadIdx.x;
     const int64_t st = (int64_t)(gridDim.x - n_inst) * blockDim.x;
     for (int64_t e = g; e < n; e += st) {
@@ -881,7 +884,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows2(
     const int j = blockIdx.x;
     if (j >= k) return;
     const bool over = coff_new[k] > cap;  // more entries than the buffers hold: write nothing, report
-    if (over && j == 0 && threadIdx.x == 0) atomicOr(error, 1ull);
+    if (over && j == 0 && threadIdx.x == 0) atomicOr(error, ERR_CAPACITY);
     if (over) return;
     const int64_t o0 = coff_new[j];
     const int64_t cb = coff_old[j], ce = coff_old[j + 1];

@@ -204,7 +204,9 @@ sivf_status sivf_init(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_t
  * reallocating: mu_j^[0] = x_{init_ids[j]}, no labels, every cluster moving,
  * first inverted file rebuilt (same as the tail of sivf_init).
  *   init_ids : HOST int32[k], distinct object ids. Copied.
- * Errors: SIVF_ERR_INVALID_ARG (ids), SIVF_ERR_CUDA.
+ * Errors: SIVF_ERR_INVALID_ARG (ids), SIVF_ERR_CUDA, SIVF_ERR_OOM (context
+ * latched: a seed's row offsets are out of range, or the seed rows do not fit the
+ * centroid buffers, as the borrowed CSR changed since sivf_init).
  */
 sivf_status sivf_reseed(sivf_ctx *ctx, const int32_t *init_ids);
 

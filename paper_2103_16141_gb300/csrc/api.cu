@@ -76,6 +76,7 @@ sivf_status check_usable(sivf_ctx *c) {
 cudaError_t read_file_counters(sivf_ctx *c) {
     SIVF_CUDA_TRY(cudaMemcpyAsync(c->ctr_host, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, c->stream));
     SIVF_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (c->ctr_host->error) return cudaErrorMemoryAllocation;  // the seed rows do not fit the centroid buffers
     c->c_nnz = c->ctr_host->c_nnz;
     c->if_nnz = c->c_nnz;
     c->dense_terms_h = c->ctr_host->dense_terms;

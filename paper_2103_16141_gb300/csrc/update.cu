@@ -94,12 +94,20 @@ __global__ void k_validate(int64_t N, int32_t D, int64_t nnz, const int64_t *row
     }
 }
 
+// Live entries of buffers that hold cap: none when the count says more (the
+// rows were then not written; the count's own kernel reports it).
+__device__ __forceinline__ int64_t live_entries(const int64_t *n_dev, int64_t cap) {
+    const int64_t n = *n_dev;
+    return n <= cap ? n : 0;
+}
+
 // State before the first assignment: no labels, no own scores, nothing added
 // to the accumulator, every cluster moving, no sums behind the centroids; and
-// the sizes of the seed rows.
+// the sizes of the seed rows. A row whose offsets are not in the CSR any more
+// (the borrowed arrays changed) is given a size that no buffer holds.
 __global__ void k_reset(int64_t N, int32_t k, int32_t *labels, int32_t *labels_prev, uint32_t *own, int32_t *acc_lab,
                         uint8_t *lam, uint8_t *lam_prev, uint8_t *moving, double *snorm, const int32_t *init_ids,
-                        const int64_t *row_ptr, int64_t *sz, DevCounters *ctr) {
+                        const int64_t *row_ptr, int64_t nnz, int64_t cap, int64_t *sz, DevCounters *ctr) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = g; i < N; i += st) {
         labels[i] = -1;
@@ -112,19 +120,24 @@ __global__ void k_reset(int64_t N, int32_t k, int32_t *labels, int32_t *labels_p
         lam_prev[j] = 0;
         moving[j] = 1;
         snorm[j] = 0.0;
-        const int64_t d = init_ids[j];
-        sz[j] = row_ptr[d + 1] - row_ptr[d];
+        const int64_t d = init_ids[j], b = row_ptr[d], e = row_ptr[d + 1];
+        sz[j] = b >= 0 && b <= e && e <= nnz ? e - b : cap + 1;
     }
     if (g == 0) *ctr = DevCounters{};
 }
 
-// The seed rows, one warp each; their total is left in the counters.
+// The seed rows, one warp each; their total is left in the counters. Rows that
+// the buffers do not hold are not written, and reported.
 __global__ void k_seed_rows(int32_t k, const int32_t *init_ids, const int64_t *row_ptr, const int32_t *idx,
-                            const float *val, const int64_t *coff, int32_t *cterm, float *cval, int32_t *cclu,
-                            DevCounters *ctr) {
+                            const float *val, const int64_t *coff, int64_t cap, int32_t *cterm, float *cval,
+                            int32_t *cclu, DevCounters *ctr) {
     const int lane = threadIdx.x & 31;
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (wid >= k) return;
+    if (coff[k] > cap) {
+        if (wid == 0 && lane == 0) ctr->error = ERR_CAPACITY;
+        return;
+    }
     const int j = (int)wid;
     const int64_t d = init_ids[j];
     const int64_t b = row_ptr[d], e = row_ptr[d + 1], o = coff[j];
@@ -1055,7 +1068,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows2(
 // unstructured file of IVF-CBICP keeps every posting in part 0.
 __global__ void k_if_keys(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
                           const uint8_t *lam, int structured, uint32_t *keys, uint32_t *vals, uint32_t *cnt2) {
-    const int64_t n = min(*n_dev, cap);
+    const int64_t n = live_entries(n_dev, cap);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t key = ((uint32_t)cterm[e] << 1) | (uint32_t)(structured && lam[cclu[e]] ? 1 : 0);
         keys[e] = key;
@@ -1067,7 +1080,7 @@ __global__ void k_if_keys(const int64_t *n_dev, int64_t cap, const int32_t *cter
 // Canonical arrays (if_cid: global cluster ids, if_val) in sorted order.
 __global__ void k_if_fill(const int64_t *n_dev, int64_t cap, const uint32_t *order, const int32_t *cclu,
                           const float *cval, int32_t *if_cid, float *if_val) {
-    const int64_t n = min(*n_dev, cap);
+    const int64_t n = live_entries(n_dev, cap);
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t e = order[q];
         if_cid[q] = cclu[e];
@@ -1317,7 +1330,7 @@ __device__ __forceinline__ uint16_t encode_lp(float u, int prec) {
 // per (term, part) posting counts of the current centroids
 __global__ void k_if_count(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
                            const uint8_t *lam, int structured, uint32_t *cnt2) {
-    const int64_t n = min(*n_dev, cap);
+    const int64_t n = live_entries(n_dev, cap);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
         atomicAdd(cnt2 + (((uint32_t)cterm[e] << 1) | (uint32_t)(structured && lam[cclu[e]] ? 1 : 0)), 1u);
 }
@@ -1333,7 +1346,7 @@ __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *ct
                             const float *cval, const uint8_t *lam, int structured, const int32_t *clu_pos,
                             const int4 *tdesc, uint32_t *cursor, int prec, void *dense, uint16_t *sc_id16,
                             int32_t *sc_id32, float *sc_val, uint32_t *sc_pack, uint16_t *sc_lp) {
-    const int64_t n = min(*n_dev, cap);
+    const int64_t n = live_entries(n_dev, cap);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t t = cterm[e], j = cclu[e];
         const float u = cval[e];
@@ -1367,7 +1380,7 @@ __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *ct
 // half of the upper half's step, as rounding u to BF16 is (2^-8 relative).
 __global__ void k_dense_odd(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
                             const float *cval, const int32_t *clu_pos, const int4 *tdesc, uint16_t *dense) {
-    const int64_t n = min(*n_dev, cap);
+    const int64_t n = live_entries(n_dev, cap);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t p = clu_pos[cclu[e]];
         if (!(p & 1)) continue;
@@ -1544,8 +1557,9 @@ cudaError_t finish_rows(sivf_ctx *c, const double *jA, const double *jU, const i
 }  // namespace
 
 // Restart from new seeds: no labels, no own scores, every cluster moving,
-// mu^[0] = seed rows (distinct documents, so they fit the centroid buffers),
-// first inverted file. No host synchronisation; the counts are in the counters.
+// mu^[0] = seed rows (distinct documents: they fit the centroid buffers unless
+// the borrowed CSR changed), first inverted file. No host synchronisation; the
+// counts and a failed check are in the counters.
 cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev) {
     const int64_t N = c->N;
     const int32_t k = c->k;
@@ -1568,15 +1582,15 @@ cudaError_t reseed_dev(sivf_ctx *c, const int32_t *init_ids_dev) {
     }
     k_reset<<<blocks_gs(std::max<int64_t>(N, k)), TPB, 0, s>>>(N, k, c->labels, c->labels_prev, c->own,
                                                                c->dense ? c->acc_lab : nullptr, c->lam, c->lam_prev,
-                                                               c->moving, c->snorm, init_ids_dev, c->row_ptr, sz,
-                                                               c->ctr);
+                                                               c->moving, c->snorm, init_ids_dev, c->row_ptr, c->nnz,
+                                                               c->cap_c, sz, c->ctr);
     note_launch();
     c->iter = 1;  // finalize below marks every cluster moving
     SIVF_CUDA_TRY(launch_finalize_assign(c));
     c->iter = 0;
     SIVF_CUDA_TRY(row_offsets(c, sz, cur));
     k_seed_rows<<<blocks_for((int64_t)k * 32), TPB, 0, s>>>(k, init_ids_dev, c->row_ptr, c->idx, c->val, c->coff[cur],
-                                                            c->cterm[cur], c->cval[cur], c->cclu, c->ctr);
+                                                            c->cap_c, c->cterm[cur], c->cval[cur], c->cclu, c->ctr);
     note_launch();
     SIVF_CUDA_TRY(cudaGetLastError());
     SIVF_CUDA_TRY(build_inverted_file(c));

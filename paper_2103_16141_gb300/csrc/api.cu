@@ -102,7 +102,7 @@ void pick_assign_config(sivf_ctx *c) {
         // k = 10,000 BF16 - / - / 23.3 / 28.7; k = 20,000 BF16 - / - / 82 / 55.
         T = 512;
         for (int t = 64; t < 512; t *= 2) {
-            const size_t cta = (size_t)((c->kmax + 7) & ~7) * 4 + (size_t)t * ASSIGN_STAGE_BYTES + 2560;  // + static, reserved
+            const size_t cta = assign_dynamic_smem(c->kmax, t, false, 0) + 2560;  // + static, reserved
             if ((size_t)sm_smem / cta * (size_t)t >= 1024) {
                 T = t;
                 break;
@@ -111,7 +111,7 @@ void pick_assign_config(sivf_ctx *c) {
     }
     c->assign_threads = T;
     c->assign_ctas_per_sm = c->cfg.ctas_per_sm > 0 ? c->cfg.ctas_per_sm : 0;
-    const bool fits = ((size_t)((c->kmax + 7) & ~7) * 4 + (size_t)T * ASSIGN_STAGE_BYTES) <= (size_t)smem;
+    const bool fits = assign_smem_fits(c->kmax, T, 0, smem);
     c->assign_global = c->cfg.score_buffer == 2 || (c->cfg.score_buffer == 0 && !fits) ? 1 : 0;
     if (c->cfg.icp == 2) {  // IVF-CBICP: 128 threads, shared score vector, no tuning
         c->assign_threads = 128;
@@ -189,9 +189,7 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     if (c->cfg.icp == 2) {  // the IVF-CBICP kernel keeps the score vector and lambda bits in shared memory
         int smem = 0;
         INIT_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device), "attr");
-        const size_t need = (size_t)((c->kmax + 7) & ~7) * 4 + 128 * (size_t)ASSIGN_STAGE_BYTES +
-                            (size_t)((k + 31) >> 5) * 4;
-        if (need > (size_t)smem) {
+        if (!assign_smem_fits(c->kmax, 128, k, smem)) {
             free_all(c);
             delete c;
             return SIVF_ERR_INVALID_ARG;

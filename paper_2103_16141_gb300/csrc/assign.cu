@@ -1408,9 +1408,7 @@ __global__ void __launch_bounds__(1024) finalize_kernel(int32_t k, int first_ite
 
 template <int T, int PREC, bool CID16, bool GRHO, bool CB = false>
 cudaError_t launch_t(sivf_ctx *c, const AssignParams &P, int ctas_per_sm) {
-    const int kpad = (c->kmax + 7) & ~7;
-    const size_t smem = (GRHO ? 0 : (size_t)kpad * 4) + (size_t)T * ASSIGN_STAGE_BYTES +
-                        (CB ? (size_t)((c->k + 31) >> 5) * 4 : 0);
+    const size_t smem = assign_dynamic_smem(c->kmax, T, GRHO, CB ? c->k : 0);
     auto kern = assign_kernel<T, PREC, CID16, GRHO, CB>;
     // the attribute and occupancy queries are host calls that a stream capture
     // refuses: they run on the first (host-launched) step and are cached
@@ -1422,7 +1420,8 @@ cudaError_t launch_t(sivf_ctx *c, const AssignParams &P, int ctas_per_sm) {
         int optin = 0;
         SIVF_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
         SIVF_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-        if (smem + fa.sharedSizeBytes > (size_t)optin) return cudaErrorInvalidConfiguration;
+        if (smem + fa.sharedSizeBytes > (size_t)optin || fa.sharedSizeBytes > assign_static_bound(T))
+            return cudaErrorInvalidConfiguration;
         SIVF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            optin - (int)fa.sharedSizeBytes));
         int occ = 0;
@@ -1650,8 +1649,8 @@ cudaError_t autotune_assign(sivf_ctx *c) {
     for (int g = 0; g < 2; ++g) {
         if (g == 1 && !c->grho) continue;
         for (int t : threads) {
-            const size_t cta_smem = (size_t)kpad * 4 + (size_t)t * ASSIGN_STAGE_BYTES;
-            if (!g && cta_smem > (size_t)dev_smem) continue;
+            const size_t cta_smem = assign_dynamic_smem(c->kmax, t, false, 0);
+            if (!g && !assign_smem_fits(c->kmax, t, 0, dev_smem)) continue;
             // a shared score vector whose size lets fewer than 512 threads
             // reside per SM is not tried (at k = 20,000 the 32- to 128-thread
             // CTAs ran 3-16x longer than 512 threads); 512-thread CTAs always

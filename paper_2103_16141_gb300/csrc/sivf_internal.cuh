@@ -68,6 +68,19 @@ constexpr int64_t IF_PAD = 256;
 // vector: a segment (first quad, quads, scaled value, end in quads) and a
 // dense term (row, scaled value)
 constexpr int ASSIGN_STAGE_BYTES = 24;
+// Shared memory of an assignment CTA of T threads: what its launch asks for
+// (score vector of kmax clusters where it is not in global memory, staging,
+// lambda bits of k clusters for IVF-CBICP), and a bound on the static arrays
+// beside it (28 bytes per warp and 72; launch_t checks the kernels against it).
+// Both count against the opt-in limit of a block.
+inline size_t assign_dynamic_smem(int32_t kmax, int T, bool global_scores, int32_t cb_k) {
+    return (global_scores ? 0 : (size_t)((kmax + 7) & ~7) * 4) + (size_t)T * ASSIGN_STAGE_BYTES +
+           (size_t)((cb_k + 31) >> 5) * 4;
+}
+constexpr size_t assign_static_bound(int T) { return (size_t)T + 128; }
+inline bool assign_smem_fits(int32_t kmax, int T, int32_t cb_k, int optin) {
+    return assign_dynamic_smem(kmax, T, false, cb_k) + assign_static_bound(T) <= (size_t)optin;
+}
 // Scores are accumulated as unsigned fixed point with quantum 2^-31:
 // q = ceil(fl(v * u) * 2^31). Cosine scores are <= 1 (+ rounding), so the
 // sum of an object's terms stays below 2^32.

@@ -1044,7 +1044,8 @@ __global__ void k_begin(int64_t N, int32_t k, int32_t n_inst, const int32_t *lab
 // with no moving cluster (a batch's converged instance) goes to neither: its
 // own cluster is the only candidate and every front is empty, so its label and
 // own score stay as they are. IVF-CBICP still walks its lists. In checked mode
-// the row offsets are checked here, before anything is read through them.
+// the row offsets are checked here, before anything is read through them, and
+// so are the terms of the objects that no kernel will read.
 __global__ void k_classify(AssignParams P, int light_max) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1068,6 +1069,10 @@ __global__ void k_classify(AssignParams P, int light_max) {
                 const int n_mov = P.mov_beg[m + 1] - P.mov_beg[m];
                 done = n_mov == 0;
                 light = !done && n_mov <= light_max;
+                if (done && P.checked) {
+                    for (int64_t h = b; h < z; ++h)
+                        if (P.idx[h] < 0 || P.idx[h] >= P.D) atomicOr(&P.ctr->error, ERR_TERM);
+                }
             }
             e = make_int4((int)i, (int)b, (int)(z - b) | (filt ? (int)0x80000000 : 0), a);
         }

@@ -1171,6 +1171,12 @@ __global__ void __launch_bounds__(TPB) k_if_lists(int32_t D, int32_t k, int32_t 
 // dense threshold from the histogram: the smallest bin >= bmin whose rows
 // (with every longer bin's) fit in cap entries; DENSE_BINS + 1 = no dense rows.
 constexpr int IF_TILE = 4 * TPB;
+// Up to this many tiles every block adds up the earlier ones for itself, above
+// it, where that grows with their square, they are scanned in a launch of their
+// own. ms per update (3000 documents, k = 50), added / scanned: 1954 tiles 0.312
+// / 0.316, 3907 0.366 / 0.373, 15,625 0.754 / 0.691, 62,500 3.37 / 1.91, 125,000
+// (128M terms) 9.91 / 3.49.
+constexpr int64_t IF_TILES_ADDED = 4096;
 
 struct IfSums {
     long long len, room, w8;
@@ -1250,13 +1256,41 @@ __global__ void __launch_bounds__(TPB) k_if_tiles(int32_t D, int32_t n_inst, con
     }
 }
 
+// The tiles' sums made sums of the earlier tiles, by one CTA of which a thread
+// takes PER tiles a turn.
+__global__ void __launch_bounds__(TPB) k_if_tile_scan(int64_t n_tiles, IfSums *tiles) {
+    constexpr int PER = 4;
+    __shared__ IfSums warp_s[TPB / 32];
+    IfSums carry = {0, 0, 0};
+    for (int64_t b = 0; b < n_tiles; b += TPB * PER) {
+        const int64_t t0 = b + (int64_t)threadIdx.x * PER;
+        IfSums v[PER], sum = {0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            v[q] = t0 + q < n_tiles ? tiles[t0 + q] : IfSums{0, 0, 0};
+            sum = if_add(sum, v[q]);
+        }
+        IfSums total;
+        const IfSums inc = if_block_scan(sum, warp_s, total);
+        IfSums at = {carry.len + inc.len - sum.len, carry.room + inc.room - sum.room, carry.w8 + inc.w8 - sum.w8};
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            if (t0 + q < n_tiles) tiles[t0 + q] = at;
+            at = if_add(at, v[q]);
+        }
+        carry = if_add(carry, total);
+    }
+}
+
 // Third pass: the offsets (sums of the earlier tiles, then within the tile)
 // and what the assignment reads about a term, in one 16-byte descriptor: the
 // first quad of its list in the scan copy, its front and list lengths, and its
 // dense row. The last quads of a sparse list's front and back are filled up
-// with zero postings here (they add 0 to a score).
+// with zero postings here (they add 0 to a score). tiles: sums of the earlier
+// tiles (summed), or the tiles' own, of which every block adds up the earlier
+// ones.
 __global__ void __launch_bounds__(TPB) k_if_offsets(int32_t D, const int64_t *len, const int32_t *mf0,
-                                                    const int32_t *w8, const IfSums *tiles, int64_t *if_off,
+                                                    const int32_t *w8, const IfSums *tiles, int summed, int64_t *if_off,
                                                     int4 *tdesc, uint16_t *sc_id16, int32_t *sc_id32, float *sc_val,
                                                     uint32_t *sc_pack, uint16_t *sc_lp, DevCounters *ctr) {
     __shared__ IfSums warp_s[TPB / 32];
@@ -1273,10 +1307,14 @@ __global__ void __launch_bounds__(TPB) k_if_offsets(int32_t D, const int64_t *le
     long long n_dense = 0;
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         IfSums base = {0, 0, 0};
-        for (int64_t q = threadIdx.x; q < tile; q += TPB) base = if_add(base, tiles[q]);
-        IfSums unused;
-        if_block_scan(base, warp_s, unused);
-        base = unused;  // every earlier tile
+        if (summed) {
+            base = tiles[tile];
+        } else {
+            for (int64_t q = threadIdx.x; q < tile; q += TPB) base = if_add(base, tiles[q]);
+            IfSums total;
+            if_block_scan(base, warp_s, total);
+            base = total;  // every earlier tile
+        }
 #pragma unroll
         for (int q = 0; q < IF_TILE / TPB; ++q) {
             const int64_t t = tile * IF_TILE + (int64_t)q * TPB + threadIdx.x;
@@ -1473,7 +1511,12 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     k_if_tiles<<<tile_blocks, TPB, 0, s>>>(D, c->n_inst, c->inst_d, c->inst_k, len, c->if_mf0, min_len, hist,
                                            dense ? bmin : DENSE_BINS + 1, (unsigned long long)c->cap_dense,
                                            c->dense_thr, w8, tiles);
-    k_if_offsets<<<tile_blocks, TPB, 0, s>>>(D, len, c->if_mf0, w8, tiles, c->if_off, c->tdesc, c->sc_id16, c->sc_id32,
+    const bool summed = n_tiles > IF_TILES_ADDED;
+    if (summed) {
+        k_if_tile_scan<<<1, TPB, 0, s>>>(n_tiles, tiles);
+        note_launch();
+    }
+    k_if_offsets<<<tile_blocks, TPB, 0, s>>>(D, len, c->if_mf0, w8, tiles, summed ? 1 : 0, c->if_off, c->tdesc, c->sc_id16, c->sc_id32,
                                              c->sc_val, c->sc_pack, c->sc_lp, c->ctr);
     note_launch(4);
     SIVF_CUDA_TRY(cudaGetLastError());

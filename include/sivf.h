@@ -118,8 +118,7 @@ typedef struct {
                             0 = automatic (96 MB, below the L2 size), < 0 = none */
     float dense_min_fraction; /* a list becomes a dense row when it holds at least this
                             fraction of its instance's k (the threshold rises while the
-                            rows would exceed dense_max_bytes); 0 = automatic (0.25 with
-                            FP32, 0.17 with BF16/FP16 postings).
+                            rows would exceed dense_max_bytes); 0 = automatic (0.25).
                             Must be in [0, 1]. IVF-CBICP (icp = 2) uses no dense rows */
     int light_max_moving;     /* filtered objects (own cluster invariant) of an instance with
                             at most this many moving clusters are scored by one warp each

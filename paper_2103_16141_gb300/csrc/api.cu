@@ -273,14 +273,14 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
                 c->cap_dense += (int64_t)(inst_d[(size_t)m + 1] - inst_d[(size_t)m]) *
                                 ((inst_k[(size_t)m + 1] - inst_k[(size_t)m] + 7) & ~7);
         }
-        // Where a row of k entries costs as much as the postings of the list:
-        // an entry of a 16-bit row is half the bytes of an FP32 one. ms per
-        // assignment at 0.25 / 0.18 / 0.14 / 0.1: BF16 k = 20,000 46.9 / 46.1 /
-        // 46.1 / 46.5, k = 10,000 19.9 / 19.6 / 19.6 / 19.6, k = 8,000 15.35 /
-        // 15.2 / 15.2 / 15.2; FP32 k = 20,000 10.7 / 10.7 / 10.9 / 11.2, k =
-        // 1000 9.97 / 10.5 / - / -.
-        const float line = c->cfg.prec == SIVF_FP32 ? 0.25f : 0.17f;
-        c->dense_frac = c->cfg.dense_min_fraction > 0.f ? c->cfg.dense_min_fraction : line;
+        // The default is the same for every precision: a shorter list keeps its
+        // exact integer sums. With 16-bit postings a line at 0.17 is 1 to 2 %
+        // faster (ms per assignment at 0.25 / 0.18: BF16 k = 20,000 46.9 / 46.1,
+        // k = 10,000 19.9 / 19.6, k = 8,000 15.35 / 15.2), but moves those lists
+        // to FP32 chains, whose partial sums hold 24 bits; a caller may choose
+        // it. FP32 is fastest here (k = 20,000 10.7 at 0.25 and 0.18, 10.9 at
+        // 0.14; k = 1000 9.97 / 10.5).
+        c->dense_frac = c->cfg.dense_min_fraction > 0.f ? c->cfg.dense_min_fraction : 0.25f;
         if (c->cap_dense / 8 >= 0x7FFFFFFFll) {  // rows are addressed in 8-entry units with 32 bits
             free_all(c);
             delete c;

@@ -710,11 +710,11 @@ __device__ __forceinline__ void add_product(unsigned long long &hi, unsigned lon
     hi += __umul64hi(a, b) + (lo < p ? 1ull : 0ull);
 }
 
-// x in [0, 2) in units of 2^-63, rounded down: exact from 2^-40 up.
+// x in [2^-40, 2) in units of 2^-63, exactly; 0 for smaller x >= 0, whose bits
+// no unit of 2^-63 holds.
 __device__ __forceinline__ unsigned long long fixed63(float x) {
-    const uint32_t b = __float_as_uint(x), e = b >> 23;  // a subnormal comes out as 0 either way
-    const unsigned long long m = (b & 0x7fffffu) | 0x800000u;
-    return e >= 87u ? m << (e - 87u) : e > 63u ? m >> (87u - e) : 0ull;
+    const uint32_t b = __float_as_uint(x), e = b >> 23;
+    return e >= 87u ? (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (e - 87u) : 0ull;
 }
 
 // Turns of a whole row's loop (ILP * WR_THREADS entry pairs each) after which
@@ -734,7 +734,8 @@ constexpr int DOT_ILP = 4;
 // 2^-63 and multiplied and added exactly in 128 bits as well: conversions and
 // products in FP64 took longer than the reads (the pass 330 us, now 273 at 1000
 // rows of 100,000 entries, 17 % non-zero). By Cauchy-Schwarz that sum stays
-// below 2^63 times 2^63. The row's words (row_words) are left with exactly its
+// below 2^63 times 2^63. Values below 2^-40, which that unit would cut short,
+// are multiplied and added in FP64, in a loop of their own. The row's words (row_words) are left with exactly its
 // non-zero entries' bits: bits of entries that became zero are cleared where the
 // row is read through its map, all words are written where it is read whole.
 // Other clusters keep their row (sizes and objective pieces as in k_write_rows).
@@ -763,6 +764,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     // WR_THREADS-th) whose terms lie below a bound, from where it stopped last
     const int32_t doff = clu_doff[j];
     unsigned long long dot_hi = 0ull, dot_lo = 0ull;
+    float least = 1.f;  // of the previous values
     const uint32_t old = (uint32_t)(ce - cb);  // a row has at most 2^31 entries
     uint32_t at = threadIdx.x;
     auto dot_upto = [&](uint32_t bound) {
@@ -776,12 +778,13 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
 #pragma unroll
             for (int q = 0; q < DOT_ILP; ++q) {
                 v[q] = t[q] < bound ? acc[base + t[q]] : 0;
-                u[q] = t[q] < bound ? cval_old[cb + (at + q * WR_THREADS)] : 0.f;
+                u[q] = t[q] < bound ? cval_old[cb + (at + q * WR_THREADS)] : 1.f;  // times 0
             }
             more = t[DOT_ILP - 1] < bound;
 #pragma unroll
             for (int q = 0; q < DOT_ILP; ++q) {
                 add_product(dot_hi, dot_lo, (unsigned long long)v[q], fixed63(u[q]));
+                least = fminf(least, u[q]);
                 at += t[q] < bound ? WR_THREADS : 0;
             }
         }
@@ -870,7 +873,15 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     const double nrm = sqrt(((double)ss_hi * 18446744073709551616.0 + (double)ss_lo) * (inv_scale * inv_scale));
     dot_upto((uint32_t)L);
     block_sum_u128(dot_hi, dot_lo, sh128);
-    const double dot = ((double)dot_hi * 18446744073709551616.0 + (double)dot_lo) * inv_scale * 0x1p-63;
+    double dot = ((double)dot_hi * 18446744073709551616.0 + (double)dot_lo) * inv_scale * 0x1p-63;
+    if (__syncthreads_or(least < 0x1p-40f)) {
+        double small = 0.0;
+        for (uint32_t q = threadIdx.x; q < old; q += WR_THREADS) {
+            const float u = cval_old[cb + q];
+            if (u < 0x1p-40f) small += (double)acc[base + (cterm_old[cb + q] - doff)] * (double)u;
+        }
+        dot += block_sum_fixed(small, reinterpret_cast<double *>(shl)) * inv_scale;
+    }
     if (threadIdx.x == 0) {
         sz[j] = nz;
         snorm_new[j] = nrm;

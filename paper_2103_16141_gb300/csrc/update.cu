@@ -159,20 +159,15 @@ __global__ void k_seed_rows(int32_t k, const int32_t *init_ids, const int64_t *r
 __global__ void k_set_labels(int64_t N, const int32_t *src, int32_t *labels, const int32_t *labels_prev, int rebuilt,
                              uint32_t *own, uint8_t *moving) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t a = src[i], old = labels[i];
+        const int32_t a = src[i], old = labels[i], prev = labels_prev[i];
         if (old != a) {
             labels[i] = a;
             own[i] = OWN_INVALID;
-            if (rebuilt) {
-                moving[a] = 1;
-                if (old >= 0) moving[old] = 1;
-            }
         }
-        const int32_t prev = labels_prev[i];
-        if (a != prev) {
-            moving[a] = 1;
-            if (prev >= 0) moving[prev] = 1;
-        }
+        const bool moved = rebuilt && old != a;
+        if (a != prev || moved) moving[a] = 1;
+        if (a != prev && prev >= 0) moving[prev] = 1;
+        if (moved && old >= 0 && old != prev) moving[old] = 1;  // a store per object and cluster, not two
     }
 }
 

@@ -49,7 +49,7 @@ cudaError_t dmalloc(sivf_ctx *c, T **p, size_t n) {
 void free_all(sivf_ctx *c) {
     void *ptrs[] = {c->labels, c->labels_prev, c->own, c->sumv, c->lam, c->lam_prev, c->moving, c->mov_list,
                     c->n_mov_dev, c->snorm, c->snorm_new, c->coff[0], c->coff[1], c->cterm[0], c->cterm[1],
-                    c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->if_cid, c->if_val, c->tdesc, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
+                    c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->tdesc, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
                     c->ctr, c->obj_dev, c->ws.base, c->inst_obj, c->inst_k, c->mov_beg, c->clu_koff,
                     c->inst_changed, c->own_row_ptr, c->own_idx, c->own_val, c->clu_doff,
                     c->loop_dev, c->done_dev, c->objf_dev, c->grho, c->acc, c->acc_off, c->acc_lab, c->acc_bits, c->acc_bit_off,
@@ -240,10 +240,8 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     INIT_CUDA(dmalloc(c, &c->cclu, capc), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_off, (size_t)D + 1), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_mf0, D), "alloc");
-    // posting arrays carry a small tail pad; the scan copy also fills the front
-    // and the back of every list up to a multiple of 4 entries
-    INIT_CUDA(dmalloc(c, &c->if_cid, capc + IF_PAD), "alloc");
-    INIT_CUDA(dmalloc(c, &c->if_val, capc + IF_PAD), "alloc");
+    // the scan copy fills the front and the back of every list up to a multiple
+    // of 4 entries, and carries a small tail pad
     c->cap_s = capc + 3 * std::min<int64_t>(2 * (int64_t)D, capc) + IF_PAD;
     const size_t caps = (size_t)c->cap_s;
     const bool ids16 = c->kmax <= 65536;
@@ -344,9 +342,10 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
         const size_t n8 = (size_t)N * 8, k8 = (size_t)k * 8;
         // u1: 4 label key/value arrays (4 B x N), tuple counts/offsets (8 B x N),
         // per-cluster arrays; u2 per tuple (sort mode only): 4 sort arrays,
-        // term, rank, value, sorted value, 64-bit key, piece sum, unique term
-        // and sum (60 B)
-        size_t phase1 = 4 * (size_t)N * 4 + 2 * n8 + 14 * k8 + (c->dense ? 0 : 60 * ((size_t)nnz + 1)) + 32 * 4096;
+        // term and rank (later the piece sum), value, sorted value, 64-bit key,
+        // unique term and sum (52 B). The dense form takes no more per object
+        // than an assignment (lists 16 B, the autotuner's snapshots 8 B).
+        size_t phase1 = (c->dense ? 3 * n8 : 4 * n8 + 52 * ((size_t)nnz + 1)) + 14 * k8 + 32 * 4096;
         // u5: sort arrays (16 B x entries), per-term counts, lengths, dense widths
         // and offsets (40 B x terms), the dense-length histogram
         // (per-term counts with the first, all of the second's arrays without it)
@@ -933,9 +932,9 @@ sivf_status sivf_get_inverted_file(sivf_ctx *c, int64_t *off, int32_t *mf0, int3
         API_CUDA(c, cudaStreamSynchronize(c->stream), "sync");
         return fail(c, SIVF_ERR_INVALID_ARG, "capacity below the inverted-file nnz");
     }
-    API_CUDA(c, cudaMemcpyAsync(cid, c->if_cid, sizeof(int32_t) * c->if_nnz, cudaMemcpyDeviceToHost, c->stream),
+    API_CUDA(c, cudaMemcpyAsync(cid, c->cterm[1 - c->cur], sizeof(int32_t) * c->if_nnz, cudaMemcpyDeviceToHost, c->stream),
              "copy");
-    API_CUDA(c, cudaMemcpyAsync(u, c->if_val, sizeof(float) * c->if_nnz, cudaMemcpyDeviceToHost, c->stream), "copy");
+    API_CUDA(c, cudaMemcpyAsync(u, c->cval[1 - c->cur], sizeof(float) * c->if_nnz, cudaMemcpyDeviceToHost, c->stream), "copy");
     API_CUDA(c, cudaStreamSynchronize(c->stream), "sync");
     return SIVF_OK;
 }

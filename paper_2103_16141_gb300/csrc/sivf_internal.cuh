@@ -11,10 +11,10 @@
 //   centroids (x2)        coff int64[k+1], cterm int32[cap], cval f32[cap], cclu int32[cap]
 //                                        cluster-major FP32 master copy, ascending terms
 //   snorm                 f64[k]        ||s_j|| of the sum behind each centroid
-//   inverted file         if_off int64[D+1], if_mf0 int32[D]; if_cid int32[cap],
-//                                        if_val f32[cap]: canonical order (front ids
-//                                        ascending, then back ids ascending), built
-//                                        on demand for the getters
+//   inverted file         if_off int64[D+1], if_mf0 int32[D]; its entries in canonical
+//                                        order (front ids ascending, then back ids
+//                                        ascending) are built on demand for the getters,
+//                                        in the centroid buffer that is not current
 //   term table            tdesc int4[D]: first quad of term t's list in the scan copy,
 //                                        front length, list length, and first entry / 8
 //                                        of its dense row or -1 (the term is scanned
@@ -32,8 +32,7 @@
 //                                        id); pos_clu int32[k]: the inverse (instance
 //                                        offset + position -> local id). Score vectors are
 //                                        indexed by position. IVF-CBICP keeps id order.
-//   dense head rows
-//                                        dense_val (u16 or f32) [cap_dense]: one row per dense
+//   dense head rows       dense_val      (u16 or f32) [cap_dense]: one row per dense
 //                                        term, the term's value for every cluster of its
 //                                        instance at the cluster's scan position (0 where
 //                                        the cluster lacks the term), padded to a multiple
@@ -183,10 +182,8 @@ struct sivf_ctx {
     // structured inverted file
     int64_t *if_off = nullptr;
     int32_t *if_mf0 = nullptr;
-    int32_t *if_cid = nullptr;
-    float *if_val = nullptr;
     int64_t if_nnz = 0;
-    bool canon_stale = true;  // if_cid / if_val predate the last inverted-file build
+    bool canon_stale = true;  // the canonical file predates the last inverted-file build
     // term table and scan copy (local ids); which arrays exist depends on the
     // id width (16 bits when every instance has k <= 65536) and the precision
     int4 *tdesc = nullptr;

@@ -1548,8 +1548,9 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
 
 // The canonical structured inverted file of the current centroids and lambda
 // (Algorithm 5: for every term, the moving centroids first and the invariant
-// ones after, ascending ids in each part) in if_cid / if_val, with the offsets
-// and front lengths of the last build: a stable radix sort of the centroid
+// ones after, ascending ids in each part), with the offsets and front lengths of
+// the last build, in the centroid buffer that is not current (terms: cluster
+// ids, values), which nothing reads until the next update writes it: a stable radix sort of the centroid
 // entries by (term, part). Used by the getters only; synchronises the stream.
 cudaError_t build_canonical_if(sivf_ctx *c) {
     if (!c->canon_stale) return cudaSuccess;
@@ -1569,8 +1570,8 @@ cudaError_t build_canonical_if(sivf_ctx *c) {
     note_launch();
     bool alt = false;
     SIVF_CUDA_TRY(radix_sort_pairs_dev(k0, v0, k1, v1, cap, n_dev, c->bits_t + 1, &alt, ws, s));
-    k_if_fill<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, alt ? v1 : v0, c->cclu, c->cval[cur], c->if_cid,
-                                              c->if_val);
+    k_if_fill<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, alt ? v1 : v0, c->cclu, c->cval[cur],
+                                              c->cterm[1 - cur], c->cval[1 - cur]);
     note_launch();
     SIVF_CUDA_TRY(cudaGetLastError());
     SIVF_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1736,18 +1737,18 @@ cudaError_t run_update(sivf_ctx *c) {
     SIVF_CUDA_TRY(scan_exclusive_i64(tc, toff, N, T_d, ws, s));
     uint32_t *sa_k = ws.take<uint32_t>(Tmax), *sa_v = ws.take<uint32_t>(Tmax);
     uint32_t *sb_k = ws.take<uint32_t>(Tmax), *sb_v = ws.take<uint32_t>(Tmax);
-    uint32_t *tterm = ws.take<uint32_t>(Tmax), *trank = ws.take<uint32_t>(Tmax);
+    double *part = ws.take<double>(Tmax);  // holds the tuples' terms and ranks before the piece sums
+    uint32_t *tterm = reinterpret_cast<uint32_t *>(part), *trank = tterm + Tmax;
     float *tval = ws.take<float>(Tmax), *sval = ws.take<float>(Tmax);
     unsigned long long *key64 = ws.take<unsigned long long>(Tmax);
-    double *part = ws.take<double>(Tmax);
+    int32_t *rank2clu = ws.take<int32_t>(k);
     int32_t *uterm = ws.take<int32_t>(Tmax);
     double *usum = ws.take<double>(Tmax);
-    if (!sa_k || !sa_v || !sb_k || !sb_v || !tterm || !trank || !tval || !sval || !key64 || !part || !uterm || !usum)
+    if (!sa_k || !sa_v || !sb_k || !sb_v || !part || !tval || !sval || !key64 || !rank2clu || !uterm || !usum)
         return cudaErrorMemoryAllocation;
     const int bits_r = bits_for((uint64_t)(k - 1));
     if (bits_r + c->bits_tl <= 32) {
         // one sort on (rank, local term) carrying the value bits
-        int32_t *rank2clu = reinterpret_cast<int32_t *>(tterm);
         k_rank2clu<<<blocks_for(k), TPB, 0, s>>>(k, flag, rrank, rank2clu);
         k_expand_packed<<<blocks_gs(N * 32), TPB, 0, s>>>(N, perm, c->labels, rrank, tc, toff, c->row_ptr, c->idx,
                                                             c->val, c->clu_doff, c->bits_tl, sa_k, sa_v);

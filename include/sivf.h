@@ -274,7 +274,8 @@ sivf_status sivf_get_centroids(sivf_ctx *ctx, int64_t *off, int32_t *term, float
                                int64_t *nnz_out);
 
 /*
- * sivf_get_inverted_file — the structured inverted file (Algorithm 5 output;
+ * sivf_get_inverted_file — the structured inverted file that the last update (or
+ * sivf_init / sivf_reseed) built, with its lambda (Algorithm 5 output;
  * with icp = 2 the unstructured file of Algorithm 3, one part per list):
  *   off : HOST int64[D+1], mf0 : HOST int32[D] (front length),
  *   cid : HOST int32[cap], u : HOST float[cap] (FP32 values), nnz_out.

@@ -49,7 +49,7 @@ cudaError_t dmalloc(sivf_ctx *c, T **p, size_t n) {
 void free_all(sivf_ctx *c) {
     void *ptrs[] = {c->labels, c->labels_prev, c->own, c->sumv, c->lam, c->lam_prev, c->moving, c->mov_list,
                     c->n_mov_dev, c->snorm, c->snorm_new, c->coff[0], c->coff[1], c->cterm[0], c->cterm[1],
-                    c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->tdesc, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
+                    c->cval[0], c->cval[1], c->cclu, c->if_off, c->if_mf0, c->lam_file, c->tdesc, c->sc_id16, c->sc_id32, c->sc_val, c->sc_pack, c->sc_lp,
                     c->ctr, c->obj_dev, c->ws.base, c->inst_obj, c->inst_k, c->mov_beg, c->clu_koff,
                     c->inst_changed, c->own_row_ptr, c->own_idx, c->own_val, c->clu_doff,
                     c->loop_dev, c->done_dev, c->objf_dev, c->grho, c->acc, c->acc_off, c->acc_lab, c->acc_bits, c->acc_bit_off,
@@ -240,6 +240,7 @@ sivf_status create_ctx(sivf_ctx **out, const sivf_config *cfg, int64_t N, int32_
     INIT_CUDA(dmalloc(c, &c->cclu, capc), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_off, (size_t)D + 1), "alloc");
     INIT_CUDA(dmalloc(c, &c->if_mf0, D), "alloc");
+    INIT_CUDA(dmalloc(c, &c->lam_file, k), "alloc");
     // the scan copy fills the front and the back of every list up to a multiple
     // of 4 entries, and carries a small tail pad
     c->cap_s = capc + 3 * std::min<int64_t>(2 * (int64_t)D, capc) + IF_PAD;

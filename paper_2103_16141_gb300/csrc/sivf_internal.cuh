@@ -183,6 +183,7 @@ struct sivf_ctx {
     int64_t *if_off = nullptr;
     int32_t *if_mf0 = nullptr;
     int64_t if_nnz = 0;
+    uint8_t *lam_file = nullptr;  // device [k]: lambda of the last build (lam changes with an assignment or set_labels)
     bool canon_stale = true;  // the canonical file predates the last inverted-file build
     // term table and scan copy (local ids); which arrays exist depends on the
     // id width (16 bits when every instance has k <= 65536) and the precision

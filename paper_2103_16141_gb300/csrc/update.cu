@@ -1119,13 +1119,15 @@ __device__ __forceinline__ void term_bin(int32_t t, int32_t n_inst, const int32_
 // postings; formed per block, then added). The scan position of every cluster
 // is found beside it: within its instance, the moving clusters of lambda^[r]
 // (mov_list, ascending) take positions 0 .. n_mov - 1 and the invariant ones
-// follow in ascending id; id_order (IVF-CBICP) keeps the ids.
+// follow in ascending id; id_order (IVF-CBICP) keeps the ids. lambda is kept as
+// the canonical file's, which may be asked for after it has changed.
 __global__ void __launch_bounds__(TPB) k_if_lists(int32_t D, int32_t k, int32_t n_inst, const int32_t *inst_d,
                                                   const int32_t *inst_k, const uint32_t *cnt2, int64_t min_len,
                                                   int dense, int64_t *len, int32_t *mf0, uint32_t *cursor,
                                                   unsigned long long *hist, const uint8_t *lam,
                                                   const int32_t *mov_list, const int32_t *mov_beg, int id_order,
-                                                  int32_t *clu_pos, int32_t *pos_clu, DevCounters *ctr) {
+                                                  int32_t *clu_pos, int32_t *pos_clu, uint8_t *lam_file,
+                                                  DevCounters *ctr) {
     __shared__ unsigned long long sh[DENSE_BINS + 1];
     for (int b = threadIdx.x; b <= DENSE_BINS; b += TPB) sh[b] = 0ull;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctr->dense_terms = 0;
@@ -1165,6 +1167,7 @@ __global__ void __launch_bounds__(TPB) k_if_lists(int32_t D, int32_t k, int32_t 
         }
         clu_pos[j] = p;
         pos_clu[koff + p] = jl;
+        lam_file[j] = lam[j];
     }
     __syncthreads();
     for (int b = threadIdx.x; b <= DENSE_BINS; b += TPB)
@@ -1513,7 +1516,7 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     // (mov_list and mov_beg belong to the current lambda^[r])
     k_if_lists<<<(unsigned)std::min<int64_t>(blocks_for(std::max(D, c->k)), 1024), TPB, 0, s>>>(
         D, c->k, c->n_inst, c->inst_d, c->inst_k, cnt2, min_len, dense ? 1 : 0, len, c->if_mf0, cursor, hist, c->lam,
-        c->mov_list, c->mov_beg, cb ? 1 : 0, c->clu_pos, c->pos_clu, c->ctr);
+        c->mov_list, c->mov_beg, cb ? 1 : 0, c->clu_pos, c->pos_clu, c->lam_file, c->ctr);
     k_if_tiles<<<tile_blocks, TPB, 0, s>>>(D, c->n_inst, c->inst_d, c->inst_k, len, c->if_mf0, min_len, hist,
                                            dense ? bmin : DENSE_BINS + 1, (unsigned long long)c->cap_dense,
                                            c->dense_thr, w8, tiles);
@@ -1546,12 +1549,13 @@ cudaError_t build_inverted_file(sivf_ctx *c) {
     return cudaSuccess;
 }
 
-// The canonical structured inverted file of the current centroids and lambda
-// (Algorithm 5: for every term, the moving centroids first and the invariant
-// ones after, ascending ids in each part), with the offsets and front lengths of
-// the last build, in the centroid buffer that is not current (terms: cluster
-// ids, values), which nothing reads until the next update writes it: a stable radix sort of the centroid
-// entries by (term, part). Used by the getters only; synchronises the stream.
+// The canonical structured inverted file of the current centroids and the lambda
+// of the last build (Algorithm 5: for every term, the moving centroids first and
+// the invariant ones after, ascending ids in each part), with the offsets and
+// front lengths of that build: a stable radix sort of the centroid entries by
+// (term, part). It lies in the centroid buffer that is not current (terms:
+// cluster ids, values), which nothing reads until the next update writes it.
+// Used by the getters only; synchronises the stream.
 cudaError_t build_canonical_if(sivf_ctx *c) {
     if (!c->canon_stale) return cudaSuccess;
     const int64_t cap = c->cap_c;
@@ -1565,8 +1569,8 @@ cudaError_t build_canonical_if(sivf_ctx *c) {
     if (!cnt2 || !k0 || !v0 || !k1 || !v1) return cudaErrorMemoryAllocation;
     cudaStream_t s = c->stream;
     SIVF_CUDA_TRY(cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * 2 * c->D, s));
-    k_if_keys<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, c->cterm[cur], c->cclu, c->lam, c->cfg.icp == 2 ? 0 : 1, k0,
-                                              v0, cnt2);
+    k_if_keys<<<blocks_gs(cap), TPB, 0, s>>>(n_dev, cap, c->cterm[cur], c->cclu, c->lam_file, c->cfg.icp == 2 ? 0 : 1,
+                                              k0, v0, cnt2);
     note_launch();
     bool alt = false;
     SIVF_CUDA_TRY(radix_sort_pairs_dev(k0, v0, k1, v1, cap, n_dev, c->bits_t + 1, &alt, ws, s));

@@ -1589,7 +1589,10 @@ namespace {
 // coff of the new buffer from the row sizes
 cudaError_t row_offsets(sivf_ctx *c, const int64_t *sz, int nw) {
     cudaStream_t s = c->stream;
-    if (c->k <= 1 << 18) {  // one CTA, 4096 rows a turn
+    // one CTA, 4096 rows a turn, or a scan of two launches: ms per update, one /
+    // two, at k = 4096 0.307 / 0.311, 16,384 0.509 / 0.505, 65,536 1.21 / 1.17,
+    // 262,144 3.95 / 3.76
+    if (c->k <= 8192) {
         k_row_offsets<<<1, 1024, 0, s>>>(c->k, sz, c->coff[nw]);
         note_launch();
         return cudaGetLastError();

@@ -75,7 +75,7 @@ struct AssignParams {
     // per term: {first quad in the scan copy, front length, list length, first
     // entry / 8 of its dense row or -1}
     const int4 *tdesc;
-    // scan copy of the inverted file (ids are scan positions)
+    // scan copy of the inverted file (ids are score slots; IVF-CBICP: cluster ids)
     const uint16_t *sc_id16;
     const int32_t *sc_id32;
     const float *sc_val;
@@ -365,18 +365,13 @@ constexpr int assign_min_blocks() {
     return b < 1 ? 1 : (b > 32 ? 32 : b);
 }
 
-// Score-vector reads and resets. A global score vector is updated by L2
+// Score-vector reads. A global score vector is updated by L2
 // atomics, so its plain reads and stores must not go through L1 (which is not
 // coherent with them): they use the L2-only (.cg) forms.
 template <bool GRHO>
 __device__ __forceinline__ uint32_t rho_ld(const uint32_t *p) {
     if constexpr (GRHO) return __ldcg(p);
     else return *p;
-}
-template <bool GRHO>
-__device__ __forceinline__ void rho_zero(uint32_t *p) {
-    if constexpr (GRHO) __stcg(p, 0u);
-    else *p = 0u;
 }
 
 // Dense head rows: 8 entries of a row per thread, loaded raw and decoded to

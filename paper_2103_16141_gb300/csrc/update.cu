@@ -33,6 +33,7 @@
 
 #include <algorithm>
 
+#include "bf16_rows.cuh"
 #include "sivf_internal.cuh"
 
 namespace sivf {
@@ -626,11 +627,13 @@ __global__ void k_acc_clear(int32_t k, const int64_t *acc_off, const int64_t *bi
 // Whether row j's accumulator entries are read through the occupancy map: the
 // row passes below read 16 bytes per lane in sequence otherwise, which is
 // cheaper once a word of the map (32 entries, eight sectors) has a few bits.
-// Measured per update, whole rows / through the map: k = 20,000 over 140,000
-// terms (0.6 % of the entries non-zero) 6.8 / 2.4 ms, k = 10,000 (1 %) 3.8 /
-// 1.8, k = 3001 over 61,000 (2 %) 0.52 / 0.41, k = 1000 over 100,000 (17 %)
-// 1.72 / 2.0 (before the passes kept 8 CTAs on an SM). The line is at 1/16, by
-// the length of the previous row, or by a third of the members' entries
+// Measured per update, whole rows without a map / whole rows beside one / through
+// it, ms, at a density of non-zero entries of 0.3 % 3.9 / 2.5 / 0.83, 0.6 % 1.50
+// / 1.58 / 0.65, 2.4 % 0.77 / 0.87 / 0.55, 4.2 % 0.59 / 0.66 / 0.47, 6.7 % 0.43 /
+// 0.46 / 0.39, 9.5 % 0.72 / 0.83 / 0.71, 11 % 0.34 / 0.37 / 0.34, 18 % 1.26 / 1.47
+// / 1.44 (k = 10,000 to 400 over 61,000 to 140,000 terms, a tenth of the labels
+// changed). The line is at 1/16, on the near side of where the two are equal,
+// by the length of the previous row, or by a third of the members' entries
 // (avg_len each) where the row has grown.
 __device__ __forceinline__ bool through_map(const uint32_t *bits, int64_t old_len, int64_t members, int64_t avg_len,
                                             int64_t L) {
@@ -1386,9 +1389,9 @@ __global__ void k_if_count(const int64_t *n_dev, int64_t cap, const int32_t *cte
 // centroid entries (one pass, no sort): an entry of a term with a dense row
 // goes to the row at its cluster's scan position; any other entry takes the
 // next free slot of its term's front (moving cluster) or back (invariant
-// cluster) in the scan copy, with the cluster's scan position as its id. The order of the postings inside a
-// segment follows the atomic cursor; no score depends on it (each posting is
-// one integer add).
+// cluster) in the scan copy, with the score slot of the cluster's scan position
+// as its id. The order of the postings inside a segment follows the atomic
+// cursor; no score depends on it (each posting is one integer add).
 __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
                             const float *cval, const uint8_t *lam, int structured, const int32_t *clu_pos,
                             const int4 *tdesc, uint32_t *cursor, int prec, void *dense, uint16_t *sc_id16,
@@ -1421,10 +1424,8 @@ __global__ void k_scan_fill(const int64_t *n_dev, int64_t cap, const int32_t *ct
     }
 }
 
-// Odd entries of the BF16 dense rows. The scan reads a word (even entry below,
-// odd entry above) as FP32 for the odd one, so the upper half is chosen such
-// that the word is the nearest to u among those with its lower half: within
-// half of the upper half's step, as rounding u to BF16 is (2^-8 relative).
+// Odd entries of the BF16 dense rows, once the even ones are there: the scan
+// reads a word (even entry below, odd entry above) as FP32 for the odd one.
 __global__ void k_dense_odd(const int64_t *n_dev, int64_t cap, const int32_t *cterm, const int32_t *cclu,
                             const float *cval, const int32_t *clu_pos, const int4 *tdesc, uint16_t *dense) {
     const int64_t n = live_entries(n_dev, cap);
@@ -1434,8 +1435,7 @@ __global__ void k_dense_odd(const int64_t *n_dev, int64_t cap, const int32_t *ct
         const int32_t row = tdesc[cterm[e]].w;
         if (row < 0) continue;
         uint16_t *at = dense + (int64_t)row * 8 + p;
-        const uint32_t u = max(__float_as_uint(cval[e]), 0x00800000u);  // at least the smallest normal
-        *at = (uint16_t)((u - at[-1] + 0x8000u) >> 16);
+        *at = odd_upper_half(__float_as_uint(cval[e]), at[-1]);
     }
 }
 

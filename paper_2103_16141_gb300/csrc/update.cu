@@ -744,8 +744,11 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     double *jA, double *jU) {
     __shared__ long long shl[WR_THREADS];
     __shared__ unsigned long long sh128[2][WR_THREADS];
+    __shared__ int s_any;  // a previous value lies below 2^-40 (a register for it costs spills, 1 % of the update)
     const int j = blockIdx.x;
     if (j >= k) return;
+    if (threadIdx.x == 0) s_any = 0;
+    __syncthreads();
     const int64_t cb = coff_old[j], ce = coff_old[j + 1];
     if (lam[j] != 0 || cnt[j] == 0) {  // invariant or empty
         if (threadIdx.x == 0) {
@@ -762,7 +765,6 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     // WR_THREADS-th) whose terms lie below a bound, from where it stopped last
     const int32_t doff = clu_doff[j];
     unsigned long long dot_hi = 0ull, dot_lo = 0ull;
-    float least = 1.f;  // of the previous values
     const uint32_t old = (uint32_t)(ce - cb);  // a row has at most 2^31 entries
     uint32_t at = threadIdx.x;
     auto dot_upto = [&](uint32_t bound) {
@@ -782,7 +784,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
 #pragma unroll
             for (int q = 0; q < DOT_ILP; ++q) {
                 add_product(dot_hi, dot_lo, (unsigned long long)v[q], fixed63(u[q]));
-                least = fminf(least, u[q]);
+                if (u[q] < 0x1p-40f) s_any = 1;
                 at += t[q] < bound ? WR_THREADS : 0;
             }
         }
@@ -872,7 +874,7 @@ __global__ void __launch_bounds__(WR_THREADS, 8) k_acc_rows1(
     dot_upto((uint32_t)L);
     block_sum_u128(dot_hi, dot_lo, sh128);
     double dot = ((double)dot_hi * 18446744073709551616.0 + (double)dot_lo) * inv_scale * 0x1p-63;
-    if (__syncthreads_or(least < 0x1p-40f)) {
+    if (s_any) {  // the same for the whole block, behind the sums' barriers
         double small = 0.0;
         for (uint32_t q = threadIdx.x; q < old; q += WR_THREADS) {
             const float u = cval_old[cb + q];

@@ -12,11 +12,11 @@
 //    clusters) is read with 16-byte loads; for every chunk of staged terms the
 //    dense terms' products are chained in FP32 fused multiply-adds per score
 //    position, and the chain's ceil is added once.
-// What bounds the CTA kernel: the row stream into an SM (64 bytes per clock,
-// about 20 TB/s in all). k = 1000 FP32 reads 18.9 TB/s of rows over a whole
-// assignment, k = 3001 FP16 15.1, k = 20,000 BF16 13.7, where two CTAs per SM
-// leave part of the per-object latency uncovered and the L1 data pipe (76 %)
-// and the issue slots (64 %) are busy too.
+// What bounds the CTA kernel: the row stream from L2 into the SMs (22.4 TB/s
+// for plain reads of an L2-resident buffer). k = 1000 FP32 reads 19 TB/s of rows
+// over a whole assignment, k = 3001 FP16 13.4, k = 10,000 BF16 15.4, k = 20,000
+// BF16 13.3, where two CTAs per SM leave part of the per-object latency
+// uncovered and the L1 data pipe (78 %) and the issue slots (64 %) are busy too.
 // Integer addition is associative, so the sums do not depend on the order in
 // which threads visit postings: the filtered and unfiltered modes produce
 // identical scores, and every run is deterministic.

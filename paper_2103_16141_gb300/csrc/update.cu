@@ -730,7 +730,7 @@ constexpr int DOT_ILP = 4;
 // integer sums added exactly in 128 bits, one rounding to FP64) and
 // <s_j, mu_j^[r-1]> over the previous row, whose values are taken in units of
 // 2^-63 and multiplied and added exactly in 128 bits as well: conversions and
-// products in FP64 took longer than the reads (the pass 330 us, now 273 at 1000
+// products in FP64 took longer than the reads (the pass 330 us against 273 at 1000
 // rows of 100,000 entries, 17 % non-zero). By Cauchy-Schwarz that sum stays
 // below 2^63 times 2^63. Values below 2^-40, which that unit would cut short,
 // are multiplied and added in FP64, in a loop of their own. The row's words (row_words) are left with exactly its
